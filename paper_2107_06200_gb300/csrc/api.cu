@@ -376,8 +376,10 @@ static bool lu_timers_enabled() {
 
 // CTAs of the panel's cluster: enough to hold the panel in shared memory,
 // and otherwise one per kPanelRows rows, up to 16 for panels of more than
-// 4096 rows and up to 8 below (a smaller cluster finds free SMs sooner
-// beside the persistent refinement kernels of concurrent solves).
+// 2048 rows and up to 8 below (a smaller cluster finds free SMs sooner
+// beside the persistent refinement kernels of concurrent solves; one CTA of
+// up to 512 rows has no exchange at all, but 16 CTAs of 256 rows still beat
+// 8 of 512: whole n = 4133 fp16 LU 8.2 against 9.1 ms).
 // MSIR_PANEL_CTAS and MSIR_PANEL_ROWS override the cap and the row count
 // (tuning only).
 static int env_int(const char* name, int dflt, int lo, int hi) {
@@ -389,7 +391,7 @@ static int env_int(const char* name, int dflt, int lo, int hi) {
 static int panel_ctas(int m, int Rmax) {
   static const int kPanelCtas = env_int("MSIR_PANEL_CTAS", 0, 1, 16);
   static const int kPanelRows = env_int("MSIR_PANEL_ROWS", 192, 32, 4096);
-  const int cap = kPanelCtas > 0 ? kPanelCtas : (m > 4096 ? 16 : 8);
+  const int cap = kPanelCtas > 0 ? kPanelCtas : (m > 2048 ? 16 : 8);
   int C = (m + Rmax - 1) / Rmax;
   if (C > 16) return -1;
   C = std::max(C, std::min(cap, (m + kPanelRows - 1) / kPanelRows));
@@ -455,7 +457,7 @@ static msir_status enqueue_lu(msir_ctx* ctx, Workspace& w, int n, int u0, int l,
   }
   const int ts = fmt == MSIR_FP64 ? 8 : 4;
   const size_t fixed = panel_smem_bytes(fmt, 0, nb, nbo);
-  const size_t budget = std::min<size_t>((size_t)ctx->max_dyn_smem, 220 * 1024);
+  const size_t budget = (size_t)ctx->max_dyn_smem - 1024;  // the panel's static shared memory
   const int Rmax = (int)((budget - fixed) / ((size_t)(nb + 1) * ts));
   const bool lookahead = ls.aux != nullptr && !lu_no_lookahead();
 
@@ -474,6 +476,7 @@ static msir_status enqueue_lu(msir_ctx* ctx, Workspace& w, int n, int u0, int l,
     pa.ipiv = L.ipiv;
     pa.info = w.iflags + 0;
     pa.nonfinite = w.iflags + 1;
+    pa.err = w.iflags + 2;
     pa.map_pos = map;
     pa.map_val = map + 2 * nbo;
     pa.map_cnt = map + 4 * nbo;
@@ -818,7 +821,7 @@ static void print_wait_site(Slot& s) {
   if (v != 1) return;
   int d[5] = {0, 0, 0, 0, 0};
   cudaMemcpy(d, s.w.iflags + 24, sizeof(d), cudaMemcpyDeviceToHost);  // err (iflags + 2) + 22
-  static const char* names[] = {"?", "grid barrier", "substitution hand-off", "?", "tensor-core mbarrier"};
+  static const char* names[] = {"?", "grid barrier", "substitution hand-off", "panel pivot exchange", "tensor-core mbarrier"};
   fprintf(stderr, "[msir wait] n=%d G=%d site=%s block=%d values=%d %d %d (0x%x; 0x%x)\n", s.job ? s.job->n : 0, s.G,
           names[(d[0] >= 0 && d[0] <= 4) ? d[0] : 0], d[1], d[2], d[3], d[4], (unsigned)d[2], (unsigned)d[4]);
 }
@@ -865,8 +868,8 @@ static void print_lu_timers(Slot& s) {
   unsigned long long t[8];
   cudaStreamSynchronize(s.st);
   cudaMemcpy(t, s.w.iflags + 8, sizeof(t), cudaMemcpyDeviceToHost);
-  fprintf(stderr, "[msir lu timers ms] colloop %.3f clsync %.3f pivot+push %.3f update %.3f store+maps %.3f inner_swap_trsm %.3f inner_update %.3f load %.3f\n",
-          t[0] * 1e-6, t[1] * 1e-6, t[2] * 1e-6, t[3] * 1e-6, t[4] * 1e-6, t[5] * 1e-6, t[6] * 1e-6, t[7] * 1e-6);
+  fprintf(stderr, "[msir lu timers ms] colloop %.3f store+maps %.3f inner_swap_trsm %.3f inner_update %.3f load %.3f\n",
+          t[0] * 1e-6, t[4] * 1e-6, t[5] * 1e-6, t[6] * 1e-6, t[7] * 1e-6);
 }
 
 static msir_status slot_enqueue_factor(msir_ctx* ctx, Slot& s, int fmt, bool squeeze) {

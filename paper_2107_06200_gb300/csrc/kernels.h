@@ -6,7 +6,8 @@
 
 namespace msir {
 
-constexpr int kPanelThreads = 512;
+// bytes of one pivot candidate of the panel's cluster exchange
+constexpr int kPanelCandBytes = 144;
 
 // lu_outer_panel: factor the (n-k) x W outer block at column k in panels of nb.
 struct PanelArgs {
@@ -19,6 +20,7 @@ struct PanelArgs {
   int* map_pos;   // outer composite permutation (positions relative to k), 2W
   int* map_val;
   int* map_cnt;
+  int* err;       // error flag of bounded waits
   unsigned long long* tdbg;  // optional section timers of rank 0 / thread 0 (ns), 8
 };
 
