@@ -33,6 +33,18 @@ namespace msir {
 
 // ------------------------------------------------- outer swaps and TRSM
 
+// Leading dimension of L in shared memory: rows fall in different banks when
+// a warp reads a column, and rows of 16-bit values start on a 32-bit word.
+__host__ __device__ inline int trsm_ldl(int W, int fsize) { return fsize == 2 ? (W + 1) / 2 * 2 + 2 : W + 1; }
+
+// The substitution U12 = L11^{-1} A12 is a chain of W steps per column.  It
+// runs in blocks of 32 rows: within a block a warp takes four columns with
+// one row per lane (the solved value of a step reaches the other rows by a
+// shuffle, four independent chains hide its latency), then every row below
+// subtracts the block's 32 products in ascending order.  Each element sees
+// the same rounded products and differences in the same order as in a
+// row-by-row substitution, with two block barriers per 32 rows instead of
+// one per row.
 template <typename F>
 __global__ void __launch_bounds__(256) lu_outer_swap_trsm(SwapTrsmArgs a) {
   using T = typename Fmt<F>::T;
@@ -42,27 +54,56 @@ __global__ void __launch_bounds__(256) lu_outer_swap_trsm(SwapTrsmArgs a) {
   const int nleft = a.do_left ? k : 0, nright = a.c_end - a.c_begin;
   const int tiles_left = (nleft + 31) / 32;
   const int tiles_right = nright > 0 ? (nright + 31) / 32 : 0;
-  const int tid = threadIdx.x;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  constexpr int NW = 256 / 32;
+  constexpr int ldx = 33;
 
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int ldL = W + (sizeof(F) == 2 ? 2 : 1);  // padded: rows of L fall in different banks
-  T* X = (T*)smem_raw;                       // W x 32
-  F* L = (F*)(X + (size_t)W * 32);           // W x ldL (only when right tiles exist)
-  F* E = L + (size_t)W * ldL;                // (cnt - W) x 32 displaced rows
-  size_t off = sizeof(T) * (size_t)W * 32 + sizeof(F) * ((size_t)W * ldL + (size_t)W * 32);
+  const int ldL = trsm_ldl(W, (int)sizeof(F));
+  T* X = (T*)smem_raw;                       // W x ldx
+  F* L = (F*)(X + (size_t)W * ldx);          // W x ldL (only when right tiles exist)
+  size_t off = sizeof(T) * (size_t)W * ldx + sizeof(F) * (size_t)W * ldL;
   off = (off + 15) & ~(size_t)15;
-  int* pos = (int*)(smem_raw + off);
-  int* val = pos + 2 * W;
+  F* E = (F*)(smem_raw + off);               // (cnt - W) x 32 displaced rows
+  int* val = (int*)(E + (size_t)W * 32);     // sources of the slots [2W]
+  int* pos = val + 2 * W;                    // positions of the slots W .. cnt-1 (slot s < W is row s)
   __shared__ int s_nf;
   if (tid == 0) s_nf = 0;
-  for (int s = tid; s < cnt; s += blockDim.x) { pos[s] = a.map_pos[s]; val[s] = a.map_val[s]; }
+  for (int s = tid; s < cnt; s += blockDim.x) {
+    val[s] = a.map_val[s];
+    if (s >= W) pos[s - W] = a.map_pos[s];
+  }
   bool need_L = false;
   for (int t = blockIdx.x; t < tiles_left + tiles_right; t += gridDim.x)
     if (t >= tiles_left) need_L = true;
+  constexpr int E16 = 16 / (int)sizeof(F);  // values per 16-byte load
+  constexpr int LPR = 32 / E16;             // lanes per 32-column row segment
   if (need_L) {
-    for (int idx = tid; idx < W * W; idx += blockDim.x) {
-      const int i = idx / W, c = idx % W;
-      L[i * ldL + c] = A[(size_t)(k + i) * lda + k + c];
+    if (k % E16 == 0 && W % E16 == 0) {
+      // eight 16-byte loads in flight per thread (rows of L in shared memory
+      // are not 16-byte aligned: stored value by value)
+      const int per = W / E16, tot = W * per;
+      for (int i0 = tid; i0 < tot; i0 += 8 * 256) {
+        uint4 u[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+          const int i = i0 + q * 256;
+          if (i < tot) u[q] = *reinterpret_cast<const uint4*>(A + (size_t)(k + i / per) * lda + k + (i % per) * E16);
+        }
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+          const int i = i0 + q * 256;
+          if (i < tot) {
+            F e[E16];
+            memcpy(e, &u[q], 16);
+#pragma unroll
+            for (int c = 0; c < E16; ++c) L[(i / per) * ldL + (i % per) * E16 + c] = e[c];
+          }
+        }
+      }
+    } else {
+      for (int i = warp; i < W; i += NW)
+        for (int c = lane; c < W; c += 32) L[i * ldL + c] = A[(size_t)(k + i) * lda + k + c];
     }
   }
   __syncthreads();
@@ -71,50 +112,148 @@ __global__ void __launch_bounds__(256) lu_outer_swap_trsm(SwapTrsmArgs a) {
     const bool right = t >= tiles_left;
     const int c0 = right ? a.c_begin + (t - tiles_left) * 32 : t * 32;
     const int cend = right ? a.c_end : k;
-    // gather sources
-    for (int idx = tid; idx < cnt * 32; idx += blockDim.x) {
-      const int s = idx / 32, cc = idx % 32, c = c0 + cc;
-      if (c < cend) {
-        F v = A[(size_t)(k + val[s]) * lda + c];
-        if (s < W) X[s * 32 + cc] = (T)to_f(v);
-        else E[(s - W) * 32 + cc] = v;
+    const int c = c0 + lane;
+    // whole tiles at aligned columns move in 16-byte pieces, LPR lanes per
+    // row and eight rows' loads in flight; ragged ones value by value
+    const bool vec = c0 % E16 == 0 && c0 + 32 <= cend;
+    const int vr = tid / LPR, vc = (tid % LPR) * E16;  // row and first column of a 16-byte piece
+    constexpr int VR = 256 / LPR;                      // rows per pass of the block
+    if (vec) {
+      for (int s0 = vr; s0 < cnt; s0 += 8 * VR) {
+        uint4 u[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+          const int s = s0 + q * VR;
+          if (s < cnt) u[q] = *reinterpret_cast<const uint4*>(A + (size_t)(k + val[s]) * lda + c0 + vc);
+        }
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+          const int s = s0 + q * VR;
+          if (s >= cnt) continue;
+          if (s < W) {
+            F e[E16];
+            memcpy(e, &u[q], 16);
+#pragma unroll
+            for (int v = 0; v < E16; ++v) X[s * ldx + vc + v] = (T)to_f(e[v]);
+          } else {
+            memcpy(E + (s - W) * 32 + vc, &u[q], 16);
+          }
+        }
+      }
+    } else {
+      for (int s = warp; s < cnt; s += NW) {
+        F v{};
+        if (c < cend) v = A[(size_t)(k + val[s]) * lda + c];
+        if (s < W) X[s * ldx + lane] = (T)to_f(v);
+        else E[(s - W) * 32 + lane] = v;
       }
     }
     __syncthreads();
-    for (int idx = tid; idx < (cnt - W) * 32; idx += blockDim.x) {
-      const int s = W + idx / 32, cc = idx % 32, c = c0 + cc;
-      if (c < cend) A[(size_t)(k + pos[s]) * lda + c] = E[(s - W) * 32 + cc];
+    if (vec) {
+      for (int s = W + vr; s < cnt; s += VR) {
+        uint4 u;
+        memcpy(&u, E + (s - W) * 32 + vc, 16);
+        *reinterpret_cast<uint4*>(A + (size_t)(k + pos[s - W]) * lda + c0 + vc) = u;
+      }
+    } else if (c < cend) {
+      for (int s = W + warp; s < cnt; s += NW) A[(size_t)(k + pos[s - W]) * lda + c] = E[(s - W) * 32 + lane];
     }
     if (right) {
-      for (int mm = 0; mm < W - 1; ++mm) {
-        const int rows = W - 1 - mm;
-        for (int idx = tid; idx < rows * 32; idx += blockDim.x) {
-          const int i = mm + 1 + idx / 32, cc = idx % 32;
-          X[i * 32 + cc] = sub_rn(X[i * 32 + cc], mul_rn((T)to_f(L[i * ldL + mm]), X[mm * 32 + cc]));
+      for (int b0 = 0; b0 < W; b0 += 32) {
+        const int bw = min(32, W - b0);
+        // the block's own rows: columns 4 warp .. 4 warp + 3, row b0 + lane
+        {
+          T lr[32], x[4];
+          const int i = min(b0 + lane, W - 1);
+#pragma unroll
+          for (int mm = 0; mm < 32; ++mm) lr[mm] = mm < bw ? (T)to_f(L[i * ldL + b0 + mm]) : (T)0;
+#pragma unroll
+          for (int q = 0; q < 4; ++q) x[q] = X[i * ldx + 4 * warp + q];
+#pragma unroll
+          for (int mm = 0; mm < 31; ++mm) {
+            if (mm + 1 < bw) {
+#pragma unroll
+              for (int q = 0; q < 4; ++q) {
+                const T xm = __shfl_sync(0xffffffffu, x[q], mm);
+                if (lane > mm) x[q] = sub_rn(x[q], mul_rn(lr[mm], xm));
+              }
+            }
+          }
+          if (lane < bw) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) X[i * ldx + 4 * warp + q] = x[q];
+          }
+        }
+        __syncthreads();
+        // the rows below: four rows per warp and pass, one column per lane
+        for (int r0 = b0 + 32 + warp * 4; r0 < W; r0 += 4 * NW) {
+          T x[4];
+          const F* lp[4];
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            const int r = min(r0 + q, W - 1);  // rows past W repeat the last one and are not stored
+            x[q] = X[r * ldx + lane];
+            lp[q] = L + r * ldL + b0;
+          }
+#pragma unroll 8
+          for (int mm = 0; mm < 32; ++mm) {
+            const T xm = X[(b0 + mm) * ldx + lane];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) x[q] = sub_rn(x[q], mul_rn((T)to_f(lp[q][mm]), xm));
+          }
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            if (r0 + q < W) X[(r0 + q) * ldx + lane] = x[q];
         }
         __syncthreads();
       }
     }
     int nf = 0;
-    for (int idx = tid; idx < W * 32; idx += blockDim.x) {
-      const int s = idx / 32, cc = idx % 32, c = c0 + cc;
-      if (c < cend) {
-        F v = store_rn<F>(X[s * 32 + cc]);
+    if (vec) {
+      for (int s = vr; s < W; s += VR) {
+        F e[E16];
+#pragma unroll
+        for (int v = 0; v < E16; ++v) {
+          e[v] = store_rn<F>(X[s * ldx + vc + v]);
+          if (right && !isfinite(to_f(e[v]))) nf = 1;
+        }
+        uint4 u;
+        memcpy(&u, e, 16);
+        *reinterpret_cast<uint4*>(A + (size_t)(k + s) * lda + c0 + vc) = u;
+      }
+    } else if (c < cend) {
+      for (int s = warp; s < W; s += NW) {
+        const F v = store_rn<F>(X[s * ldx + lane]);
         A[(size_t)(k + s) * lda + c] = v;
         if (right && !isfinite(to_f(v))) nf = 1;
       }
     }
     if (right && a.Ut != nullptr) {
       F* Ut = (F*)a.Ut;
-      for (int idx = tid; idx < W * 32; idx += blockDim.x) {
-        const int cc = idx / W, s = idx % W, c = c0 + cc;
-        if (c < cend) Ut[(size_t)(c - k - W) * a.ldut + s] = store_rn<F>(X[s * 32 + cc]);
+      if (W % E16 == 0 && a.ldut % E16 == 0) {
+        // 16 bytes (E16 rows of one column) per thread, neighbouring lanes on
+        // neighbouring columns of X (no bank conflicts)
+        for (int i = tid; i < 32 * (W / E16); i += 256) {
+          const int cc = i % 32, s = (i / 32) * E16;
+          if (c0 + cc >= cend) continue;
+          F e[E16];
+#pragma unroll
+          for (int v = 0; v < E16; ++v) e[v] = store_rn<F>(X[(s + v) * ldx + cc]);
+          uint4 u;
+          memcpy(&u, e, 16);
+          *reinterpret_cast<uint4*>(Ut + (size_t)(c0 + cc - k - W) * a.ldut + s) = u;
+        }
+      } else {
+        for (int cc = warp; cc < 32; cc += NW)
+          if (c0 + cc < cend)
+            for (int s = lane; s < W; s += 32)
+              Ut[(size_t)(c0 + cc - k - W) * a.ldut + s] = store_rn<F>(X[s * ldx + cc]);
       }
     }
     if (nf) s_nf = 1;
     __syncthreads();
   }
-  if (s_nf) atomicExch(a.nonfinite, 1);
+  if (tid == 0 && s_nf) atomicExch(a.nonfinite, 1);
 }
 
 // ------------------------------------------------------- SIMT update
@@ -191,10 +330,9 @@ size_t panel_smem_bytes(int fmt, int R_cap, int nb, int W) {
 size_t swap_trsm_smem_bytes(int fmt, int W) {
   const size_t ts = fmt == MSIR_FP64 ? 8 : 4;
   const size_t fs = fmt == MSIR_FP64 ? 8 : fmt == MSIR_FP32 ? 4 : 2;
-  const size_t ldL = W + (fs == 2 ? 2 : 1);
-  size_t off = ts * (size_t)W * 32 + fs * ((size_t)W * ldL + (size_t)W * 32);
+  size_t off = ts * (size_t)W * 33 + fs * (size_t)W * trsm_ldl(W, (int)fs);
   off = (off + 15) & ~(size_t)15;
-  return off + 4 * (size_t)W * sizeof(int);
+  return off + fs * (size_t)W * 32 + 3 * (size_t)W * sizeof(int);
 }
 
 cudaError_t launch_panel_f16(const PanelArgs& a, int C, cudaStream_t st);
