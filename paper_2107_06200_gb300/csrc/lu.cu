@@ -258,60 +258,135 @@ __global__ void __launch_bounds__(256) lu_outer_swap_trsm(SwapTrsmArgs a) {
 
 // ------------------------------------------------------- SIMT update
 
-template <typename F>
+// A22 <- A22 - L21 U12 for fp32 / fp64 factors: per element one ascending
+// fused multiply-add chain from zero, then one rounded difference.  Tiles of
+// BM x BN elements per block of 256 threads, BM/16 x BN/16 per thread (as
+// two halves BM/2 and BN/2 apart, so that a warp's 16-byte shared-memory
+// reads fall in different banks); the next BK slice is loaded into registers
+// while the current one is used, and shared memory holds two slices, so a
+// slice costs one block barrier.
+template <typename T, int BM, int BN>
 __global__ void __launch_bounds__(256) lu_update_simt(UpdateArgs a) {
-  using T = typename Fmt<F>::T;
-  F* A = (F*)a.A;
+  constexpr int BK = 16;
+  constexpr int E = 16 / (int)sizeof(T);       // values per 16-byte load
+  constexpr int TM = BM / 16, TN = BN / 16;    // elements per thread
+  constexpr int VM = TM < E ? TM : E, VN = TN < E ? TN : E;  // consecutive rows / columns of a thread
+  constexpr int HM = TM / VM, HN = TN / VN;    // groups of them
+  constexpr int LA = BM * BK / 256, LB = BK * BN / 256;  // values loaded per thread and slice
+  static_assert(LA % E == 0 && LB % E == 0, "whole 16-byte loads");
+  T* A = (T*)a.A;
   const int lda = a.lda, k = a.k, W = a.W;
   const int r0 = k + W, M = a.n - r0;
   const int c0 = a.c_begin, NC = a.c_end - a.c_begin;
-  constexpr int BM = 64, BN = 64, BK = 16;
-  __shared__ T As[BK][BM + 1];
-  __shared__ T Bs[BK][BN];
+  __shared__ __align__(16) T As[2][BK][BM + E];
+  __shared__ __align__(16) T Bs[2][BK][BN];
   const int tid = threadIdx.x;
   const int tm = blockIdx.y * BM, tn = blockIdx.x * BN;
   const int ty = tid / 16, tx = tid % 16;
-  T acc[4][4];
+  // 16-byte loads need aligned columns (rows start on 64-element boundaries)
+  const bool vecA = (k % E) == 0, vecB = (c0 % E) == 0;
+  T acc[TM][TN];
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < TM; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = 0;
-  for (int kc = 0; kc < W; kc += BK) {
-    for (int idx = tid; idx < BM * BK; idx += 256) {
-      const int i = idx / BK, kq = idx % BK;
-      const int row = tm + i, kk = kc + kq;
-      As[kq][i] = (row < M && kk < W) ? (T)to_f(A[(size_t)(r0 + row) * lda + k + kk]) : (T)0;
+    for (int j = 0; j < TN; ++j) acc[i][j] = 0;
+  // slice loads: L21 values kq = E (idx % (BK / E)) .. of row idx / (BK / E);
+  // U12 columns E (idx % (BN / E)) .. of row idx / (BN / E)
+  T ra[LA], rb[LB];
+  auto load = [&](int kc) {
+#pragma unroll
+    for (int v = 0; v < LA / E; ++v) {
+      const int idx = tid + v * 256, i = tm + idx / (BK / E), kq = kc + (idx % (BK / E)) * E;
+      const T* p = A + (size_t)(r0 + i) * lda + k + kq;
+      if (i < M && kq + E <= W && vecA) {
+        const uint4 u = *reinterpret_cast<const uint4*>(p);
+        memcpy(&ra[v * E], &u, 16);
+      } else {
+#pragma unroll
+        for (int e = 0; e < E; ++e) ra[v * E + e] = (i < M && kq + e < W) ? p[e] : (T)0;
+      }
     }
-    for (int idx = tid; idx < BK * BN; idx += 256) {
-      const int kq = idx / BN, j = idx % BN;
-      const int col = tn + j, kk = kc + kq;
-      Bs[kq][j] = (col < NC && kk < W) ? (T)to_f(A[(size_t)(k + kk) * lda + c0 + col]) : (T)0;
+#pragma unroll
+    for (int v = 0; v < LB / E; ++v) {
+      const int idx = tid + v * 256, kq = kc + idx / (BN / E), j = tn + (idx % (BN / E)) * E;
+      const T* p = A + (size_t)(k + kq) * lda + c0 + j;
+      if (kq < W && j + E <= NC && vecB) {
+        const uint4 u = *reinterpret_cast<const uint4*>(p);
+        memcpy(&rb[v * E], &u, 16);
+      } else {
+#pragma unroll
+        for (int e = 0; e < E; ++e) rb[v * E + e] = (kq < W && j + e < NC) ? p[e] : (T)0;
+      }
     }
-    __syncthreads();
+  };
+  auto put = [&](int buf) {
 #pragma unroll
-    for (int kq = 0; kq < BK; ++kq) {
-      T av[4], bv[4];
+    for (int v = 0; v < LA / E; ++v) {
+      const int idx = tid + v * 256;
 #pragma unroll
-      for (int i = 0; i < 4; ++i) av[i] = As[kq][ty * 4 + i];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) bv[j] = Bs[kq][tx * 4 + j];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fma_rn(av[i], bv[j], acc[i][j]);
+      for (int e = 0; e < E; ++e) As[buf][(idx % (BK / E)) * E + e][idx / (BK / E)] = ra[v * E + e];
     }
+#pragma unroll
+    for (int v = 0; v < LB / E; ++v) {
+      const int idx = tid + v * 256;
+      uint4 u;
+      memcpy(&u, &rb[v * E], 16);
+      *reinterpret_cast<uint4*>(&Bs[buf][idx / (BN / E)][(idx % (BN / E)) * E]) = u;
+    }
+  };
+  auto step = [&](int buf, int kq) {
+    T av[TM], bv[TN];
+#pragma unroll
+    for (int h = 0; h < HM; ++h)
+#pragma unroll
+      for (int i = 0; i < VM; ++i) av[h * VM + i] = As[buf][kq][h * (BM / HM) + ty * VM + i];
+#pragma unroll
+    for (int h = 0; h < HN; ++h)
+#pragma unroll
+      for (int j = 0; j < VN; ++j) bv[h * VN + j] = Bs[buf][kq][h * (BN / HN) + tx * VN + j];
+#pragma unroll
+    for (int i = 0; i < TM; ++i)
+#pragma unroll
+      for (int j = 0; j < TN; ++j) acc[i][j] = fma_rn(av[i], bv[j], acc[i][j]);
+  };
+  load(0);
+  put(0);
+  __syncthreads();
+  int buf = 0;
+  for (int kc = 0; kc < W; kc += BK, buf ^= 1) {
+    const bool more = kc + BK < W;
+    if (more) load(kc + BK);
+    if (W - kc >= BK) {
+#pragma unroll
+      for (int kq = 0; kq < BK; ++kq) step(buf, kq);
+    } else {
+      for (int kq = 0; kq < W - kc; ++kq) step(buf, kq);
+    }
+    if (more) put(buf ^ 1);  // last read one slice ago, before the previous barrier
     __syncthreads();
   }
+  const bool vecC = vecB && VN == E;
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int row = tm + ty * 4 + i;
+  for (int i = 0; i < TM; ++i) {
+    const int row = tm + (i / VM) * (BM / HM) + ty * VM + i % VM;
     if (row >= M) continue;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int col = tn + tx * 4 + j;
-      if (col >= NC) continue;
-      F* p = A + (size_t)(r0 + row) * lda + c0 + col;
-      *p = store_rn<F>(sub_rn((T)to_f(*p), acc[i][j]));
+    for (int h = 0; h < HN; ++h) {
+      const int col = tn + h * (BN / HN) + tx * VN;
+      T* p = A + (size_t)(r0 + row) * lda + c0 + col;
+      if (vecC && col + VN <= NC) {
+        uint4 u = *reinterpret_cast<const uint4*>(p);
+        T c[E];
+        memcpy(c, &u, 16);
+#pragma unroll
+        for (int j = 0; j < E; ++j) c[j] = sub_rn(c[j], acc[i][h * VN + (j < VN ? j : 0)]);
+        memcpy(&u, c, 16);
+        *reinterpret_cast<uint4*>(p) = u;
+      } else {
+#pragma unroll
+        for (int j = 0; j < VN; ++j)
+          if (col + j < NC) p[j] = sub_rn(p[j], acc[i][h * VN + j]);
+      }
     }
   }
 }
@@ -370,18 +445,22 @@ cudaError_t launch_swap_trsm(int fmt, const SwapTrsmArgs& a, int grid, cudaStrea
   return cudaErrorInvalidValue;
 }
 
+// fp32: 128 x 128 tiles (64 multiply-adds per four 16-byte shared-memory
+// loads) when there are enough of them for the SMs, else 64 x 64; fp64: 64 x
+// 64 (the narrow fp64 pipe bounds it, not the loads).
+template <typename T, int BM, int BN>
+static cudaError_t launch_simt_t(const UpdateArgs& a, int M, int NC, cudaStream_t st) {
+  lu_update_simt<T, BM, BN><<<dim3((NC + BN - 1) / BN, (M + BM - 1) / BM), 256, 0, st>>>(a);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_update_simt(int fmt, const UpdateArgs& a, cudaStream_t st) {
   const int M = a.n - a.k - a.W, NC = a.c_end - a.c_begin;
   if (M <= 0 || NC <= 0) return cudaSuccess;
-  dim3 grid((NC + 63) / 64, (M + 63) / 64);
-  switch (fmt) {
-    case MSIR_FP16: lu_update_simt<__half><<<grid, 256, 0, st>>>(a); break;
-    case MSIR_BF16: lu_update_simt<__nv_bfloat16><<<grid, 256, 0, st>>>(a); break;
-    case MSIR_FP32: lu_update_simt<float><<<grid, 256, 0, st>>>(a); break;
-    case MSIR_FP64: lu_update_simt<double><<<grid, 256, 0, st>>>(a); break;
-    default: return cudaErrorInvalidValue;
-  }
-  return cudaGetLastError();
+  if (fmt == MSIR_FP64) return launch_simt_t<double, 64, 64>(a, M, NC, st);
+  if (fmt != MSIR_FP32) return cudaErrorInvalidValue;
+  if ((long long)((M + 127) / 128) * ((NC + 127) / 128) >= 128) return launch_simt_t<float, 128, 128>(a, M, NC, st);
+  return launch_simt_t<float, 64, 64>(a, M, NC, st);
 }
 
 }  // namespace msir
