@@ -171,10 +171,7 @@ struct Level {  // one factorisation of the current matrix
   double* R = nullptr;
   double* S = nullptr;
   double mu = 1.0;
-  float* inv32 = nullptr;    // inverses of the diagonal blocks (inv.cu)
-  double* inv_hi = nullptr;
-  double* inv_lo = nullptr;
-  int serial = 0;            // identifies this factorisation (scaled blocks follow it)
+  int serial = 0;            // identifies this factorisation (inverses and scaled blocks follow it)
   float t_ms = 0;            // device time of this factorisation
 };
 
@@ -195,9 +192,12 @@ struct Workspace {
   int* perm[3] = {};
   double* R[3] = {};
   double* S[3] = {};
-  float* inv32[3] = {};
-  double* inv_hi[3] = {};
-  double* inv_lo[3] = {};
+  // of the current factorisation, built by the refinement kernel: inverses of
+  // the diagonal blocks
+  float* inv32 = nullptr;
+  float* inv32l = nullptr;
+  double* inv_hi = nullptr;
+  double* inv_lo = nullptr;
   void* Ut = nullptr;
   int* map = nullptr;       // map_pos | map_val | map_cnt
   int* iflags = nullptr;    // info, nonfinite, err
@@ -251,11 +251,12 @@ static size_t ws_layout(Workspace& w, int n, int kcap, int G, bool alloc_f64_lev
     w.perm[l] = (int*)take(n * 4);
     w.R[l] = (double*)take(n * 8);
     w.S[l] = (double*)take(n * 8);
-    const size_t ninv = lvl_bytes[l] ? (size_t)2 * ((n + kBlk - 1) / kBlk) * kBlk * kBlk : 0;
-    w.inv32[l] = ninv ? (float*)take(ninv * 4) : nullptr;
-    w.inv_hi[l] = ninv ? (double*)take(ninv * 8) : nullptr;
-    w.inv_lo[l] = ninv ? (double*)take(ninv * 8) : nullptr;
   }
+  const size_t ninv = (size_t)2 * ((n + kBlk - 1) / kBlk) * kBlk * kBlk;
+  w.inv32 = (float*)take(ninv * 4);
+  w.inv32l = (float*)take(ninv * 4);
+  w.inv_hi = (double*)take(ninv * 8);
+  w.inv_lo = (double*)take(ninv * 8);
   w.Ut = take((size_t)n * 256 * 2);
   w.map = (int*)take(2 * kMapInts * 4);  // two outer blocks' maps (look-ahead)
   w.iflags = (int*)take(32 * 4);
@@ -579,13 +580,8 @@ static msir_status enqueue_lu(msir_ctx* ctx, Workspace& w, int n, int u0, int l,
   }
   CK(ipiv_to_perm(L.ipiv, n, L.perm, st));
   *launches += 1;
-  L.inv32 = w.inv32[l];
-  L.inv_hi = w.inv_hi[l];
-  L.inv_lo = w.inv_lo[l];
   static std::atomic<int> serials{0};
   L.serial = ++serials;
-  CK(launch_inv_diag(fmt, L.F, ldf, n, L.inv32, L.inv_hi, L.inv_lo, st));
-  *launches += 1;
   return MSIR_OK;
 }
 
@@ -769,7 +765,7 @@ static void fill_args(msir_ctx* ctx, Slot& s, RefineArgs& a, int mode) {
   a.d = w.d; a.w = w.w; a.V = w.V; a.ldv = w.ldv; a.vk = w.vk;
   a.H = w.H; a.yv = w.yv; a.red = w.red; a.hred = w.hred; a.hvec = w.hvec;
   a.ll = w.ll; a.bar = w.bar;
-  a.inv32 = L.inv32; a.inv_hi = L.inv_hi; a.inv_lo = L.inv_lo;
+  a.inv32 = w.inv32; a.inv32l = w.inv32l; a.inv_hi = w.inv_hi; a.inv_lo = w.inv_lo;
   a.M32 = w.M32; a.M64 = w.M64; a.Mdh = w.Mdh; a.Mdl = w.Mdl; a.err = w.iflags + 2; a.st = w.st; a.rep = w.rep;
   a.tsv = trsv_timers_enabled() ? w.tsv : nullptr;
   a.i_max = j.p.i_max;
@@ -900,7 +896,7 @@ static msir_status slot_enqueue_factor(msir_ctx* ctx, Slot& s, int fmt, bool squ
 static msir_status slot_enqueue_refine(msir_ctx* ctx, Slot& s) {
   RefineArgs a;
   fill_args(ctx, s, a, MODE_SOLVE);
-  // the scaled blocks in the workspace belong to one factorisation
+  // the inverses and scaled blocks in the workspace belong to one factorisation
   if (s.m_serial != s.lv[s.cur].serial) {
     s.state.mready = 0;
     s.m_serial = s.lv[s.cur].serial;
@@ -940,9 +936,6 @@ static void ws_alias(Workspace& w, const Workspace& o) {
     w.perm[l] = o.perm[l];
     w.R[l] = o.R[l];
     w.S[l] = o.S[l];
-    w.inv32[l] = o.inv32[l];
-    w.inv_hi[l] = o.inv_hi[l];
-    w.inv_lo[l] = o.inv_lo[l];
   }
 }
 
@@ -1640,14 +1633,14 @@ static BatchLayout batch_layout(int nmax, int kcap) {
   L.colmax = off(w.colmax);
   for (int l = 0; l < 3; ++l) {
     L.F[l] = off(w.Fbuf[l]); L.ipiv[l] = off(w.ipiv[l]); L.perm[l] = off(w.perm[l]);
-    L.R[l] = off(w.R[l]); L.S[l] = off(w.S[l]); L.inv32[l] = off(w.inv32[l]);
-    L.inv_hi[l] = off(w.inv_hi[l]); L.inv_lo[l] = off(w.inv_lo[l]);
+    L.R[l] = off(w.R[l]); L.S[l] = off(w.S[l]);
   }
   L.x = off(w.x); L.xn = off(w.xn); L.x0 = off(w.x0); L.xbest = off(w.xbest);
   L.r_hi = off(w.r_hi); L.r_lo = off(w.r_lo); L.c_hi = off(w.c_hi); L.c_lo = off(w.c_lo);
   L.y_hi = off(w.y_hi); L.y_lo = off(w.y_lo); L.z_hi = off(w.z_hi); L.z_lo = off(w.z_lo);
   L.d = off(w.d); L.w = off(w.w); L.vk = off(w.vk);
   L.V = off(w.V); L.H = off(w.H); L.yv = off(w.yv); L.red = off(w.red); L.hred = off(w.hred);
+  L.inv32 = off(w.inv32); L.inv32l = off(w.inv32l); L.inv_hi = off(w.inv_hi); L.inv_lo = off(w.inv_lo);
   L.hvec = off(w.hvec); L.ll = off(w.ll); L.M32 = off(w.M32); L.M64 = off(w.M64); L.Mdh = off(w.Mdh);
   L.Mdl = off(w.Mdl); L.bar = off(w.bar); L.iflags = off(w.iflags);
   L.ldu = w.ldu;

@@ -12,7 +12,7 @@ void* batched_solve_entry_f64();
 size_t batch_smem_bytes(int kcap) {
   const size_t lu = std::max(cta_lu_smem<float>(32), cta_lu_smem<double>(16));
   const size_t refine = refine_smem_bytes(kcap);
-  return std::max(std::max(lu, kInvSmem), refine);
+  return std::max(lu, refine);
 }
 
 int batched_max_grid(int u0, int kcap) {

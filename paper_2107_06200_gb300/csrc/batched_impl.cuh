@@ -2,8 +2,7 @@
 // systems (n <= kBatchMaxN).  Each thread block takes the next system from
 // a work counter and runs all of Algorithm 4 on it alone: ingest
 // (A_u = fl_u0(A), b_u, norms), the LU in u_f (lu_cta.cuh), the factor
-// check with the squeezed retry (Sec. 2.1.2), the inverses of the diagonal
-// blocks, and the refinement (refine_msir with a grid of one block: the
+// check with the squeezed retry (Sec. 2.1.2), and the refinement (refine_msir with a grid of one block: the
 // same SIR / SGMRES-IR / GMRES-IR steps, stopping logic and substitutions
 // as the single-system kernel).  When a stage asks for a finer u_f
 // (Algorithm 4's escalation) the block refactors at the next precision and
@@ -16,14 +15,13 @@
 #include <cuda_bf16.h>
 
 #include "batched.h"
-#include "inv_impl.cuh"
 #include "lu_cta.cuh"
 #include "refine_impl.cuh"
 
 namespace msir {
 
 constexpr int kBatchThreads = kRefThreads;
-static_assert(kBatchThreads == kCtaLuThreads && kBatchThreads == kInvThreads, "one block shape");
+static_assert(kBatchThreads == kCtaLuThreads, "one block shape");
 
 __device__ __forceinline__ int next_uf_d(int f) {
   if (f == MSIR_BF16 || f == MSIR_FP16) return MSIR_FP32;
@@ -48,16 +46,6 @@ __device__ __noinline__ void batch_lu(void* A, int lda, int n, int nb, int nbo, 
                                       int* nonfinite, unsigned char* smem) {
   cta_lu<F>((F*)A, lda, n, nb, nbo, ipiv, info, nonfinite, smem);
 }
-template <typename F>
-__device__ __noinline__ void batch_inv(const void* LU, int ldf, int n, float* inv32, double* inv_hi,
-                                       double* inv_lo, unsigned char* smem) {
-  const int nblk = (n + kIB - 1) / kIB;
-  for (int q = 0; q < 2 * nblk; ++q) {
-    inv_diag_block<F>((const F*)LU, ldf, n, nblk, q % nblk, q < nblk, inv32, inv_hi, inv_lo, (double*)smem);
-    __syncthreads();
-  }
-}
-
 __device__ __forceinline__ void batch_lu_fmt(int fmt, void* A, int lda, int n, int nb, int nbo, int* ipiv,
                                              int* info, int* nonfinite, unsigned char* smem) {
   switch (fmt) {
@@ -67,16 +55,6 @@ __device__ __forceinline__ void batch_lu_fmt(int fmt, void* A, int lda, int n, i
     default: batch_lu<double>(A, lda, n, nb, nbo, ipiv, info, nonfinite, smem); break;
   }
 }
-__device__ __forceinline__ void batch_inv_fmt(int fmt, const void* LU, int ldf, int n, float* inv32,
-                                              double* inv_hi, double* inv_lo, unsigned char* smem) {
-  switch (fmt) {
-    case MSIR_FP16: batch_inv<__half>(LU, ldf, n, inv32, inv_hi, inv_lo, smem); break;
-    case MSIR_BF16: batch_inv<__nv_bfloat16>(LU, ldf, n, inv32, inv_hi, inv_lo, smem); break;
-    case MSIR_FP32: batch_inv<float>(LU, ldf, n, inv32, inv_hi, inv_lo, smem); break;
-    default: batch_inv<double>(LU, ldf, n, inv32, inv_hi, inv_lo, smem); break;
-  }
-}
-
 // A_f = fl_f(A_u), or fl_f(mu R_i a_ij S_j) when squeezed (the same
 // product order as the single-system path)
 template <typename A0>
@@ -148,7 +126,7 @@ __device__ __forceinline__ double batch_mu(const BatchArgs& B, int fmt) {
 template <typename A0>
 __global__ void __launch_bounds__(kBatchThreads, 1) batched_solve_kernel(BatchArgs B) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  unsigned char* gsm = smem_raw + kTrsvSmem + kScaledSmem + kInboxSmem;
+  unsigned char* gsm = smem_raw + kGmresOff;
   __shared__ RefState S;
   __shared__ int s_act, s_reset, s_alg, s_task, s_info, s_nonfinite;
   __shared__ double s_w[kBatchThreads / 32];
@@ -243,6 +221,8 @@ __global__ void __launch_bounds__(kBatchThreads, 1) batched_solve_kernel(BatchAr
     a.H = (double*)(ws + L.H); a.yv = (double*)(ws + L.yv);
     a.red = (double*)(ws + L.red); a.hred = (double*)(ws + L.hred); a.hvec = (double*)(ws + L.hvec);
     a.ll = (unsigned long long*)(ws + L.ll);
+    a.inv32 = (float*)(ws + L.inv32); a.inv32l = (float*)(ws + L.inv32l);
+    a.inv_hi = (double*)(ws + L.inv_hi); a.inv_lo = (double*)(ws + L.inv_lo);
     a.M32 = (float*)(ws + L.M32); a.M64 = (double*)(ws + L.M64);
     a.Mdh = (double*)(ws + L.Mdh); a.Mdl = (double*)(ws + L.Mdl);
     a.bar = (unsigned*)(ws + L.bar);
@@ -259,9 +239,9 @@ __global__ void __launch_bounds__(kBatchThreads, 1) batched_solve_kernel(BatchAr
     a.u0 = u0;
     a.cluster = 1;
     Cx cx;
-    cx.tsm = smem_raw;
-    cx.ssm = smem_raw + kTrsvSmem;
-    cx.inbox = (unsigned long long*)(smem_raw + kTrsvSmem + kScaledSmem);
+    cx.tsm = smem_raw + kScratchOff;
+    cx.ssm = cx.tsm + kTrsvSmem;
+    cx.inbox = (unsigned long long*)smem_raw;
     cx.C = 1;
     cx.G = 1;
     cx.cta = 0;
@@ -319,10 +299,6 @@ __global__ void __launch_bounds__(kBatchThreads, 1) batched_solve_kernel(BatchAr
       lu_info = 0;
       scaled = squeeze ? 1 : 0;
       batch_perm(ipiv, n, perm);
-      float* inv32 = (float*)(ws + L.inv32[l]);
-      double* inv_hi = (double*)(ws + L.inv_hi[l]);
-      double* inv_lo = (double*)(ws + L.inv_lo[l]);
-      batch_inv_fmt(fmt, Fl, ldu, n, inv32, inv_hi, inv_lo, smem_raw);
       t_factor += 1e-6 * (double)(gtimer() - tf0);
       if (tid == 0 && fmt != S.uf) {  // precision raised (Algorithm 4's escalation)
         S.uf = fmt;
@@ -337,11 +313,8 @@ __global__ void __launch_bounds__(kBatchThreads, 1) batched_solve_kernel(BatchAr
       a.Rsc = squeeze ? R : nullptr;
       a.Ssc = squeeze ? Sc : nullptr;
       a.mu = mu;
-      a.inv32 = inv32;
-      a.inv_hi = inv_hi;
-      a.inv_lo = inv_lo;
       cx.epoch = S.epoch;
-      cx.mready = 0;  // the scaled blocks belong to the previous factors
+      cx.mready = 0;  // inverses and scaled blocks belong to the previous factors
       const unsigned long long tr0 = gtimer();
       ok = batch_refine<A0>(cx, a, S, gsm, s_act, s_reset, s_alg);
       ok = __syncthreads_and(ok) != 0;  // one decision for the whole block

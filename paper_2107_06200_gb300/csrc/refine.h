@@ -19,11 +19,20 @@ constexpr int kLLWords = 4;
 // Shared scratch of the substitutions: 8 warps x 64 staged values plus the
 // 64 values of z, for the widest value type (double-double, 16 bytes).
 constexpr int kTrsvSmem = (kRefThreads / 32 + 1) * kBlk * 16;
-// Shared staging of the scaled-block construction: half the inner
-// dimension of one tile at a time (inverse high and low words, 64 x 33
-// doubles each; factor rows, 32 x 65 doubles).
+// Shared staging of the scaled-block construction.  fp64 / dd: half the
+// inner dimension of one tile at a time (inverse high and low words, 64 x 33
+// doubles each; factor rows, 32 x 65 doubles).  fp32: the whole tile
+// (inverse high and low words transposed and factor rows, 64 x 68 floats).
 constexpr int kScLd = kBlk + 1;
-constexpr int kScaledSmem = (2 * kBlk * (kBlk / 2 + 1) + (kBlk / 2) * kScLd) * 8;
+constexpr int kSc32Ld = kBlk + 4;
+constexpr int kScaledSmem64 = (2 * kBlk * (kBlk / 2 + 1) + (kBlk / 2) * kScLd) * 8;
+constexpr int kScaledSmem32 = 3 * kBlk * kSc32Ld * 4;
+constexpr int kScaledSmem = kScaledSmem64 > kScaledSmem32 ? kScaledSmem64 : kScaledSmem32;
+// Shared scratch of one phase at a time: the substitutions (staged values
+// and the tile ring in the staging area), the scaled-block construction, or
+// the inverse of one diagonal block (inv_impl.cuh).
+constexpr int kInvScratch = 8 * (3 * kBlk * (kBlk + 1) + 2 * (kBlk / 2) * (kBlk / 2 + 1) + 2 * kBlk);
+constexpr int kPhaseSmem = kTrsvSmem + kScaledSmem > kInvScratch ? kTrsvSmem + kScaledSmem : kInvScratch;
 // Thread-block clusters of the refinement launch: at most kMaxCluster CTAs.
 // Each CTA keeps an inbox in shared memory where the CTAs of its cluster
 // that solve the blocks just before it (forward) or after it (backward)
@@ -31,6 +40,19 @@ constexpr int kScaledSmem = (2 * kBlk * (kBlk / 2 + 1) + (kBlk / 2) * kScLd) * 8
 // team position in the cluster.
 constexpr int kMaxCluster = 8;
 constexpr int kInboxSmem = kMaxCluster * kBlk * kLLWords * 8;
+
+// Dynamic shared memory of the refinement: the inbox (it keeps its contents
+// between phases), the scratch, the GMRES scalars.
+constexpr int kScratchOff = kInboxSmem;
+constexpr int kGmresOff = kInboxSmem + kPhaseSmem;
+
+// What a workspace holds for the current factors (RefState::mready).
+enum ReadyBits : unsigned {
+  RDY_M32 = 1u,  // inv32 and the fp32 scaled blocks
+  RDY_MDD = 2u,  // double-double scaled blocks
+  RDY_M64 = 4u,  // fp64 scaled blocks
+  RDY_INV = 8u   // inv_hi, inv_lo
+};
 
 enum RefMode { MODE_SOLVE = 0, MODE_APPLY = 1, MODE_RESIDUAL = 2 };
 enum RefPhase {
@@ -49,7 +71,7 @@ struct RefState {
   int cged, status;
   int have_phi0;
   unsigned epoch;     // substitution epoch (one per triangular solve)
-  unsigned mready;    // scaled blocks built for the current factors: bit 0 fp32+fp64, bit 1 dd
+  unsigned mready;    // ReadyBits of the current factors
   int nstages;
   int total_steps, total_gmres;
   double rho_max, delta_prev, phi0, phi;
@@ -98,9 +120,14 @@ struct RefineArgs {
   double* hred;            // CGS partial sums: gridDim.x * (kcap+1)
   double* hvec;            // reduced CGS coefficients (kcap+1)
   unsigned long long* ll;  // substitution hand-off words (see kLLWords)
-  const float* inv32;      // inverses of the diagonal blocks of L and U:
-  const double* inv_hi;    // [2][ceil(n/kBlk)][kBlk][kBlk], fp32 and dd
-  const double* inv_lo;
+  // inverses of the diagonal blocks of L and U, [2][ceil(n/kBlk)][kBlk][kBlk],
+  // zero outside the n - 64 b rows and columns of a ragged last block: a pair
+  // of fp32 (inv32 is its fp32 rounding) and a double-double (inv_hi is its
+  // fp64 rounding); built in the kernel when first needed
+  float* inv32;
+  float* inv32l;
+  double* inv_hi;
+  double* inv_lo;
   // scaled off-diagonal blocks D_b^{-1} F_bj (j != b) of L (j < b) and U
   // (j > b), row-major with leading dimension ldf, built in the kernel when a
   // solve in that precision first needs them (RefState::mready)

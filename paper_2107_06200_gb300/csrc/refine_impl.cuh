@@ -12,7 +12,9 @@
 // only rows its own CTA computed.  Triangular solves are wavefronts: a CTA
 // accumulates the off-diagonal products of its block as soon as the blocks
 // it depends on publish their values (epoch-tagged 64-bit words), then
-// applies the inverse of its diagonal block and publishes.
+// applies the inverse of its diagonal block and publishes.  The inverses
+// and the scaled blocks are built here when a solve in their precision first
+// needs them.
 // Grid barriers are used only where a full vector is needed (matrix-vector
 // products) or a global reduction (norms, Gram-Schmidt coefficients).  The
 // stage controller is replicated in every CTA: all CTAs compute the same
@@ -23,6 +25,7 @@
 #include "common.cuh"
 #include <type_traits>
 
+#include "inv_impl.cuh"
 #include "refine.h"
 
 namespace msir {
@@ -312,7 +315,7 @@ static __device__ double cta_reduce(double v, int op, int tid) {
 // Block substitution with inverted diagonal blocks.  Block b of the forward
 // solve computes z_b = c_b - sum_{j<b} L_bj y_j, then y_b = inv(L_bb) z_b
 // rounded to the storage format; the backward solve runs the same way from
-// the last block up with U.  The inverses come from inv.cu, in the
+// the last block up with U.  The inverses (build_inverses) are in the
 // arithmetic format of the solve.
 //
 // Thread (r, seg) of the CTA owning block b handles row r and the 16
@@ -434,7 +437,7 @@ struct AccF {
   static __device__ __forceinline__ V sub(V a, V b) { return __fsub_rn(a, b); }
   static __device__ __forceinline__ V store(V v, int fmt) { return round_f(v, fmt); }
   static __device__ __forceinline__ V sx(V v, int m) { return __shfl_xor_sync(0xffffffffu, v, m); }
-  static __device__ __forceinline__ I inv(const RefineArgs& a, size_t o) { return __ldg(a.inv32 + o); }
+  static __device__ __forceinline__ I inv(const RefineArgs& a, size_t o) { return __ldcg(a.inv32 + o); }
   // 16 consecutive scaled-block values of one row (zero outside the matrix)
   using Tm = float;
   template <int N>
@@ -468,7 +471,7 @@ struct AccD {
   static __device__ __forceinline__ V sub(V a, V b) { return __dsub_rn(a, b); }
   static __device__ __forceinline__ V store(V v, int) { return v; }
   static __device__ __forceinline__ V sx(V v, int m) { return __shfl_xor_sync(0xffffffffu, v, m); }
-  static __device__ __forceinline__ I inv(const RefineArgs& a, size_t o) { return __ldg(a.inv_hi + o); }
+  static __device__ __forceinline__ I inv(const RefineArgs& a, size_t o) { return __ldcg(a.inv_hi + o); }
   using Tm = double;
   template <int N>
   static __device__ __forceinline__ void tile(const RefineArgs& a, int n, int row, int col, Tm (&v)[N]) {
@@ -541,7 +544,7 @@ struct AccDD {
   static __device__ __forceinline__ V store(V v, int) { return v; }
   static __device__ __forceinline__ V sx(V v, int m) { return dd_shfl_xor(v, m); }
   static __device__ __forceinline__ I inv(const RefineArgs& a, size_t o) {
-    return dd_t{__ldg(a.inv_hi + o), __ldg(a.inv_lo + o)};
+    return dd_t{__ldcg(a.inv_hi + o), __ldcg(a.inv_lo + o)};
   }
   using Tm = dd_t;
   template <int N>
@@ -749,15 +752,137 @@ __device__ __forceinline__ double factor_at<FAny>(const RefineArgs& a, size_t i)
   }
 }
 
+static_assert(kInvScratch == (int)kInvSmem && kInvThreads == kRefThreads, "inverse scratch");
+
+// Inverses of the diagonal blocks of L and U by all CTAs of the grid, once
+// per factorisation: as fp32 pairs (dd = false; inv32, inv32l) or in
+// double-double (inv_hi, inv_lo, and for fp64 factors inv32, inv32l too).  An
+// fp32 pair keeps its 2^-46 as long as the block's diagonal is far from
+// fp32's range ends; other blocks take the double-double arithmetic.
+template <typename F>
+__device__ __noinline__ bool build_inverses(Cx& cx, const RefineArgs& a, bool dd) {
+  float* smf = (float*)cx.tsm;
+  double* smd = (double*)cx.tsm;
+  const bool want32 = !dd || factor_fmt<F>(a) == MSIR_FP64;
+  for (int q = cx.cta; q < 2 * cx.nblk; q += cx.G) {
+    const int b = q % cx.nblk;
+    const bool lower = q < cx.nblk;
+    const size_t f0 = (size_t)b * kBlk * a.ldf + (size_t)b * kBlk;
+    auto get = [&](int i, int k) { return factor_at<F>(a, f0 + (size_t)i * a.ldf + k); };
+    bool pair64 = dd;
+    __syncthreads();  // the scratch is no longer read
+    if (!dd) {
+      inv_load<float>(smf, cx.n, b, lower, get);
+      const float d = cx.tid < kBlk ? fabsf(smf[cx.tid * kXld + cx.tid]) : 1.0f;
+      pair64 = __syncthreads_or(!(d >= 0x1p-60f && d <= 0x1p60f)) != 0;
+    }
+    if (pair64) {
+      inv_load<double>(smd, cx.n, b, lower, get);
+      inv_triangle<ArDD>(lower, smd);
+    } else {
+      inv_triangle<ArFF>(lower, smf);
+    }
+    const size_t base = ((size_t)(lower ? 0 : 1) * cx.nblk + b) * kBlk * kBlk;
+    const int nr = min(kBlk, cx.n - b * kBlk);
+    for (int e = cx.tid; e < kBlk * kBlk; e += kRefThreads) {
+      const int i = e / kBlk, k = e % kBlk, x = kIB * kXld + i * kXld + k;
+      const bool in = i < nr && k < nr;
+      if (pair64) {
+        const double h = in ? smd[x] : 0.0, l = in ? smd[x + kIB * kXld] : 0.0;
+        if (dd) {
+          a.inv_hi[base + e] = h;
+          a.inv_lo[base + e] = l;
+        }
+        if (want32) {
+          const float r = dd_to_f32(h, l);
+          a.inv32[base + e] = r;
+          a.inv32l[base + e] = isfinite(r) ? (float)((h - (double)r) + l) : 0.0f;
+        }
+      } else {
+        a.inv32[base + e] = in ? smf[x] : 0.0f;
+        a.inv32l[base + e] = in ? smf[x + kIB * kXld] : 0.0f;
+      }
+    }
+  }
+  return grid_barrier(a.bar, a.err, cx.G);
+}
+
 // Scaled off-diagonal blocks M_bj = D_b^{-1} F_bj (j != b; L below the
 // diagonal blocks, U above), formed by all CTAs of the grid once per
-// factorisation and precision, the first time a solve needs them.  One
-// 64x64 tile per step: the inverse of the diagonal block and the factor
-// block are staged in shared memory (half the inner dimension at a time);
-// thread (i, g) forms row i, columns
-// 16g .. 16g+15 of the product, 64 terms each.  fp32/fp64: fp64 inverse,
-// fp64 sums, stored as fp64 and rounded to fp32.  dd: dd inverse, sums
-// compensated as in the substitutions (Dot2 with the inverse's low word).
+// factorisation and precision, the first time a solve needs them: one 64x64
+// tile per step.
+//
+// fp32 (bf16 / fp16 / fp32 factors): the inverse as an fp32 pair times the
+// factor's values (exact in fp32), compensated sums, rounded once to fp32;
+// its error before that rounding is about 2^-45 of the sum of magnitudes,
+// and no fp64 instruction is issued (GB300's fp64 pipe runs 2 multiply-adds
+// per clock and SM against 128 in fp32, and about 11 fp32 instructions do a
+// term).  The inverse is staged transposed, so that a thread's 4 x 4 elements
+// take three 16-byte loads per inner step; terms outside the triangle of the
+// inverse are zero and skipped (a warp has 8 rows, warps w and w + 4 of one
+// scheduler have long and short sums).  Measured (n = 8192): 7.2 -> 1.0 ms
+// against fp64 sums.
+template <typename F>
+__device__ __noinline__ bool build_scaled32(Cx& cx, const RefineArgs& a) {
+  float* Xh = (float*)cx.ssm;  // [k][i], kBlk x kSc32Ld
+  float* Xl = Xh + kBlk * kSc32Ld;
+  float* Fb = Xl + kBlk * kSc32Ld;  // [k][c]
+  const int n = cx.n, nb = cx.nblk, ld = a.ldf;
+  const int wr = cx.warp < 4 ? cx.warp : 11 - cx.warp;
+  const int i0 = wr * 8 + (cx.lane >> 4) * 4, c0 = (cx.lane & 15) * 4;
+  for (int t = cx.cta; t < nb * nb; t += cx.G) {
+    const int b = t / nb, j = t % nb;
+    if (b == j) continue;
+    const bool lower = j < b;
+    const size_t ib = ((size_t)(lower ? 0 : 1) * nb + b) * kBlk * kBlk;
+    const int r0 = b * kBlk, q0 = j * kBlk;
+    __syncthreads();  // the previous staging is no longer read
+    for (int e = cx.tid; e < kBlk * kBlk; e += kRefThreads) {
+      const int i = e / kBlk, k = e % kBlk;
+      Xh[k * kSc32Ld + i] = __ldcg(a.inv32 + ib + e);
+      Xl[k * kSc32Ld + i] = __ldcg(a.inv32l + ib + e);
+      Fb[i * kSc32Ld + k] = (r0 + i < n && q0 + k < n) ? (float)factor_at<F>(a, (size_t)(r0 + i) * ld + q0 + k) : 0.0f;
+    }
+    __syncthreads();
+    ff_t acc[4][4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) acc[r][q] = ff_t{0.0f, 0.0f};
+    const int k0 = lower ? 0 : wr * 8, k1 = lower ? wr * 8 + 8 : kBlk;
+    for (int k = k0; k < k1; ++k) {
+      const float4 xh = *(const float4*)(Xh + k * kSc32Ld + i0);
+      const float4 xl = *(const float4*)(Xl + k * kSc32Ld + i0);
+      const float4 f = *(const float4*)(Fb + k * kSc32Ld + c0);
+      const float h4[4] = {xh.x, xh.y, xh.z, xh.w}, l4[4] = {xl.x, xl.y, xl.z, xl.w}, f4[4] = {f.x, f.y, f.z, f.w};
+#pragma unroll
+      for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[r][q] = ArFF::term(f4[q], ArFF::V{h4[r], l4[r]}, acc[r][q]);
+    }
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const int row = r0 + i0 + r, col = q0 + c0;
+      if (row >= n) continue;
+      float* dst = a.M32 + (size_t)row * ld + col;
+      if (col + 4 <= n) {
+        *(float4*)dst = make_float4(ff_fin(acc[r][0]), ff_fin(acc[r][1]), ff_fin(acc[r][2]), ff_fin(acc[r][3]));
+      } else {
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          if (col + q < n) dst[q] = ff_fin(acc[r][q]);
+      }
+    }
+  }
+  return grid_barrier(a.bar, a.err, cx.G);
+}
+
+// fp64 and dd (and fp32 with fp64 factors): the inverse of the diagonal block
+// and the factor block are staged in shared memory (half the inner dimension
+// at a time); thread (i, g) forms row i, columns 16g .. 16g+15 of the
+// product, 64 terms each.  fp64: fp64 inverse, fp64 sums (with fp64 factors
+// rounded to fp32 for M32 too); dd: dd inverse, sums compensated as in the
+// substitutions (Dot2 with the inverse's low word).
 template <typename F>
 __device__ __noinline__ bool build_scaled(Cx& cx, const RefineArgs& a, bool dd) {
   // staging of half the inner dimension at a time: inverse columns k0..k0+31
@@ -766,6 +891,7 @@ __device__ __noinline__ bool build_scaled(Cx& cx, const RefineArgs& a, bool dd) 
   double* Xh = (double*)cx.ssm;       // 64 x (KH + 1)
   double* Xl = Xh + kBlk * (KH + 1);  // 64 x (KH + 1)
   double* Fb = Xl + kBlk * (KH + 1);  // KH x kScLd
+  const bool with32 = factor_fmt<F>(a) == MSIR_FP64;
   const int n = cx.n, nb = cx.nblk, ld = a.ldf;
   const int i = cx.tid >> 2, cg = cx.tid & 3;
   for (int t = cx.cta; t < nb * nb; t += cx.G) {
@@ -782,8 +908,8 @@ __device__ __noinline__ bool build_scaled(Cx& cx, const RefineArgs& a, bool dd) 
       __syncthreads();  // the previous staging is no longer read
       for (int e = cx.tid; e < kBlk * KH; e += kRefThreads) {
         const int rr = e / KH, kk = e % KH;
-        Xh[rr * (KH + 1) + kk] = __ldg(a.inv_hi + ib + (size_t)rr * kBlk + k0 + kk);
-        if (dd) Xl[rr * (KH + 1) + kk] = __ldg(a.inv_lo + ib + (size_t)rr * kBlk + k0 + kk);
+        Xh[rr * (KH + 1) + kk] = __ldcg(a.inv_hi + ib + (size_t)rr * kBlk + k0 + kk);
+        if (dd) Xl[rr * (KH + 1) + kk] = __ldcg(a.inv_lo + ib + (size_t)rr * kBlk + k0 + kk);
       }
       for (int e = cx.tid; e < KH * kBlk; e += kRefThreads) {
         const int kk = e / kBlk, cc = e % kBlk;
@@ -819,7 +945,7 @@ __device__ __noinline__ bool build_scaled(Cx& cx, const RefineArgs& a, bool dd) 
         if (col >= n) continue;
         if (!dd) {
           a.M64[(size_t)row * ld + col] = sh[q];
-          a.M32[(size_t)row * ld + col] = __double2float_rn(sh[q]);
+          if (with32) a.M32[(size_t)row * ld + col] = __double2float_rn(sh[q]);
         } else {
           const dd_t v = two_sum(sh[q], sc[q]);
           a.Mdh[(size_t)row * ld + col] = v.hi;
@@ -1133,10 +1259,17 @@ __device__ __forceinline__ bool trsv(Cx& cx, const RefineArgs& a, int store_fmt)
 // substitution.  Result in z (natural order, before the S*mu scaling).
 template <typename F, typename ACC>
 __device__ bool msolve(Cx& cx, const RefineArgs& a, int store_fmt) {
-  // scaled blocks of the current factors in this precision, once
-  const unsigned need = ACC::kW == 4 ? 2u : 1u;
+  // inverses and scaled blocks of the current factors in this precision, once
+  const bool f64 = factor_fmt<F>(a) == MSIR_FP64;
+  const unsigned need = ACC::kW == 4 ? RDY_MDD : (ACC::kW == 2 || f64) ? RDY_M64 : RDY_M32;
   if (!(cx.mready & need)) {
-    if (!build_scaled<F>(cx, a, need == 2u)) return false;
+    if (need == RDY_M32) {
+      if (!build_inverses<F>(cx, a, false) || !build_scaled32<F>(cx, a)) return false;
+    } else {
+      if (!(cx.mready & RDY_INV) && !build_inverses<F>(cx, a, true)) return false;
+      if (!build_scaled<F>(cx, a, need == RDY_MDD)) return false;
+      cx.mready |= RDY_INV;
+    }
     cx.mready |= need;
   }
   // Rows of block b are prepared (c) and consumed (z) by CTA b mod G.  A
@@ -2052,13 +2185,13 @@ template <typename A0, typename F>
 // of one system then slow the other's.)
 __global__ void __launch_bounds__(kRefThreads, 1) refine_kernel(RefineArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  unsigned char* gsm = smem_raw + kTrsvSmem + kScaledSmem + kInboxSmem;  // GMRES scalars
+  unsigned char* gsm = smem_raw + kGmresOff;  // GMRES scalars
   __shared__ RefState S;
   __shared__ int s_act, s_reset, s_alg;
 
   Cx cx;
-  cx.tsm = smem_raw;
-  cx.ssm = smem_raw + kTrsvSmem;
+  cx.tsm = smem_raw + kScratchOff;
+  cx.ssm = cx.tsm + kTrsvSmem;
   cx.G = gridDim.x;
   cx.cta = blockIdx.x;
   cx.tid = threadIdx.x;
@@ -2068,7 +2201,7 @@ __global__ void __launch_bounds__(kRefThreads, 1) refine_kernel(RefineArgs a) {
   cx.nblk = (a.n + kBlk - 1) / kBlk;
   cx.team_k = a.team_k;
   cx.redbuf = 0;
-  cx.inbox = (unsigned long long*)(smem_raw + kTrsvSmem + kScaledSmem);
+  cx.inbox = (unsigned long long*)smem_raw;
   cx.C = 1;
   if (a.cluster > 1) {
     // the inbox starts all ones (a tag no hand-off uses); peers write into

@@ -13,7 +13,7 @@ template <typename A0, typename F> void* refine_entry();
 // ---------------------------------------------------------- launchers
 
 size_t refine_smem_bytes(int kcap) {
-  return kTrsvSmem + kScaledSmem + kInboxSmem +
+  return kGmresOff +
          sizeof(double) * (3 * ((size_t)kcap + 2) + 2 * ((size_t)kcap + 1));
 }
 
