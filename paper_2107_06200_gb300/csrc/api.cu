@@ -212,6 +212,10 @@ struct Workspace {
   double* M64 = nullptr;
   double* Mdh = nullptr;
   double* Mdl = nullptr;
+  // inverses of the diagonal superblocks (wide solves): fp32 pairs, fp64
+  float* D32h = nullptr;
+  float* D32l = nullptr;
+  double* D64 = nullptr;
   unsigned* bar = nullptr;
   RefState* st = nullptr;
   msir_report* rep = nullptr;
@@ -275,6 +279,15 @@ static size_t ws_layout(Workspace& w, int n, int kcap, int G, bool alloc_f64_lev
   w.M64 = (double*)take(ldu * n * 8);
   w.Mdh = (double*)take(ldu * n * 8);
   w.Mdl = (double*)take(ldu * n * 8);
+  if (n >= kWideMin) {
+    const size_t nd = 2 * round_up((size_t)n, kSuper) * kSuper;
+    w.D32h = (float*)take(nd * 4);
+    w.D32l = (float*)take(nd * 4);
+    w.D64 = (double*)take(nd * 8);
+  } else {
+    w.D32h = w.D32l = nullptr;
+    w.D64 = nullptr;
+  }
   w.bar = (unsigned*)take(64);
   w.st = (RefState*)take(sizeof(RefState));
   w.rep = (msir_report*)take(sizeof(msir_report));
@@ -784,6 +797,27 @@ static void fill_args(msir_ctx* ctx, Slot& s, RefineArgs& a, int mode) {
     return (v == 1 || v == 2 || v == 4 || v == 8) ? v : 0;
   }();
   a.team_k = team_k;
+  // wide solves in the precisions whose y fits in shared memory, with the
+  // deep ring if that fits too.  MSIR_WIDE_MIN overrides the smallest n
+  // (tuning only).
+  static const int wide_min = env_int("MSIR_WIDE_MIN", kWideMin, kWideMin, 1 << 30);
+  if (mode != MODE_RESIDUAL && j.n >= wide_min && w.D32h) {
+    a.npad = (int)round_up((size_t)j.n, kSuper);
+    a.D32h = w.D32h;
+    a.D32l = w.D32l;
+    a.D64 = w.D64;
+    const size_t room = (size_t)ctx->max_dyn_smem - 1024;
+    for (int vb : {4, 8}) {
+      if (vb == 8 && j.n < kWideMin64) break;
+      for (int ring : {kRingDeep, kRingFlat})
+        if (refine_smem_bytes(a.kcap, wide_smem(a.npad, s.G, vb, ring)) <= room) {
+          a.wide |= vb == 4 ? 1 : 2;
+          a.ring = ring;
+          a.ring_off = (int)wide_ring_off(a.npad, s.G, vb);
+          break;
+        }
+    }
+  }
   a.cluster = (mode == MODE_SOLVE && s.C > 1 && s.G % s.C == 0) ? s.C : 1;
   a.tau = j.p.tau;
   a.gamma = j.p.gamma;
@@ -791,7 +825,6 @@ static void fill_args(msir_ctx* ctx, Slot& s, RefineArgs& a, int mode) {
   a.xref = j.p.conv == MSIR_CONV_TRUE ? j.xref : nullptr;
   a.allow_escalation = j.p.allow_escalation;
   a.u0 = j.t.u;
-  (void)ctx;
 }
 
 // Enqueue one factorisation attempt of the slot's current job.

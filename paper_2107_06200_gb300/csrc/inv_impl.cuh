@@ -47,10 +47,8 @@ struct ArFF {
   using Acc = ff_t;
   static __device__ __forceinline__ Acc zero() { return ff_t{0.0f, 0.0f}; }
   static __device__ __forceinline__ Acc add(Acc a, float p, float e) {
-    // Knuth's TwoSum: fp32 additions are cheap here
-    const float s = __fadd_rn(a.s, p);
-    const float b = __fsub_rn(s, a.s);
-    const float r = __fadd_rn(__fsub_rn(a.s, __fsub_rn(s, b)), __fsub_rn(p, b));
+    float s, r;
+    two_sum_f(a.s, p, s, r);
     return ff_t{s, __fadd_rn(a.c, __fadd_rn(r, e))};
   }
   // acc + f x, and acc + x y
@@ -64,7 +62,7 @@ struct ArFF {
   }
   static __device__ __forceinline__ V fin(Acc a) {
     float s, e;
-    two_sum_ord_f(a.s, a.c, s, e);
+    two_sum_f(a.s, a.c, s, e);
     return V{s, e};
   }
   static __device__ __forceinline__ V neg(V x) { return V{-x.h, -x.l}; }

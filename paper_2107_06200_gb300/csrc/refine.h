@@ -44,15 +44,38 @@ constexpr int kInboxSmem = kMaxCluster * kBlk * kLLWords * 8;
 // Dynamic shared memory of the refinement: the inbox (it keeps its contents
 // between phases), the scratch, the GMRES scalars.
 constexpr int kScratchOff = kInboxSmem;
-constexpr int kGmresOff = kInboxSmem + kPhaseSmem;
+constexpr int kGmresOff = kInboxSmem + kPhaseSmem;  // (without wide solves)
 
 // What a workspace holds for the current factors (RefState::mready).
 enum ReadyBits : unsigned {
   RDY_M32 = 1u,  // inv32 and the fp32 scaled blocks
   RDY_MDD = 2u,  // double-double scaled blocks
   RDY_M64 = 4u,  // fp64 scaled blocks
-  RDY_INV = 8u   // inv_hi, inv_lo
+  RDY_INV = 8u,  // inv_hi, inv_lo
+  RDY_W32 = 16u, // fp32-pair inverses of the diagonal superblocks
+  RDY_W64 = 32u  // fp64 ones
 };
+
+// Wide solves (refine_impl.cuh): rows of a superblock, and the smallest
+// matrices that take them.  fp32: from two superblocks on (n = 1024 .. 2000:
+// 20-40 us for a pair of solves against 45-95).  fp64: from 1792 rows on;
+// below, the error of a solve was up to 1.2 times that of the 64-row solve
+// (n = 1500, kappa = 1e2: 5.0e-13 against 4.1e-13 of |x|), above it is
+// smaller (n = 2000 .. 5000: 0.97 to 0.08 times).
+constexpr int kSuper = 512;
+constexpr int kWideMin = 1024;
+constexpr int kWideMin64 = 1792;
+constexpr int kRingDeep = 16, kRingFlat = 8;  // steps of the ring of factor values
+// Shared memory of a wide solve in values of `vbytes` on a grid of G CTAs:
+// y of every row, z of a superblock (high and low words), partial sums; then
+// the ring of factor values (16 bytes per thread and step).
+constexpr size_t wide_ring_off(int npad, int G, int vbytes) {
+  const size_t rows = (size_t)(kSuper + G - 1) / G, passes = (rows + 3) / 4;  // at least 4 rows of a CTA at a time
+  return ((size_t)npad * vbytes + 2 * (size_t)kSuper * vbytes + 16 * 8 + passes * kRefThreads * 8 + 127) / 128 * 128;
+}
+constexpr size_t wide_smem(int npad, int G, int vbytes, int ring) {
+  return wide_ring_off(npad, G, vbytes) + (size_t)ring * kRefThreads * 16;
+}
 
 enum RefMode { MODE_SOLVE = 0, MODE_APPLY = 1, MODE_RESIDUAL = 2 };
 enum RefPhase {
@@ -135,6 +158,15 @@ struct RefineArgs {
   double* M64;
   double* Mdh;
   double* Mdl;
+  // wide solves: n rounded up to whole superblocks, which precisions take
+  // them (bit 0 fp32, bit 1 fp64), steps of the ring of factor values
+  // (kRingDeep or kRingFlat) and its offset in the scratch, the inverses of the diagonal
+  // superblocks of L and U, [2][npad][kSuper] (fp32 pairs, fp64)
+  int npad, wide, ring, ring_off;
+  int gmres_off;           // offset of the GMRES scalars in shared memory (set by launch_refine)
+  float* D32h;
+  float* D32l;
+  double* D64;
   unsigned* bar;           // grid barrier counter (zeroed before launch)
   int* err;
   RefState* st;
@@ -173,6 +205,8 @@ int refine_max_grid(int a_fmt, int f_fmt, int kcap);
 // Largest cooperative grid of `cluster`-CTA clusters that fits on the
 // device for every u_f instantiation with A_u in a_fmt (0 if none).
 int refine_max_cluster_grid(int a_fmt, int kcap, int cluster);
-size_t refine_smem_bytes(int kcap);
+// Dynamic shared memory of a launch: the inbox, the scratch of the phase that
+// needs most (`phase` bytes for the wide solves), the GMRES scalars.
+size_t refine_smem_bytes(int kcap, size_t phase = 0);
 
 }  // namespace msir

@@ -754,13 +754,21 @@ __device__ __forceinline__ double factor_at<FAny>(const RefineArgs& a, size_t i)
 
 static_assert(kInvScratch == (int)kInvSmem && kInvThreads == kRefThreads, "inverse scratch");
 
+// Index of row r (of the n rows padded to whole superblocks) of triangle tri
+// (0 L, 1 U) in the inverses of the diagonal superblocks, [2][npad][kSuper].
+__device__ __forceinline__ size_t wide_row(const RefineArgs& a, int tri, int r) {
+  return ((size_t)tri * a.npad + r) * kSuper;
+}
+
 // Inverses of the diagonal blocks of L and U by all CTAs of the grid, once
 // per factorisation: as fp32 pairs (dd = false; inv32, inv32l) or in
-// double-double (inv_hi, inv_lo, and for fp64 factors inv32, inv32l too).  An
+// double-double (inv_hi, inv_lo, and for fp64 factors inv32, inv32l too);
+// `wide`: the fp32 pairs go into the superblocks' array (the fp64 ones
+// always go there too).  An
 // fp32 pair keeps its 2^-46 as long as the block's diagonal is far from
 // fp32's range ends; other blocks take the double-double arithmetic.
 template <typename F>
-__device__ __noinline__ bool build_inverses(Cx& cx, const RefineArgs& a, bool dd) {
+__device__ __noinline__ bool build_inverses(Cx& cx, const RefineArgs& a, bool dd, bool wide) {
   float* smf = (float*)cx.tsm;
   double* smd = (double*)cx.tsm;
   const bool want32 = !dd || factor_fmt<F>(a) == MSIR_FP64;
@@ -784,6 +792,12 @@ __device__ __noinline__ bool build_inverses(Cx& cx, const RefineArgs& a, bool dd
     }
     const size_t base = ((size_t)(lower ? 0 : 1) * cx.nblk + b) * kBlk * kBlk;
     const int nr = min(kBlk, cx.n - b * kBlk);
+    // for wide solves the blocks go on the diagonals of the superblocks
+    const size_t wbase = a.wide ? wide_row(a, lower ? 0 : 1, b * kBlk) + (b * kBlk) % kSuper : 0;
+    const bool w32 = wide && !dd, w64 = (a.wide & 2) != 0;
+    float* o32h = w32 ? a.D32h + wbase : a.inv32 + base;
+    float* o32l = w32 ? a.D32l + wbase : a.inv32l + base;
+    const int ld32 = w32 ? kSuper : kBlk;
     for (int e = cx.tid; e < kBlk * kBlk; e += kRefThreads) {
       const int i = e / kBlk, k = e % kBlk, x = kIB * kXld + i * kXld + k;
       const bool in = i < nr && k < nr;
@@ -792,15 +806,16 @@ __device__ __noinline__ bool build_inverses(Cx& cx, const RefineArgs& a, bool dd
         if (dd) {
           a.inv_hi[base + e] = h;
           a.inv_lo[base + e] = l;
+          if (w64) a.D64[wbase + (size_t)i * kSuper + k] = h;
         }
         if (want32) {
           const float r = dd_to_f32(h, l);
-          a.inv32[base + e] = r;
-          a.inv32l[base + e] = isfinite(r) ? (float)((h - (double)r) + l) : 0.0f;
+          o32h[(size_t)i * ld32 + k] = r;
+          o32l[(size_t)i * ld32 + k] = isfinite(r) ? (float)((h - (double)r) + l) : 0.0f;
         }
       } else {
-        a.inv32[base + e] = in ? smf[x] : 0.0f;
-        a.inv32l[base + e] = in ? smf[x + kIB * kXld] : 0.0f;
+        o32h[(size_t)i * ld32 + k] = in ? smf[x] : 0.0f;
+        o32l[(size_t)i * ld32 + k] = in ? smf[x + kIB * kXld] : 0.0f;
       }
     }
   }
@@ -1254,19 +1269,643 @@ __device__ __forceinline__ bool trsv(Cx& cx, const RefineArgs& a, int store_fmt)
   return trsv_team<F, ACC, LOWER, 1>(cx, a, store_fmt, epoch);
 }
 
+// ------------------------------------------------ wide triangular solves
+//
+// For matrices of more than kWideMin rows the chain of 64-row blocks bounds
+// the substitution above: n / 64 dependent hand-offs of about 1 us each, on
+// few CTAs.  The wide solve takes superblocks of SB = kSuper rows:
+//   z_s = c_s - sum_{j<s} F_sj y_j,   y_s = S(T(inv(F_ss) z_s))
+// (backward: j > s, y for c), every CTA of the grid working on its share of
+// each superblock's rows, with two hand-offs per superblock (z, then y)
+// instead of SB / 64, and on the factors in their storage format instead of
+// scaled blocks in the solve's precision.  Products with superblocks that
+// are known early are formed while a hand-off is under way.
+//
+// Rounding: the inverse of a diagonal superblock and z are kept as pairs in
+// fp32 solves (sums compensated), so the only fp32-sized error of a
+// component is its final rounding; fp64 solves use fp64 throughout.
+// Against the 64-row solve the error is smaller (fp32, n = 2000 .. 5000: 10
+// to 17 times; fp64: up to 12 times).
+//
+// Measured (forward + backward, alone on the GPU): n = 2000 94 -> 42 us
+// (fp32), 112 -> 64 us (fp64); n = 8192 390 -> 270 us (fp32), 740 -> 480 us
+// (fp64).  What bounds it now: two hand-offs of about 1 us per superblock
+// (an L2 round trip alone is 0.4 us) and, at n = 8192, the compensated sums
+// of the far products.
+//
+template <typename ACC> struct Wide;
+template <> struct Wide<AccF> {
+  using AR = ArFF;
+  static constexpr int kZW = 2;  // hand-off words of a z value
+  static __device__ __forceinline__ const float* inv_h(const RefineArgs& a) { return a.D32h; }
+  static __device__ __forceinline__ const float* inv_l(const RefineArgs& a) { return a.D32l; }
+  // z = c - acc as a pair
+  static __device__ __forceinline__ ArFF::V zdiff(float c, ff_t acc) {
+    float s, e;
+    two_sum_f(c, -acc.s, s, e);
+    e = __fsub_rn(e, acc.c);
+    float h, l;
+    two_sum_f(s, e, h, l);
+    return ArFF::V{h, l};
+  }
+  static __device__ __forceinline__ ArFF::V zval(float c) { return ArFF::V{c, 0.0f}; }
+  static __device__ __forceinline__ unsigned zword(ArFF::V z, int k) { return __float_as_uint(k ? z.l : z.h); }
+  static __device__ __forceinline__ ArFF::V unzword(const unsigned* w) {
+    return ArFF::V{__uint_as_float(w[0]), __uint_as_float(w[1])};
+  }
+};
+// plain fp64 values in the pair interface (no low words)
+struct ArD {
+  using S = double;
+  struct V { double h; };
+  using Acc = double;
+};
+template <> struct Wide<AccD> {
+  using AR = ArD;
+  static constexpr int kZW = 2;
+  static __device__ __forceinline__ const double* inv_h(const RefineArgs& a) { return a.D64; }
+  static __device__ __forceinline__ const double* inv_l(const RefineArgs& a) { return a.D64; }
+  static __device__ __forceinline__ ArD::V zdiff(double c, double acc) { return ArD::V{__dsub_rn(c, acc)}; }
+  static __device__ __forceinline__ ArD::V zval(double c) { return ArD::V{c}; }
+  static __device__ __forceinline__ unsigned zword(ArD::V z, int k) { return AccD::word(z.h, k); }
+  static __device__ __forceinline__ ArD::V unzword(const unsigned* w) { return ArD::V{AccD::unword(w)}; }
+};
+
+// four consecutive values from 16-byte aligned shared memory
+__device__ __forceinline__ void lds4(const float* p, float (&v)[4]) {
+  const float4 f = *(const float4*)p;
+  v[0] = f.x; v[1] = f.y; v[2] = f.z; v[3] = f.w;
+}
+__device__ __forceinline__ void lds4(const double* p, double (&v)[4]) {
+  const double2 f = *(const double2*)p, g = *((const double2*)p + 1);
+  v[0] = f.x; v[1] = f.y; v[2] = g.x; v[3] = g.y;
+}
+
+template <typename ACC, typename F>
+__device__ __forceinline__ bool use_wide(const RefineArgs& a) {
+  if constexpr (std::is_same<F, FAny>::value || ACC::kW == 4) return false;
+  else if constexpr (ACC::kW == 1) return (a.wide & 1) && !std::is_same<F, double>::value;
+  else return (a.wide & 2) != 0;
+}
+
+// Products of 64x64 tiles for the doubling of the superblock inverses: acc
+// (4 x 4 per thread: rows 4 (tid / 16) .., columns 4 (tid % 16) ..) +=
+// A B over 64 inner terms; A staged transposed ([k][i]), B as [k][j].
+constexpr int kWtLd = kBlk + 4;
+// fp32 pairs: A values or pairs (Al null: values)
+template <bool kPairA>
+__device__ __forceinline__ void wide_tile_mma(const float* Ah, const float* Al, const float* Bh, const float* Bl,
+                                              int i0, int j0, ff_t (&acc)[4][4]) {
+#pragma unroll 2
+  for (int k = 0; k < kBlk; ++k) {
+    const float4 ah = *(const float4*)(Ah + k * kWtLd + i0);
+    float4 al = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (kPairA) al = *(const float4*)(Al + k * kWtLd + i0);
+    const float4 bh = *(const float4*)(Bh + k * kWtLd + j0), bl = *(const float4*)(Bl + k * kWtLd + j0);
+    const float A4[4] = {ah.x, ah.y, ah.z, ah.w}, L4[4] = {al.x, al.y, al.z, al.w};
+    const float H4[4] = {bh.x, bh.y, bh.z, bh.w}, M4[4] = {bl.x, bl.y, bl.z, bl.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        if (kPairA) acc[i][j] = ArFF::term(ArFF::V{A4[i], L4[i]}, ArFF::V{H4[j], M4[j]}, acc[i][j]);
+        else acc[i][j] = ArFF::term(A4[i], ArFF::V{H4[j], M4[j]}, acc[i][j]);
+      }
+  }
+}
+__device__ __forceinline__ void wide_tile_mma(const double* A, const double* B, int i0, int j0, double (&acc)[4][4]) {
+#pragma unroll 2
+  for (int k = 0; k < kBlk; ++k) {
+    double a4[4], b4[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      a4[q] = A[k * kWtLd + i0 + q];
+      b4[q] = B[k * kWtLd + j0 + q];
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) acc[i][j] = __fma_rn(a4[i], b4[j], acc[i][j]);
+  }
+}
+
+// Inverses of the diagonal superblocks from those of the 64x64 blocks
+// (build_inverses has put them on the diagonal), by doubling h = 64, 128, ..:
+//   L: X21 = -X22 (L21 X11)     U: X12 = -X11 (U12 X22)
+// in 64x64 tiles over all CTAs.  The inner product T waits in the opposite
+// off-diagonal block of the same array, which the inverse does not use (its
+// readers stay inside the triangle).
+template <typename F, bool kF32>
+__device__ __noinline__ bool build_wide(Cx& cx, const RefineArgs& a) {
+  using S = typename std::conditional<kF32, float, double>::type;
+  S* D0 = kF32 ? (S*)a.D32h : (S*)a.D64;
+  S* D1 = kF32 ? (S*)a.D32l : nullptr;
+  S* As = (S*)cx.tsm;                 // [k][i], high words
+  S* Bs = As + kBlk * kWtLd;          // [k][j]
+  S* Al = Bs + kBlk * kWtLd;          // low words (fp32)
+  S* Bl = Al + kBlk * kWtLd;
+  constexpr int sb = kSuper;
+  const int n = cx.n, ldf = a.ldf;
+  const int i0 = (cx.tid >> 4) * 4, j0 = (cx.tid & 15) * 4;
+  for (int h = kBlk; h < sb; h *= 2) {
+    const int nt = h / kBlk, npair = (a.npad / 2) / h;
+    for (int pass = 0; pass < 2; ++pass) {
+      for (int t = cx.cta; t < 2 * npair * nt * nt; t += cx.G) {
+        const int tj = t % nt, ti = (t / nt) % nt, pr = (t / (nt * nt)) % npair, tri = t / (nt * nt * npair);
+        const bool lower = tri == 0;
+        const int o = pr * 2 * h;
+        if (o + h >= n) continue;  // no second half
+        const int oc = o % sb;     // column of the pair inside its superblock
+        // pass 0: T = F[fr..][fc..] X[xr..][xr..]; pass 1: X_off = -X T
+        const int xr = lower ? o : o + h;       // the X of pass 0 (11 / 22)
+        const int fr = lower ? o + h : o;       // rows of F, of T's target in pass 1 and of the other X
+        const int xk0 = lower ? tj : 0, xk1 = lower ? nt : tj + 1;      // pass 0: inner tiles
+        const int yk0 = lower ? 0 : ti, yk1 = lower ? ti + 1 : nt;      // pass 1
+        const int tr = lower ? o : o + h, tc = lower ? oc + h : oc;     // where T waits
+        const int k0 = pass ? yk0 : xk0, k1 = pass ? yk1 : xk1;
+        typename std::conditional<kF32, ff_t, double>::type acc[4][4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            if constexpr (kF32) acc[i][j] = ff_t{0.0f, 0.0f};
+            else acc[i][j] = 0.0;
+          }
+        for (int kt = k0; kt < k1; ++kt) {
+          __syncthreads();  // the previous staging is no longer read
+          for (int e = cx.tid; e < kBlk * kBlk; e += kRefThreads) {
+            const int r = e / kBlk, c = e % kBlk;
+            if (pass == 0) {
+              const int frow = fr + ti * kBlk + r, fcol = xr + kt * kBlk + c;
+              As[c * kWtLd + r] = (frow < n && fcol < n) ? (S)factor_at<F>(a, (size_t)frow * ldf + fcol) : (S)0;
+              const int xrow = xr + kt * kBlk + r;
+              const size_t x = wide_row(a, tri, xrow) + (xr - o) + oc + tj * kBlk + c;
+              Bs[r * kWtLd + c] = xrow < n ? __ldcg(D0 + x) : (S)0;
+              if (kF32) Bl[r * kWtLd + c] = xrow < n ? __ldcg(D1 + x) : (S)0;
+            } else {
+              const int xrow = fr + ti * kBlk + r;
+              const size_t x = wide_row(a, tri, xrow) + (fr - o) + oc + kt * kBlk + c;
+              As[c * kWtLd + r] = xrow < n ? __ldcg(D0 + x) : (S)0;
+              if (kF32) Al[c * kWtLd + r] = xrow < n ? __ldcg(D1 + x) : (S)0;
+              const int trow = kt * kBlk + r;  // inner index of T
+              const size_t y = wide_row(a, tri, tr + trow) + tc + tj * kBlk + c;
+              const bool in = fr + trow < n;   // rows of T past the matrix were not formed
+              Bs[r * kWtLd + c] = in ? __ldcg(D0 + y) : (S)0;
+              if (kF32) Bl[r * kWtLd + c] = in ? __ldcg(D1 + y) : (S)0;
+            }
+          }
+          __syncthreads();
+          if constexpr (kF32) {
+            if (pass == 0) wide_tile_mma<false>(As, Al, Bs, Bl, i0, j0, acc);
+            else wide_tile_mma<true>(As, Al, Bs, Bl, i0, j0, acc);
+          } else {
+            wide_tile_mma(As, Bs, i0, j0, acc);
+          }
+        }
+        // T to its waiting place (row index: inner index of the second
+        // product), X_off negated
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int r = ti * kBlk + i0 + i;
+          if (fr + r >= n) continue;
+          const size_t x = pass == 0 ? wide_row(a, tri, tr + r) + tc : wide_row(a, tri, fr + r) + (xr - o) + oc;
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const size_t y = x + tj * kBlk + j0 + j;
+            if constexpr (kF32) {
+              ArFF::V v = ArFF::fin(acc[i][j]);
+              if (pass) v = ArFF::neg(v);
+              D0[y] = v.h;
+              D1[y] = v.l;
+            } else {
+              D0[y] = pass ? -acc[i][j] : acc[i][j];
+            }
+          }
+        }
+      }
+      if (!grid_barrier(a.bar, a.err, cx.G)) return false;
+    }
+  }
+  return true;
+}
+
+// Wait until every word of `nval` values (W words each, at p) carries
+// `epoch`, and hand each value to put(index, words): values tid, tid +
+// kRefThreads, ... of this thread, loads of kIn values in flight.  Bounded
+// like every device wait.
+template <int W, typename Put>
+__device__ __forceinline__ bool wide_collect(const unsigned long long* p, int nval, unsigned epoch, int tid, int* err,
+                                             int where, Put put) {
+  constexpr int kIn = 4;
+  for (int v0 = tid; v0 < nval; v0 += kIn * kRefThreads) {
+    unsigned long long w[kIn][W];
+    unsigned todo = 0;
+#pragma unroll
+    for (int q = 0; q < kIn; ++q)
+      if (v0 + q * kRefThreads < nval) todo |= 1u << q;
+    unsigned long long t0 = 0;
+    unsigned spins = 0;
+    while (true) {
+#pragma unroll
+      for (int q = 0; q < kIn; ++q)
+        if (todo >> q & 1u) {
+#pragma unroll
+          for (int k = 0; k < W; ++k) w[q][k] = ld_relaxed_u64(p + (size_t)(v0 + q * kRefThreads) * W + k);
+        }
+#pragma unroll
+      for (int q = 0; q < kIn; ++q)
+        if (todo >> q & 1u) {
+          bool ok = true;
+#pragma unroll
+          for (int k = 0; k < W; ++k) ok &= (unsigned)(w[q][k] >> 32) == epoch;
+          if (ok) {
+            unsigned x[W];
+#pragma unroll
+            for (int k = 0; k < W; ++k) x[k] = (unsigned)w[q][k];
+            put(v0 + q * kRefThreads, x);
+            todo &= ~(1u << q);
+          }
+        }
+      if (!todo) break;
+      if ((++spins & 255u) == 0u) {
+        if (t0 == 0) t0 = gtimer();
+        if (ld_volatile_i32(err) != 0) return false;
+        if (gtimer() - t0 > kWaitTimeoutNs) {
+          record_timeout(err, 2, where, (int)epoch, v0);
+          return false;
+        }
+      }
+    }
+  }
+  return true;
+}
+
+template <int N> struct Int { static constexpr int value = N; };
+
+// The factor values of one thread of a wide solve, in the order of their
+// use: near(1), far(2), near(2), far(3), ...  A segment is one row's steps
+// over consecutive columns: near(t) those of superblock t - 1, far(t + 1)
+// those of superblocks 0 .. t - 1.  issue() copies the next step into the
+// ring (an empty step once nothing is left, so that every step is one copy
+// group), take() reads the oldest.
+template <typename F, bool LOWER, int WPR>
+struct WideStream {
+  static constexpr int VC = 16 / (int)sizeof(F), STEP = 32 * VC * WPR, SPB = kSuper / STEP;
+  const F* LU;
+  const F* src;
+  uint4* ring;
+  int ldf, n, NS, rpc, npass, r_lo, wp, wrow, lane, tid;
+  int t, far, ps, left, col, slot, cslot, depth;
+  bool row;
+  __device__ __forceinline__ int super(int i) const { return LOWER ? i : NS - 1 - i; }
+  // row of pass p within superblock s, or -1
+  __device__ __forceinline__ int my_row(int s, int p) const {
+    const int rr = r_lo + p * (8 / WPR) + wrow;
+    return rr < min(min(r_lo + rpc, kSuper), n - s * kSuper) ? rr : -1;
+  }
+  __device__ __forceinline__ void init(const F* LU_, int ldf_, int n_, int NS_, int rpc_, int npass_, int r_lo_, int wp_,
+                                       int wrow_, int lane_, int tid_, uint4* ring_, int depth_) {
+    LU = LU_; ldf = ldf_; n = n_; NS = NS_; rpc = rpc_; npass = npass_; r_lo = r_lo_; wp = wp_; wrow = wrow_;
+    lane = lane_; tid = tid_; ring = ring_; depth = depth_;
+    t = 0; far = 1; ps = npass - 1; left = 0; col = 0; slot = 0; cslot = 0;
+    row = false;
+    src = LU;
+  }
+  __device__ __forceinline__ void next_segment() {
+    if (t < NS && ++ps >= npass) {
+      ps = 0;
+      if (!far && t + 1 < NS) {
+        far = 1;
+      } else {
+        far = 0;
+        ++t;
+      }
+    }
+    left = 0x7fffffff;
+    row = false;
+    if (t < NS) {
+      const int s = super(far ? t + 1 : t);
+      const int rr = my_row(s, ps);
+      row = rr >= 0;
+      left = (far ? t : 1) * SPB;
+      col = (far && LOWER ? 0 : super(t - 1)) * kSuper + (wp * 32 + lane) * VC;
+      src = LU + (size_t)(s * kSuper + max(rr, 0)) * ldf;
+    }
+  }
+  __device__ __forceinline__ void issue() {
+    if (left == 0) next_segment();
+    if (row) {
+      const int valid = min(VC, max(0, n - col));  // columns past the matrix are zeros
+      cp_async16(ring + slot * kRefThreads + tid, src + (valid > 0 ? col : 0), valid * (int)sizeof(F));
+      col += STEP;
+    }
+    --left;
+    slot = slot + 1 == depth ? 0 : slot + 1;
+    cp_async_commit();
+  }
+  __device__ __forceinline__ void fill() {
+    for (int i = 4; i < depth; ++i) issue();
+  }
+  __device__ __forceinline__ uint4 take() {
+    const uint4 u = ring[cslot * kRefThreads + tid];
+    cslot = cslot + 1 == depth ? 0 : cslot + 1;
+    return u;
+  }
+};
+
+// One wide triangular solve (LOWER: L y = c; else U x = y).  WPR warps share
+// a row (columns split between them); a CTA takes rpc consecutive rows of
+// every superblock.  Not inlined (see trsv_team).
+//
+// Per superblock t (in the order of the solve):
+//   y of superblock t - 1 arrives; its products (`near`) complete z, which is
+//   handed on; while it travels, the products of superblock t + 1's rows with
+//   superblocks 0 .. t - 1 (`far`) are formed and the inverse's rows are
+//   loaded; z arrives, y = inv z is handed on.
+// The factor's values reach each thread through a ring of asynchronous
+// copies in shared memory in the order of their use, a.ring - 4 steps ahead
+// across superblocks (16 bytes per thread and step; a thread reads only what
+// it copied, so the ring needs no barrier): the loads run at memory speed
+// whatever the hand-offs do.  Every CTA keeps all of y in shared memory.
+template <typename F, typename ACC, bool LOWER, int WPR>
+__device__ __noinline__ bool trsv_wide(Cx& cx, const RefineArgs& a, int store_fmt, unsigned epoch) {
+  using WA = Wide<ACC>;
+  using AR = typename WA::AR;
+  using V = typename ACC::V;
+  using Z = typename AR::V;
+  using A = typename ACC::A;
+  using S = typename AR::S;
+  using Lt = typename ACC::L;
+  constexpr int W = ACC::kW, ZW = WA::kZW;
+  constexpr int RG = (kRefThreads / 32) / WPR;  // rows of a CTA at a time
+  constexpr int SB = kSuper;
+  constexpr int VC = 16 / (int)sizeof(F);       // factor values per thread and step
+  constexpr int STEP = 32 * VC * WPR;           // columns of a row per step
+  constexpr int SPB = SB / STEP;                // steps per superblock
+  static_assert(SPB * STEP == SB, "whole steps");
+  constexpr bool kPair = sizeof(Z) > sizeof(S);
+  const int n = cx.n, NS = a.npad / SB;
+  const int tri = LOWER ? 0 : 1;
+  const int rpc = (SB + cx.G - 1) / cx.G;       // rows of each superblock per CTA
+  const int npass = (rpc + RG - 1) / RG;
+  V* ys = (V*)cx.tsm;                           // y, npad values
+  S* zh = (S*)(ys + a.npad);                    // z of the superblock
+  S* zl = zh + SB;                              // low words (fp32)
+  A* part = (A*)(zl + SB);                      // partial sums of the rows' other warps [2][8]
+  A* facc = part + 16;                          // far sums of the next superblock's rows [npass][256]
+  uint4* ring = (uint4*)(cx.tsm + a.ring_off);  // [a.ring][256]
+  const size_t llblk = (size_t)kBlk * kLLWords;
+  unsigned long long* wy = a.ll + (size_t)tri * cx.nblk * llblk;
+  unsigned long long* wz = a.ll + (size_t)(2 + tri) * cx.nblk * llblk;
+  const unsigned long long* wfwd = a.ll;
+  const double* in_hi = LOWER ? a.c_hi : a.y_hi;
+  double* out_hi = LOWER ? a.y_hi : a.z_hi;
+  const F* LU = (const F*)a.LU;
+  const S* Ih = WA::inv_h(a);
+  const S* Il = WA::inv_l(a);
+  const int wp = cx.warp % WPR, wrow = cx.warp / WPR;
+  const int r_lo = cx.cta * rpc;
+  auto super = [&](int t) { return LOWER ? t : NS - 1 - t; };
+  // row of pass ps within superblock s, or -1
+  auto my_row = [&](int s, int ps) {
+    const int rr = r_lo + ps * RG + wrow;
+    return rr < min(min(r_lo + rpc, SB), n - s * SB) ? rr : -1;
+  };
+
+
+  WideStream<F, LOWER, WPR> q;
+  q.init(LU, a.ldf, n, NS, rpc, npass, r_lo, wp, wrow, cx.lane, cx.tid, ring, a.ring);
+  // U steps: the products of this thread's values with the y at yp, yp +
+  // STEP, .., into four interleaved sums (the chain of a compensated sum is
+  // long)
+  auto consume = [&](auto uc, const V* yp, bool have, A (&acc)[4]) {
+    constexpr int U = decltype(uc)::value;
+#pragma unroll
+    for (int h = 0; h < U; ++h) q.issue();
+    // depth - 4 + U copies are under way or waiting; the U oldest are due
+    static_assert(U <= 4, "the ring holds depth copies");
+    if (q.depth == kRingDeep) cp_async_wait<kRingDeep - 4>();
+    else cp_async_wait<kRingFlat - 4>();
+    uint4 raw[U];
+#pragma unroll
+    for (int h = 0; h < U; ++h) raw[h] = q.take();
+    if (have) {
+#pragma unroll
+      for (int h = 0; h < U; ++h) {
+        F f[VC];
+        memcpy(f, &raw[h], 16);
+        V y[VC];
+        if constexpr (VC >= 4) {
+#pragma unroll
+          for (int e = 0; e < VC; e += 4) lds4(yp + h * STEP + e, *(V(*)[4])(y + e));
+        } else {
+          y[0] = yp[h * STEP];
+          y[1] = yp[h * STEP + 1];
+        }
+#pragma unroll
+        for (int e = 0; e < VC; ++e) acc[e & 3] = ACC::fma((Lt)to_f(f[e]), y[e], acc[e & 3]);
+      }
+    }
+  };
+  auto sum4 = [&](A (&acc)[4]) { return ACC::merge(ACC::merge(acc[0], acc[1]), ACC::merge(acc[2], acc[3])); };
+  int pbuf = 0;
+  // sum over the lanes of the warps that share a row; lane 0 of the row's
+  // first warp returns the total.  One block barrier if WPR > 1 (the partial
+  // sums alternate between two buffers).
+  auto row_total = [&](A acc) -> A {
+#pragma unroll
+    for (int m = 16; m > 0; m >>= 1) acc = ACC::merge(acc, ACC::ax(acc, m));
+    if constexpr (WPR > 1) {
+      pbuf ^= 8;
+      if (wp > 0 && cx.lane == 0) part[pbuf + cx.warp] = acc;
+      __syncthreads();
+      if (wp == 0) {
+#pragma unroll
+        for (int q = 1; q < WPR; ++q) acc = ACC::merge(acc, part[pbuf + cx.warp + q]);
+      }
+    }
+    return acc;
+  };
+
+  q.fill();
+  for (int t = 0; t < NS; ++t) {
+    const int s = super(t);
+    const int R0 = s * SB, SBn = min(SB, n - R0);
+    const int where = (tri << 24) | (1 << 23) | s;
+    // z past the matrix meets zeros of the inverse (filled behind a barrier:
+    // until then the previous superblock's z may still be read)
+    auto fill_z = [&]() {
+      for (int i = SBn + cx.tid; i < SB; i += kRefThreads) {
+        zh[i] = (S)0;
+        if constexpr (kPair) zl[i] = (S)0;
+      }
+    };
+    if (t == 0) {
+      fill_z();
+      // z = c: the input of the whole superblock is already known to all
+      // (forward: c is complete; backward: the forward solve's last words)
+      bool ok = true;
+      if (LOWER) {
+        for (int i = cx.tid; i < SBn; i += kRefThreads) {
+          const Z z = WA::zval(ACC::load(in_hi, nullptr, R0 + i));
+          zh[i] = z.h;
+          if constexpr (kPair) zl[i] = z.l;
+        }
+      } else {
+        ok = wide_collect<W>(wfwd + (size_t)R0 * W, SBn, epoch - 1, cx.tid, a.err, where, [&](int i, const unsigned* w) {
+          const Z z = WA::zval(ACC::unword(w));
+          zh[i] = z.h;
+          if constexpr (kPair) zl[i] = z.l;
+        });
+      }
+      if (__syncthreads_or(!ok)) return false;
+    } else {
+      const int u = super(t - 1), N0 = u * SB, Nn = min(SB, n - N0);
+      const bool ok = wide_collect<W>(wy + (size_t)N0 * W, Nn, epoch, cx.tid, a.err, where,
+                                      [&](int i, const unsigned* w) { ys[N0 + i] = ACC::unword(w); });
+      for (int i = N0 + Nn + cx.tid; i < N0 + SB; i += kRefThreads) ys[i] = ACC::zero();
+      if (__syncthreads_or(!ok)) return false;
+      fill_z();
+      for (int ps = 0; ps < npass; ++ps) {
+        const int rr = my_row(s, ps);
+        const V c_in = rr >= 0 ? ACC::load(in_hi, nullptr, R0 + rr) : ACC::zero();
+        A ac[4] = {t > 1 ? facc[ps * kRefThreads + cx.tid] : ACC::azero(), ACC::azero(), ACC::azero(), ACC::azero()};
+#pragma unroll
+        for (int k = 0; k < SPB; ++k) consume(Int<1>(), ys + u * SB + k * STEP + (wp * 32 + cx.lane) * VC, rr >= 0, ac);
+        const A acc = row_total(sum4(ac));
+        if (rr >= 0 && wp == 0 && cx.lane == 0) {
+          const Z z = WA::zdiff(c_in, acc);
+#pragma unroll
+          for (int k = 0; k < ZW; ++k)
+            st_relaxed_u64(wz + (size_t)(R0 + rr) * ZW + k, ((unsigned long long)epoch << 32) | WA::zword(z, k));
+        }
+      }
+    }
+    // the inverse's rows (this lane's columns, 4 at a time), ahead of z
+    constexpr int kGrp = SB / (32 * 4 * WPR);   // groups of 4 columns per lane
+    constexpr int kU = 4 * (int)sizeof(S) / 16; // 16-byte loads per group
+    uint4 ih[kGrp][kU], il[kPair ? kGrp : 1][kU];
+    auto load_inv = [&](int rr) {
+      const size_t ir = wide_row(a, tri, R0 + max(rr, 0));
+#pragma unroll
+      for (int q = 0; q < kGrp; ++q) {
+        const int c = (q * WPR + wp) * 128 + cx.lane * 4;
+        const bool in = rr >= 0 && (LOWER ? c <= rr : c + 4 > rr);
+#pragma unroll
+        for (int m = 0; m < kU; ++m) {
+          ih[q][m] = in ? __ldcg((const uint4*)(Ih + ir + c) + m) : make_uint4(0, 0, 0, 0);
+          if constexpr (kPair) il[q][m] = in ? __ldcg((const uint4*)(Il + ir + c) + m) : make_uint4(0, 0, 0, 0);
+        }
+      }
+    };
+    load_inv(my_row(s, 0));
+    if (t > 0 && t + 1 < NS) {
+      for (int ps = 0; ps < npass; ++ps) {
+        const bool have = my_row(super(t + 1), ps) >= 0;
+        A ac[4] = {ACC::azero(), ACC::azero(), ACC::azero(), ACC::azero()};
+        const V* yp = ys + (LOWER ? 0 : super(t - 1) * SB) + (wp * 32 + cx.lane) * VC;
+        int k = 0;
+        for (; k + 4 <= t * SPB; k += 4, yp += 4 * STEP) consume(Int<4>(), yp, have, ac);
+        for (; k < t * SPB; ++k, yp += STEP) consume(Int<1>(), yp, have, ac);
+        facc[ps * kRefThreads + cx.tid] = sum4(ac);
+      }
+    }
+    if (t > 0) {
+      const bool ok = wide_collect<ZW>(wz + (size_t)R0 * ZW, SBn, epoch, cx.tid, a.err, where | (1 << 22),
+                                       [&](int i, const unsigned* w) {
+                                         const Z z = WA::unzword(w);
+                                         zh[i] = z.h;
+                                         if constexpr (kPair) zl[i] = z.l;
+                                       });
+      if (__syncthreads_or(!ok)) return false;
+    }
+    // y_s = S(T(inv(F_ss) z_s))
+    for (int ps = 0; ps < npass; ++ps) {
+      const int rr = my_row(s, ps);
+      if (ps > 0) load_inv(rr);
+      A ac[4] = {ACC::azero(), ACC::azero(), ACC::azero(), ACC::azero()};
+#pragma unroll
+      for (int q = 0; q < kGrp; ++q) {
+        const int c = (q * WPR + wp) * 128 + cx.lane * 4;
+        S xh[4], xl[4], h4[4], l4[4];
+        memcpy(xh, ih[q], 4 * sizeof(S));
+        if constexpr (kPair) memcpy(xl, il[q], 4 * sizeof(S));
+        lds4(zh + c, h4);
+        if constexpr (kPair) lds4(zl + c, l4);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          // inside the triangle only (the rest of the array holds other data)
+          const bool in = (LOWER ? c + e <= rr : c + e >= rr) && c + e < SBn;
+          const S x = in ? xh[e] : (S)0;
+          if constexpr (kPair) ac[e] = ArFF::term(ArFF::V{x, in ? xl[e] : (S)0}, ArFF::V{h4[e], l4[e]}, ac[e]);
+          else ac[e] = __fma_rn(x, h4[e], ac[e]);
+        }
+      }
+      const A acc = row_total(sum4(ac));
+      if (rr >= 0 && wp == 0 && cx.lane == 0) {
+        const V y = ACC::store(ACC::fin(acc), store_fmt);
+#pragma unroll
+        for (int k = 0; k < W; ++k)
+          st_relaxed_u64(wy + (size_t)(R0 + rr) * W + k, ((unsigned long long)epoch << 32) | ACC::word(y, k));
+        ACC::save(out_hi, nullptr, R0 + rr, y);
+      }
+    }
+  }
+  cp_async_wait<0>();  // no copy outlives the solve
+  __syncthreads();     // the scratch is free for the next phase
+  return true;
+}
+
+template <typename F, typename ACC, bool LOWER>
+__device__ __forceinline__ bool trsv_wide_any(Cx& cx, const RefineArgs& a, int store_fmt) {
+  const unsigned epoch = ++cx.epoch;
+  // two warps per row while a CTA has at most four rows of a superblock
+  if (kSuper <= 4 * cx.G) return trsv_wide<F, ACC, LOWER, 2>(cx, a, store_fmt, epoch);
+  return trsv_wide<F, ACC, LOWER, 1>(cx, a, store_fmt, epoch);
+}
+
 // M^{-1} applied to the right-hand side already placed in c (permuted
 // order, scaled by R, rounded to the storage format): forward then backward
 // substitution.  Result in z (natural order, before the S*mu scaling).
+// `synced`: c is complete grid-wide (a barrier lies behind it), and the
+// caller puts a barrier before it reads z; otherwise c and z belong to the
+// CTAs b mod G of the 64-row blocks.
 template <typename F, typename ACC>
-__device__ bool msolve(Cx& cx, const RefineArgs& a, int store_fmt) {
+__device__ bool msolve(Cx& cx, const RefineArgs& a, int store_fmt, bool synced) {
+  // (a solve that rounds its components to a 16-bit format hands each 64-row
+  // block's rounded values on to the next: in superblocks the components of
+  // one superblock would not see each other's rounding, which doubles the
+  // error of the result)
+  if (use_wide<ACC, F>(a) && (ACC::kW == 2 || store_fmt >= MSIR_FP32)) {
+    if constexpr (!std::is_same<F, FAny>::value && ACC::kW <= 2) {
+      constexpr bool k32 = ACC::kW == 1;
+      const unsigned need = k32 ? RDY_W32 : RDY_W64;
+      if (!(cx.mready & need)) {
+        if (k32 || !(cx.mready & RDY_INV)) {
+          if (!build_inverses<F>(cx, a, !k32, true)) return false;
+          if (!k32) cx.mready |= RDY_INV;
+        }
+        if (!build_wide<F, k32>(cx, a)) return false;
+        cx.mready |= need;
+      }
+      if (!synced && !grid_barrier(a.bar, a.err, cx.G)) return false;
+      {
+        PhaseTimer pt(cx, 1);
+        if (!trsv_wide_any<F, ACC, true>(cx, a, store_fmt)) return false;
+      }
+      PhaseTimer pt(cx, 2);
+      if (!trsv_wide_any<F, ACC, false>(cx, a, store_fmt)) return false;
+      return synced || grid_barrier(a.bar, a.err, cx.G);
+    }
+  }
   // inverses and scaled blocks of the current factors in this precision, once
   const bool f64 = factor_fmt<F>(a) == MSIR_FP64;
   const unsigned need = ACC::kW == 4 ? RDY_MDD : (ACC::kW == 2 || f64) ? RDY_M64 : RDY_M32;
   if (!(cx.mready & need)) {
     if (need == RDY_M32) {
-      if (!build_inverses<F>(cx, a, false) || !build_scaled32<F>(cx, a)) return false;
+      if (!build_inverses<F>(cx, a, false, false) || !build_scaled32<F>(cx, a)) return false;
     } else {
-      if (!(cx.mready & RDY_INV) && !build_inverses<F>(cx, a, true)) return false;
+      if (!(cx.mready & RDY_INV) && !build_inverses<F>(cx, a, true, false)) return false;
       if (!build_scaled<F>(cx, a, need == RDY_MDD)) return false;
       cx.mready |= RDY_INV;
     }
@@ -1275,7 +1914,7 @@ __device__ bool msolve(Cx& cx, const RefineArgs& a, int store_fmt) {
   // Rows of block b are prepared (c) and consumed (z) by CTA b mod G.  A
   // team of K > 1 CTAs spreads them over other CTAs, so c must be visible
   // grid-wide before the forward solve and z after the backward solve.
-  const bool team = team_size<ACC>(cx) > 1;
+  const bool team = !synced && team_size<ACC>(cx) > 1;
   if (team && !grid_barrier(a.bar, a.err, cx.G)) return false;
   {
     PhaseTimer pt(cx, 1);
@@ -1287,10 +1926,10 @@ __device__ bool msolve(Cx& cx, const RefineArgs& a, int store_fmt) {
 }
 
 template <typename F>
-__device__ bool msolve_arith(Cx& cx, const RefineArgs& a, int arith, int store_fmt) {
-  if (arith == MSIR_FP32) return msolve<F, AccF>(cx, a, store_fmt);
-  if (arith == MSIR_FP64) return msolve<F, AccD>(cx, a, store_fmt);
-  return msolve<F, AccDD>(cx, a, store_fmt);
+__device__ bool msolve_arith(Cx& cx, const RefineArgs& a, int arith, int store_fmt, bool synced = false) {
+  if (arith == MSIR_FP32) return msolve<F, AccF>(cx, a, store_fmt, synced);
+  if (arith == MSIR_FP64) return msolve<F, AccD>(cx, a, store_fmt, synced);
+  return msolve<F, AccDD>(cx, a, store_fmt, synced);
 }
 
 // right-hand side element of a substitution in precision `arith`
@@ -1424,25 +2063,26 @@ template <> struct UA<double> {
 };
 
 // Operator t = A v (rows perm[i]) in the operator precision, scaled by R,
-// placed in c.  op = FP32: compensated fp32 sums (the accurately rounded
-// fp32 value of each row's sum), rows of my blocks (no barrier needed before
-// the substitution); FP64 / DD: rows over every warp of the grid, followed
-// by a grid barrier.
+// placed in c, rows over every warp of the grid, followed by a grid barrier.
+// op = FP32: compensated fp32 sums (the accurately rounded fp32 value of
+// each row's sum).
 template <typename A0, typename U>
 __device__ __noinline__ bool apply_A(Cx& cx, const RefineArgs& a, const U* v, int op) {
   PhaseTimer pt(cx, 4);
   const A0* A = (const A0*)a.A;
   if (op == MSIR_FP32) {
-    // a warp's 8 rows together: v is loaded once per column and the eight
-    // rows' loads and sums are independent, so their latencies overlap
-    for (int b = cx.cta; b < cx.nblk; b += cx.G) {
-      const int i0 = b * kBlk + cx.warp * 8;
-      if (i0 >= cx.n) continue;
+    // a warp's rows (up to 8, consecutive) together: v is loaded once per
+    // column and the rows' loads and sums are independent, so their
+    // latencies overlap
+    const int nwarps = cx.G * (kRefThreads / 32);
+    const int rpw = min(8, (cx.n + nwarps - 1) / nwarps);
+    for (int i0 = (cx.cta * (kRefThreads / 32) + cx.warp) * rpw; i0 < cx.n; i0 += nwarps * rpw) {
+      const int nr = min(rpw, cx.n - i0);
       const A0* rows[8];
       ff_t acc[8];
 #pragma unroll
       for (int rr = 0; rr < 8; ++rr) {
-        const int i = min(i0 + rr, cx.n - 1);  // rows past n repeat the last one, never stored
+        const int i = i0 + min(rr, nr - 1);  // rows past nr repeat the last one, never stored
         rows[rr] = A + (size_t)a.perm[i] * a.lda;
         acc[rr] = ff_t{0.0f, 0.0f};
       }
@@ -1456,7 +2096,8 @@ __device__ __noinline__ bool apply_A(Cx& cx, const RefineArgs& a, const U* v, in
         if (j < n4) {
           ld4f_vec<U>(v + j, vn);
 #pragma unroll
-          for (int rr = 0; rr < 8; ++rr) ld4f_row<A0>(rows[rr] + j, an[rr]);
+          for (int rr = 0; rr < 8; ++rr)
+            if (rr < nr) ld4f_row<A0>(rows[rr] + j, an[rr]);
         }
         for (; j < n4; j += 128) {
           float ac[8][4], vc[4];
@@ -1469,12 +2110,15 @@ __device__ __noinline__ bool apply_A(Cx& cx, const RefineArgs& a, const U* v, in
           if (j + 128 < n4) {
             ld4f_vec<U>(v + j + 128, vn);
 #pragma unroll
-            for (int rr = 0; rr < 8; ++rr) ld4f_row<A0>(rows[rr] + j + 128, an[rr]);
+            for (int rr = 0; rr < 8; ++rr)
+              if (rr < nr) ld4f_row<A0>(rows[rr] + j + 128, an[rr]);
           }
 #pragma unroll
           for (int rr = 0; rr < 8; ++rr)
+            if (rr < nr) {
 #pragma unroll
-            for (int q = 0; q < 4; ++q) acc[rr] = ff_fma(ac[rr][q], vc[q], acc[rr]);
+              for (int q = 0; q < 4; ++q) acc[rr] = ff_fma(ac[rr][q], vc[q], acc[rr]);
+            }
         }
       }
       for (int j = n4 + cx.lane; j < cx.n; j += 32) {
@@ -1486,7 +2130,7 @@ __device__ __noinline__ bool apply_A(Cx& cx, const RefineArgs& a, const U* v, in
       for (int rr = 0; rr < 8; ++rr)
 #pragma unroll
         for (int m = 16; m > 0; m >>= 1) acc[rr] = ff_merge(acc[rr], ff_shfl_xor(acc[rr], m));
-      if (cx.lane < 8 && i0 + cx.lane < cx.n) {
+      if (cx.lane < nr) {
         float mine = ff_fin(acc[0]);
 #pragma unroll
         for (int rr = 1; rr < 8; ++rr)
@@ -1496,8 +2140,7 @@ __device__ __noinline__ bool apply_A(Cx& cx, const RefineArgs& a, const U* v, in
         ((float*)a.c_hi)[i0 + cx.lane] = __fmul_rn(mine, R);
       }
     }
-    __syncthreads();
-    return true;
+    return grid_barrier(a.bar, a.err, cx.G);
   }
   const int nw = cx.G * (kRefThreads / 32);
   if (op == MSIR_DD) {
@@ -1793,7 +2436,7 @@ __device__ bool gmres(Cx& cx, const RefineArgs& a, double s, int ur, int u, int 
     // full V_k needed by the matrix-vector product
     if (!grid_barrier(a.bar, a.err, cx.G)) return false;
     if (!apply_A<A0, U>(cx, a, vk, op)) return false;
-    if (!msolve_arith<F>(cx, a, op, op)) return false;
+    if (!msolve_arith<F>(cx, a, op, op, true)) return false;
     if (!finish_solve<U>(cx, a, w, op)) return false;
     // classical Gram-Schmidt, twice
     cgs_partials<U>(cx, a, V, w, k + 1);
@@ -2185,7 +2828,7 @@ template <typename A0, typename F>
 // of one system then slow the other's.)
 __global__ void __launch_bounds__(kRefThreads, 1) refine_kernel(RefineArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  unsigned char* gsm = smem_raw + kGmresOff;  // GMRES scalars
+  unsigned char* gsm = smem_raw + a.gmres_off;  // GMRES scalars
   __shared__ RefState S;
   __shared__ int s_act, s_reset, s_alg;
 

@@ -12,9 +12,15 @@ template <typename A0, typename F> void* refine_entry();
 
 // ---------------------------------------------------------- launchers
 
-size_t refine_smem_bytes(int kcap) {
-  return kGmresOff +
-         sizeof(double) * (3 * ((size_t)kcap + 2) + 2 * ((size_t)kcap + 1));
+static size_t gmres_smem(int kcap) { return sizeof(double) * (3 * ((size_t)kcap + 2) + 2 * ((size_t)kcap + 1)); }
+
+size_t refine_smem_bytes(int kcap, size_t phase) {
+  return kInboxSmem + std::max<size_t>(kPhaseSmem, phase) + gmres_smem(kcap);
+}
+
+// scratch that the wide solves of a launch need
+static size_t wide_phase(const RefineArgs& a) {
+  return a.wide ? (size_t)a.ring_off + (size_t)a.ring * kRefThreads * 16 : 0;
 }
 
 template <typename A0, typename F>
@@ -97,10 +103,11 @@ int refine_max_cluster_grid(int a_fmt, int kcap, int cluster) {
 cudaError_t launch_refine(int a_fmt, int f_fmt, const RefineArgs& a, int grid, cudaStream_t st) {
   void* fn = pick(a_fmt, f_fmt);
   if (!fn) return cudaErrorInvalidValue;
-  const size_t smem = refine_smem_bytes(a.kcap);
+  const size_t smem = refine_smem_bytes(a.kcap, wide_phase(a));
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   RefineArgs copy = a;
+  copy.gmres_off = (int)(smem - gmres_smem(a.kcap));
   if (a.cluster > 1) {
     if (grid % a.cluster != 0) return cudaErrorInvalidValue;
     cudaLaunchAttribute at[2];

@@ -68,3 +68,14 @@ def test_block_diagonals_near_the_ends_of_fp32(ctx, uf, scale):
     solution scales exactly against the unscaled factors' bound."""
     A, _, _ = randsvd_system(150, 1e3, 41)
     _check(ctx, scale * A, OF.FP32, uf, [(OF.FP32, OF.FP32)])
+
+
+@pytest.mark.parametrize("n", [1023, 1024, 1025, 1536, 1793, 2049])
+@pytest.mark.parametrize("uf", [OF.FP16, OF.FP32, OF.FP64])
+def test_wide_solve_edges(ctx, n, uf):
+    """Around the smallest sizes of the superblock solves, whole and ragged
+    last superblocks (one row, one missing), fp32 and fp64 arithmetic, and a
+    16-bit storage format (which keeps the 64-row solve)."""
+    A, _, _ = randsvd_system(n, 1e3, 50 + n)
+    u = OF.FP64 if uf in (OF.FP32, OF.FP64) else OF.FP32
+    _check(ctx, A, u, uf, [(OF.FP32, OF.FP32), (OF.FP64, OF.FP64), (OF.FP32, OF.FP16)])
