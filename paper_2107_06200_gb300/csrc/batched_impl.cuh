@@ -238,6 +238,8 @@ __global__ void __launch_bounds__(kBatchThreads, 1) batched_solve_kernel(BatchAr
     a.allow_escalation = B.allow_escalation;
     a.u0 = u0;
     a.cluster = 1;
+    a.gmres_off = kGmresOff;
+    a.scratch = kPhaseSmem;
     Cx cx;
     cx.tsm = smem_raw + kScratchOff;
     cx.ssm = cx.tsm + kTrsvSmem;

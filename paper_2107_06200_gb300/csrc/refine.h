@@ -137,7 +137,7 @@ struct RefineArgs {
   double* V;               // Krylov basis in u, row-major: entry j of row i at
   int ldv;                 //   V + i*ldv (ldv >= kcap + 1)
   double* vk;              // the newest basis vector, contiguous (operator input)
-  double* H;               // rotated Hessenberg, column-major (kcap+1) x kcap
+  double* H;               // rotated Hessenberg, row-major, leading dimension kcap + 1
   double* yv;              // GMRES least-squares solution (kcap)
   double* red;             // reduction scratch: 2 * gridDim.x * kRedW
   double* hred;            // CGS partial sums: gridDim.x * (kcap+1)
@@ -163,7 +163,8 @@ struct RefineArgs {
   // (kRingDeep or kRingFlat) and its offset in the scratch, the inverses of the diagonal
   // superblocks of L and U, [2][npad][kSuper] (fp32 pairs, fp64)
   int npad, wide, ring, ring_off;
-  int gmres_off;           // offset of the GMRES scalars in shared memory (set by launch_refine)
+  int gmres_off;           // offset of the GMRES scalars in shared memory, and
+  int scratch;             // bytes of the scratch before them (set by the launcher)
   float* D32h;
   float* D32l;
   double* D64;

@@ -87,184 +87,191 @@ static __device__ __forceinline__ double unit_roundoff(int f) {
   }
 }
 
-template <typename A0> struct AV;
-template <> struct AV<float> {
-  static __device__ __forceinline__ double ld(const float* p) { return (double)__ldg(p); }
-};
-template <> struct AV<double> {
-  static __device__ __forceinline__ double ld(const double* p) { return __ldg(p); }
-};
+// 16-byte asynchronous copy global -> shared (L2 only) with zero fill past
+// `bytes` (0..16); groups of them are committed and waited for per thread.
+__device__ __forceinline__ void cp_async16(void* sdst, const void* gsrc, int bytes) {
+  const unsigned sa = (unsigned)__cvta_generic_to_shared(sdst);
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(sa), "l"(gsrc), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
-// Four consecutive values widened to double from a 16-byte aligned
-// address: matrix rows through the read-only path, vectors through L2
-// (they are rewritten during the kernel).
-template <typename T> struct Ld4;
-template <> struct Ld4<float> {
-  static __device__ __forceinline__ void row(const float* p, double (&v)[4]) {
-    const float4 f = __ldg((const float4*)p);
-    v[0] = f.x; v[1] = f.y; v[2] = f.z; v[3] = f.w;
-  }
-  static __device__ __forceinline__ void vec(const float* p, double (&v)[4]) {
-    const float4 f = __ldcg((const float4*)p);
-    v[0] = f.x; v[1] = f.y; v[2] = f.z; v[3] = f.w;
-  }
+// Accumulators of the row products: fp32 compensated (Dot2), fp64, and
+// fp64 compensated (twice the working precision, result as dd).
+template <int OP> struct RowAcc;
+template <> struct RowAcc<MSIR_FP32> {
+  using R = float;
+  ff_t a{0.0f, 0.0f};
+  __device__ __forceinline__ void add(float x, float y) { a = ff_fma(x, y, a); }
+  __device__ __forceinline__ void merge(const RowAcc& o) { a = ff_merge(a, o.a); }
+  __device__ __forceinline__ RowAcc peer(int m) const { return RowAcc{ff_shfl_xor(a, m)}; }
+  __device__ __forceinline__ R fin() const { return ff_fin(a); }
 };
-template <> struct Ld4<double> {
-  static __device__ __forceinline__ void row(const double* p, double (&v)[4]) {
-    const double2 f = __ldg((const double2*)p), g = __ldg((const double2*)p + 1);
-    v[0] = f.x; v[1] = f.y; v[2] = g.x; v[3] = g.y;
-  }
-  static __device__ __forceinline__ void vec(const double* p, double (&v)[4]) {
-    const double2 f = __ldcg((const double2*)p), g = __ldcg((const double2*)p + 1);
-    v[0] = f.x; v[1] = f.y; v[2] = g.x; v[3] = g.y;
-  }
+template <> struct RowAcc<MSIR_FP64> {
+  using R = double;
+  double a = 0.0;
+  __device__ __forceinline__ void add(double x, double y) { a = __fma_rn(x, y, a); }
+  __device__ __forceinline__ void merge(const RowAcc& o) { a = __dadd_rn(a, o.a); }
+  __device__ __forceinline__ RowAcc peer(int m) const { return RowAcc{__shfl_xor_sync(0xffffffffu, a, m)}; }
+  __device__ __forceinline__ R fin() const { return a; }
 };
-
-// Four consecutive values as float (fp32 paths: no fp64 conversions).
-template <typename T>
-__device__ __forceinline__ void ld4f_row(const T* p, float (&v)[4]) {
-  if constexpr (sizeof(T) == 4) {
-    const float4 f = __ldg((const float4*)p);
-    v[0] = f.x; v[1] = f.y; v[2] = f.z; v[3] = f.w;
-  } else {
-#pragma unroll
-    for (int q = 0; q < 4; ++q) v[q] = (float)__ldg(p + q);
-  }
-}
-template <typename T>
-__device__ __forceinline__ void ld4f_vec(const T* p, float (&v)[4]) {
-  if constexpr (sizeof(T) == 4) {
-    const float4 f = __ldcg((const float4*)p);
-    v[0] = f.x; v[1] = f.y; v[2] = f.z; v[3] = f.w;
-  } else {
-#pragma unroll
-    for (int q = 0; q < 4; ++q) v[q] = (float)__ldcg(p + q);
-  }
-}
-
-// Row dot products a_row . x by one warp (result on every lane).  Lanes
-// take four consecutive columns at a time with 16-byte loads, several
-// steps in flight, so that a warp streams its row at HBM speed; rows start
-// on 64-element boundaries, x is checked for 16-byte alignment.
-template <typename A0, typename X>
-__device__ double row_dot_d(const A0* row, const X* x, int n, int lane) {
-  double acc = 0.0;
-  const int n4 = ((reinterpret_cast<uintptr_t>(x) & 15) == 0) ? (n & ~3) : 0;
-#pragma unroll 4
-  for (int j = lane * 4; j < n4; j += 128) {
-    double av[4], xv[4];
-    Ld4<A0>::row(row + j, av);
-    Ld4<X>::vec(x + j, xv);
-#pragma unroll
-    for (int q = 0; q < 4; ++q) acc = __fma_rn(av[q], xv[q], acc);
-  }
-  for (int j = n4 + lane; j < n; j += 32) acc = __fma_rn(AV<A0>::ld(row + j), (double)__ldcg(x + j), acc);
-  return warp_sum_d(acc);
-}
-// row_dot_d for NR rows at once (the same sums, row by row): x is loaded
-// once for all rows, and the rows' chains and reductions are independent,
-// so one warp keeps more loads and fp64 work in flight.  (The dd product
-// keeps one row per warp: it is bound by fp64 throughput, not latency.)
-template <typename A0, typename X, int NR>
-__device__ void rows_dot_d(const A0* const (&row)[NR], const X* x, int n, int lane, double (&out)[NR]) {
-  double acc[NR];
-#pragma unroll
-  for (int r = 0; r < NR; ++r) acc[r] = 0.0;
-  const int n4 = ((reinterpret_cast<uintptr_t>(x) & 15) == 0) ? (n & ~3) : 0;
-  if constexpr (sizeof(A0) == 4 && sizeof(X) == 4) {
-    // fp32 matrix and vector: widened by integer instructions (the fp64
-    // pipe then only does the fused multiply-adds); a step with a subnormal,
-    // infinite or NaN operand on any lane takes the hardware conversion.
-    // The step loop is warp-uniform (the vote needs every lane): lanes past
-    // n4 in the last step load nothing and add zeros.  Two accumulators per
-    // row (columns 0, 2 and 1, 3 of each step) keep four independent fp64
-    // chains per warp in flight.
-    double acc2[NR];
-#pragma unroll
-    for (int r = 0; r < NR; ++r) acc2[r] = 0.0;
-#pragma unroll 2
-    for (int j0 = 0; j0 < n4; j0 += 128) {
-      const int j = j0 + lane * 4;
-      const bool in = j < n4;
-      const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
-      const float4 xf = in ? __ldcg((const float4*)(x + j)) : z4;
-      float4 af[NR];
-      bool sp = widen_special4(xf);
-#pragma unroll
-      for (int r = 0; r < NR; ++r) {
-        af[r] = in ? __ldg((const float4*)(row[r] + j)) : z4;
-        sp |= widen_special4(af[r]);
-      }
-      if (__any_sync(0xffffffffu, sp)) {
-#pragma unroll
-        for (int r = 0; r < NR; ++r) {
-          acc[r] = __fma_rn((double)af[r].x, (double)xf.x, acc[r]);
-          acc2[r] = __fma_rn((double)af[r].y, (double)xf.y, acc2[r]);
-          acc[r] = __fma_rn((double)af[r].z, (double)xf.z, acc[r]);
-          acc2[r] = __fma_rn((double)af[r].w, (double)xf.w, acc2[r]);
-        }
-      } else {
-        const double x0 = widen_normal(xf.x), x1 = widen_normal(xf.y), x2 = widen_normal(xf.z),
-                     x3 = widen_normal(xf.w);
-#pragma unroll
-        for (int r = 0; r < NR; ++r) {
-          acc[r] = __fma_rn(widen_normal(af[r].x), x0, acc[r]);
-          acc2[r] = __fma_rn(widen_normal(af[r].y), x1, acc2[r]);
-          acc[r] = __fma_rn(widen_normal(af[r].z), x2, acc[r]);
-          acc2[r] = __fma_rn(widen_normal(af[r].w), x3, acc2[r]);
-        }
-      }
-    }
-#pragma unroll
-    for (int r = 0; r < NR; ++r) acc[r] = __dadd_rn(acc[r], acc2[r]);
-  } else {
-#pragma unroll 2
-    for (int j = lane * 4; j < n4; j += 128) {
-      double xv[4];
-      Ld4<X>::vec(x + j, xv);
-#pragma unroll
-      for (int r = 0; r < NR; ++r) {
-        double av[4];
-        Ld4<A0>::row(row[r] + j, av);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) acc[r] = __fma_rn(av[q], xv[q], acc[r]);
-      }
-    }
-  }
-  for (int j = n4 + lane; j < n; j += 32) {
-    const double xj = (double)__ldcg(x + j);
-#pragma unroll
-    for (int r = 0; r < NR; ++r) acc[r] = __fma_rn(AV<A0>::ld(row[r] + j), xj, acc[r]);
-  }
-#pragma unroll
-  for (int r = 0; r < NR; ++r) out[r] = warp_sum_d(acc[r]);
-}
-// Compensated (twice-working-precision) dot product, result as dd.
-template <typename A0, typename X>
-__device__ dd_t row_dot_dd(const A0* row, const X* x, int n, int lane) {
+template <> struct RowAcc<MSIR_DD> {
+  using R = dd_t;
   double s = 0.0, c = 0.0;
-  const int n4 = ((reinterpret_cast<uintptr_t>(x) & 15) == 0) ? (n & ~3) : 0;
-#pragma unroll 2
-  for (int j = lane * 4; j < n4; j += 128) {
-    double av[4], xv[4];
-    Ld4<A0>::row(row + j, av);
-    Ld4<X>::vec(x + j, xv);
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const dd_t p = two_prod(av[q], xv[q]);
-      const dd_t t = two_sum_ord(s, p.hi);
-      s = t.hi;
-      c = __dadd_rn(c, __dadd_rn(t.lo, p.lo));
-    }
-  }
-  for (int j = n4 + lane; j < n; j += 32) {
-    const dd_t p = two_prod(AV<A0>::ld(row + j), (double)__ldcg(x + j));
+  __device__ __forceinline__ void add(double x, double y) {
+    const dd_t p = two_prod(x, y);
     const dd_t t = two_sum_ord(s, p.hi);
     s = t.hi;
     c = __dadd_rn(c, __dadd_rn(t.lo, p.lo));
   }
-  dd_t v = fast_two_sum(s, c);
-  return warp_sum_dd(v);
+  __device__ __forceinline__ void merge(const RowAcc& o) {
+    const dd_t v = dd_add(fast_two_sum(s, c), fast_two_sum(o.s, o.c));
+    s = v.hi;
+    c = v.lo;
+  }
+  __device__ __forceinline__ RowAcc peer(int m) const {
+    return RowAcc{__shfl_xor_sync(0xffffffffu, s, m), __shfl_xor_sync(0xffffffffu, c, m)};
+  }
+  __device__ __forceinline__ R fin() const { return fast_two_sum(s, c); }
+};
+
+// Products of rows perm[i] of A with x in arithmetic OP, NR consecutive rows
+// per warp; epi(i, perm[i], a . x) runs on one lane per row.
+//
+// The rows' values and x's reach each lane through a ring of asynchronous
+// copies in the shared scratch (16 bytes per row and step, up to 4 steps
+// deep; a lane reads only what it copied itself: no barriers), so a CTA
+// keeps up to 100 KB of loads in flight whatever its registers hold.  NR is
+// fixed at compile time and rows past the matrix repeat the last one: with a
+// test per row the rows' sums ran one after another (n = 2000 fp64: 43 us
+// instead of 11).  Each row has two sums (even and odd columns), because
+// the chain of one is longer than a step's loads.  What bounds it: HBM for
+// fp32 sums (n = 8192: 94 -> 60 us, 4.5 TB/s), the fp64 pipe (2 multiply-adds
+// per clock and SM) for fp64 ones on fp32 data, where values are widened by
+// integer instructions (steps with a subnormal, infinite or NaN operand on
+// any lane take the hardware conversion).
+template <typename A0, typename X, int OP, int NR, typename Epi>
+__device__ __forceinline__ void gemv_rows_n(Cx& cx, const RefineArgs& a, const X* x, Epi& epi) {
+  constexpr int VC = 16 / (int)sizeof(A0);               // columns per lane and step
+  constexpr int XS = (VC * (int)sizeof(X) + 15) / 16;    // 16-byte pieces of x per lane and step
+  constexpr int STEP = 32 * VC, UNIT = (NR + XS) * kRefThreads;
+  static_assert(VC * sizeof(X) >= 16, "a lane's x fills whole pieces");
+  static_assert(2 * UNIT * 16 <= kPhaseSmem, "the scratch holds two steps");
+  using Acc = RowAcc<OP>;
+  const A0* A = (const A0*)a.A;
+  const int n = cx.n, lane = cx.lane, nwarps = cx.G * (kRefThreads / 32), gw = cx.cta * (kRefThreads / 32) + cx.warp;
+  const int depth = min(4, a.scratch / (UNIT * 16));     // 2, 3 or 4
+  uint4* ring = (uint4*)cx.tsm + cx.tid;
+  const int nsteps = (n + STEP - 1) / STEP;
+  for (int i0 = gw * NR; i0 < n; i0 += nwarps * NR) {
+    const A0* row[NR];
+    Acc acc[NR][2];
+#pragma unroll
+    for (int r = 0; r < NR; ++r) row[r] = A + (size_t)a.perm[min(i0 + r, n - 1)] * a.lda;
+    // each warp starts at columns of its own and wraps around: in step, the
+    // warps would all read the same few lines of x at once, and the L2 slices
+    // that hold them would serve one after another
+    int ist = (int)((long long)gw * nsteps / nwarps), islot = 0;
+    auto issue = [&](int st) {
+      if (st < nsteps) {
+        const int col = ist * STEP + lane * VC;
+        ist = ist + 1 == nsteps ? 0 : ist + 1;
+        const int valid = min(VC, max(0, n - col)), c = valid > 0 ? col : 0;  // zeros past n
+        uint4* dst = ring + islot * UNIT;
+#pragma unroll
+        for (int r = 0; r < NR; ++r) cp_async16(dst + r * kRefThreads, row[r] + c, valid * (int)sizeof(A0));
+#pragma unroll
+        for (int q = 0; q < XS; ++q) {
+          constexpr int XC = 16 / (int)sizeof(X);
+          const int xc = col + q * XC, xv = min(XC, max(0, n - xc));
+          cp_async16(dst + (NR + q) * kRefThreads, x + (xv > 0 ? xc : 0), xv * (int)sizeof(X));
+        }
+      }
+      islot = islot + 1 == depth ? 0 : islot + 1;
+      cp_async_commit();
+    };
+    for (int st = 0; st < depth - 1; ++st) issue(st);
+    int slot = 0;
+    for (int st = 0; st < nsteps; ++st) {
+      issue(st + depth - 1);
+      if (depth == 4) cp_async_wait<3>();
+      else if (depth == 3) cp_async_wait<2>();
+      else cp_async_wait<1>();
+      const uint4* src = ring + slot * UNIT;
+      slot = slot + 1 == depth ? 0 : slot + 1;
+      X xv[VC];
+#pragma unroll
+      for (int q = 0; q < XS; ++q) {
+        const uint4 u = src[(NR + q) * kRefThreads];
+        memcpy((char*)xv + 16 * q, &u, 16);
+      }
+      A0 av[NR][VC];
+#pragma unroll
+      for (int r = 0; r < NR; ++r) {
+        const uint4 u = src[r * kRefThreads];
+        memcpy(av[r], &u, 16);
+      }
+      if constexpr (OP != MSIR_FP32 && sizeof(A0) == 4) {
+        bool sp = false;
+        double xd[VC];
+#pragma unroll
+        for (int q = 0; q < VC; ++q) {
+          if constexpr (sizeof(X) == 4) {
+            sp |= widen_special(xv[q]);
+            xd[q] = widen_normal(xv[q]);
+          } else {
+            xd[q] = xv[q];
+          }
+        }
+#pragma unroll
+        for (int r = 0; r < NR; ++r)
+#pragma unroll
+          for (int q = 0; q < VC; ++q) sp |= widen_special(av[r][q]);
+        if (__any_sync(0xffffffffu, sp)) {
+#pragma unroll
+          for (int q = 0; q < VC; ++q)
+#pragma unroll
+            for (int r = 0; r < NR; ++r) acc[r][q & 1].add((double)av[r][q], (double)xv[q]);
+        } else {
+#pragma unroll
+          for (int q = 0; q < VC; ++q)
+#pragma unroll
+            for (int r = 0; r < NR; ++r) acc[r][q & 1].add(widen_normal(av[r][q]), xd[q]);
+        }
+      } else {
+#pragma unroll
+        for (int q = 0; q < VC; ++q)
+#pragma unroll
+          for (int r = 0; r < NR; ++r) acc[r][q & 1].add(av[r][q], xv[q]);
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < NR; ++r) acc[r][0].merge(acc[r][1]);
+#pragma unroll
+    for (int m = 16; m > 0; m >>= 1)
+#pragma unroll
+      for (int r = 0; r < NR; ++r) acc[r][0].merge(acc[r][0].peer(m));
+#pragma unroll
+    for (int r = 0; r < NR; ++r)
+      if (lane == r && i0 + r < n) epi(i0 + r, a.perm[i0 + r], acc[r][0].fin());
+  }
+  cp_async_wait<0>();  // (empty groups: every copy has been waited for)
+}
+
+// All rows: the fewest rows per warp (of 1, 2, 4, 7, 8) that take one round;
+// one at a time in double-double, which the fp64 pipe bounds (n = 8192: 7
+// rounds of one row 1.26 ms, 2 rounds of four 1.47 ms).
+template <typename A0, typename X, int OP, typename Epi>
+__device__ __forceinline__ void gemv_rows(Cx& cx, const RefineArgs& a, const X* x, Epi epi) {
+  const int nwarps = cx.G * (kRefThreads / 32);
+  const int rpw = (cx.n + nwarps - 1) / nwarps;
+  if (rpw <= 1 || OP == MSIR_DD) gemv_rows_n<A0, X, OP, 1>(cx, a, x, epi);
+  else if constexpr (OP == MSIR_DD) return;
+  else if (rpw <= 2) gemv_rows_n<A0, X, OP, 2>(cx, a, x, epi);
+  else if (rpw <= 4) gemv_rows_n<A0, X, OP, 4>(cx, a, x, epi);
+  else if (rpw <= 7) gemv_rows_n<A0, X, OP, 7>(cx, a, x, epi);
+  else gemv_rows_n<A0, X, OP, 8>(cx, a, x, epi);
 }
 
 // Reduce NV per-CTA values (each already reduced within the CTA and held by
@@ -971,16 +978,6 @@ __device__ __noinline__ bool build_scaled(Cx& cx, const RefineArgs& a, bool dd) 
   }
   return grid_barrier(a.bar, a.err, cx.G);
 }
-
-// 16-byte asynchronous copy global -> shared (L2 only) with zero fill past
-// `bytes` (0..16); groups of them are committed and waited for per thread.
-__device__ __forceinline__ void cp_async16(void* sdst, const void* gsrc, int bytes) {
-  const unsigned sa = (unsigned)__cvta_generic_to_shared(sdst);
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(sa), "l"(gsrc), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
 // Depth of the ring of scaled-block tiles that fp32 / fp64 substitutions
 // stream through shared memory (the scaled-block staging area, idle during
@@ -1972,23 +1969,21 @@ template <typename A0>
 __device__ __noinline__ bool residual(Cx& cx, const RefineArgs& a, const double* x, int ur, double& s,
                          double& xnorm, double* ferr = nullptr) {
   PhaseTimer pt(cx, 0);
-  const A0* A = (const A0*)a.A;
   double mr = 0.0, mx = 0.0;
-  const int nw = cx.G * (kRefThreads / 32);
-  for (int i = cx.cta * (kRefThreads / 32) + cx.warp; i < cx.n; i += nw) {
-    const int ar = a.perm[i];
-    const A0* row = A + (size_t)ar * a.lda;
-    if (ur == MSIR_DD) {
-      const dd_t ax = row_dot_dd<A0>(row, x, cx.n, cx.lane);
+  if (ur == MSIR_DD) {
+    gemv_rows<A0, double, MSIR_DD>(cx, a, x, [&](int i, int ar, dd_t ax) {
       const dd_t r = dd_sub(dd_t{a.b[ar], 0.0}, ax);
-      if (cx.lane == 0) { a.r_hi[i] = r.hi; a.r_lo[i] = r.lo; }
+      a.r_hi[i] = r.hi;
+      a.r_lo[i] = r.lo;
       mr = nanmax(mr, fabs(r.hi));
-    } else {
-      const double ax = row_dot_d<A0>(row, x, cx.n, cx.lane);
+    });
+  } else {
+    gemv_rows<A0, double, MSIR_FP64>(cx, a, x, [&](int i, int ar, double ax) {
       const double r = __dsub_rn(a.b[ar], ax);
-      if (cx.lane == 0) { a.r_hi[i] = r; a.r_lo[i] = 0.0; }
+      a.r_hi[i] = r;
+      a.r_lo[i] = 0.0;
       mr = nanmax(mr, fabs(r));
-    }
+    });
   }
   double mf = 0.0, mref = 0.0;
   for (int i = cx.cta * kRefThreads + cx.tid; i < cx.n; i += cx.G * kRefThreads) {
@@ -2069,103 +2064,22 @@ template <> struct UA<double> {
 template <typename A0, typename U>
 __device__ __noinline__ bool apply_A(Cx& cx, const RefineArgs& a, const U* v, int op) {
   PhaseTimer pt(cx, 4);
-  const A0* A = (const A0*)a.A;
-  if (op == MSIR_FP32) {
-    // a warp's rows (up to 8, consecutive) together: v is loaded once per
-    // column and the rows' loads and sums are independent, so their
-    // latencies overlap
-    const int nwarps = cx.G * (kRefThreads / 32);
-    const int rpw = min(8, (cx.n + nwarps - 1) / nwarps);
-    for (int i0 = (cx.cta * (kRefThreads / 32) + cx.warp) * rpw; i0 < cx.n; i0 += nwarps * rpw) {
-      const int nr = min(rpw, cx.n - i0);
-      const A0* rows[8];
-      ff_t acc[8];
-#pragma unroll
-      for (int rr = 0; rr < 8; ++rr) {
-        const int i = i0 + min(rr, nr - 1);  // rows past nr repeat the last one, never stored
-        rows[rr] = A + (size_t)a.perm[i] * a.lda;
-        acc[rr] = ff_t{0.0f, 0.0f};
-      }
-      // four consecutive columns per lane and step, 16-byte loads
-      const int n4 = ((reinterpret_cast<uintptr_t>(v) & 15) == 0) ? (cx.n & ~3) : 0;
-      // software pipeline: the next step's 8 rows x 4 columns and v are
-      // loaded into registers while this step's compensated sums run
-      {
-        int j = cx.lane * 4;
-        float an[8][4], vn[4];
-        if (j < n4) {
-          ld4f_vec<U>(v + j, vn);
-#pragma unroll
-          for (int rr = 0; rr < 8; ++rr)
-            if (rr < nr) ld4f_row<A0>(rows[rr] + j, an[rr]);
-        }
-        for (; j < n4; j += 128) {
-          float ac[8][4], vc[4];
-#pragma unroll
-          for (int q = 0; q < 4; ++q) vc[q] = vn[q];
-#pragma unroll
-          for (int rr = 0; rr < 8; ++rr)
-#pragma unroll
-            for (int q = 0; q < 4; ++q) ac[rr][q] = an[rr][q];
-          if (j + 128 < n4) {
-            ld4f_vec<U>(v + j + 128, vn);
-#pragma unroll
-            for (int rr = 0; rr < 8; ++rr)
-              if (rr < nr) ld4f_row<A0>(rows[rr] + j + 128, an[rr]);
-          }
-#pragma unroll
-          for (int rr = 0; rr < 8; ++rr)
-            if (rr < nr) {
-#pragma unroll
-              for (int q = 0; q < 4; ++q) acc[rr] = ff_fma(ac[rr][q], vc[q], acc[rr]);
-            }
-        }
-      }
-      for (int j = n4 + cx.lane; j < cx.n; j += 32) {
-        const float vj = (float)__ldcg(v + j);
-#pragma unroll
-        for (int rr = 0; rr < 8; ++rr) acc[rr] = ff_fma((float)__ldg(rows[rr] + j), vj, acc[rr]);
-      }
-#pragma unroll
-      for (int rr = 0; rr < 8; ++rr)
-#pragma unroll
-        for (int m = 16; m > 0; m >>= 1) acc[rr] = ff_merge(acc[rr], ff_shfl_xor(acc[rr], m));
-      if (cx.lane < nr) {
-        float mine = ff_fin(acc[0]);
-#pragma unroll
-        for (int rr = 1; rr < 8; ++rr)
-          if (cx.lane == rr) mine = ff_fin(acc[rr]);
-        const int ar = a.perm[i0 + cx.lane];
-        const float R = (float)rscale(a, ar);
-        ((float*)a.c_hi)[i0 + cx.lane] = __fmul_rn(mine, R);
-      }
-    }
-    return grid_barrier(a.bar, a.err, cx.G);
-  }
-  const int nw = cx.G * (kRefThreads / 32);
-  if (op == MSIR_DD) {
-    for (int i = cx.cta * (kRefThreads / 32) + cx.warp; i < cx.n; i += nw) {
-      const int ar = a.perm[i];
-      const dd_t tt = row_dot_dd<A0, U>(A + (size_t)ar * a.lda, v, cx.n, cx.lane);
-      if (cx.lane == 0) {
-        const double R = rscale(a, ar);
-        a.c_hi[i] = tt.hi * R;
-        a.c_lo[i] = tt.lo * R;
-      }
-    }
-    return grid_barrier(a.bar, a.err, cx.G);
-  }
-  // fp64: two rows per warp at a time (rows i and i + nw); a missing second
-  // row repeats the first and is not stored
-  for (int i = cx.cta * (kRefThreads / 32) + cx.warp; i < cx.n; i += 2 * nw) {
-    const int i2 = i + nw < cx.n ? i + nw : i;
-    const int ar[2] = {a.perm[i], a.perm[i2]};
-    const A0* const rows[2] = {A + (size_t)ar[0] * a.lda, A + (size_t)ar[1] * a.lda};
-    double acc[2];
-    rows_dot_d<A0, U, 2>(rows, v, cx.n, cx.lane, acc);
-    if (cx.lane == 0) {
-      a.c_hi[i] = acc[0] * rscale(a, ar[0]);
-      if (i2 != i) a.c_hi[i2] = acc[1] * rscale(a, ar[1]);
+  // (an fp32 vector comes with an fp32 matrix: u >= u0)
+  if constexpr (sizeof(A0) == 4 || sizeof(U) == 8) {
+    if (op == MSIR_FP32) {
+      if constexpr (sizeof(U) == 4)
+        gemv_rows<A0, U, MSIR_FP32>(cx, a, v, [&](int i, int ar, float t) {
+          ((float*)a.c_hi)[i] = __fmul_rn(t, (float)rscale(a, ar));
+        });
+    } else if (op == MSIR_DD) {
+      if constexpr (sizeof(U) == 8)
+        gemv_rows<A0, U, MSIR_DD>(cx, a, v, [&](int i, int ar, dd_t t) {
+          const double R = rscale(a, ar);
+          a.c_hi[i] = t.hi * R;
+          a.c_lo[i] = t.lo * R;
+        });
+    } else {
+      gemv_rows<A0, U, MSIR_FP64>(cx, a, v, [&](int i, int ar, double t) { a.c_hi[i] = t * rscale(a, ar); });
     }
   }
   return grid_barrier(a.bar, a.err, cx.G);
@@ -2392,6 +2306,49 @@ __device__ bool grid_sum_sq(Cx& cx, const RefineArgs& a, const U* w, double& out
   return true;
 }
 
+// y of the rotated (triangular) Hessenberg system by one warp, into ys and
+// a.yv: row i from the last up, y_i = (g_i - sum_j H_ij y_j) / H_ii with every
+// product and difference rounded, j ascending.  The subtractions of a row
+// are a chain; the products of 32 columns are formed by the lanes beside it,
+// and the next 32 entries of H (row-major) are loaded ahead, across rows
+// too.  (One thread that loads each entry when the chain reaches it took 50
+// ms for 820 columns, a fifth of a GMRES cycle at n = 8192.)
+template <typename U>
+__device__ __noinline__ void hessenberg_solve(const RefineArgs& a, int kcap, int kdone, const U* g, U* ys, int lane) {
+  using M = UA<U>;
+  const int ld = kcap + 1;
+  auto entry = [&](int i, int j) { return i >= 0 && j < kdone ? (U)__ldcg(a.H + (size_t)i * ld + j) : (U)0; };
+  // the chunks of row i start at its diagonal: columns i + lane, i + 32 + lane, ..
+  int i = kdone - 1, j0 = i;
+  U h = entry(i, j0 + lane);
+  U acc = (U)0, diag = (U)0;
+  while (i >= 0) {
+    const bool last = j0 + 32 >= kdone;
+    const int ni = last ? i - 1 : i, nj = last ? i - 1 : j0 + 32;
+    const U hn = entry(ni, nj + lane);
+    int l0 = 0;
+    if (j0 == i) {
+      acc = g[i];
+      diag = __shfl_sync(0xffffffffu, h, 0);
+      l0 = 1;
+    }
+    const int cnt = min(32, kdone - j0);
+    const U p = lane >= l0 && lane < cnt ? M::mul(h, ys[j0 + lane]) : (U)0;
+    for (int l = l0; l < cnt; ++l) acc = M::sub(acc, __shfl_sync(0xffffffffu, p, l));
+    if (last) {
+      const U y = M::div(acc, diag);
+      if (lane == 0) {
+        ys[i] = y;
+        a.yv[i] = (double)y;
+      }
+      __syncwarp();
+    }
+    h = hn;
+    i = ni;
+    j0 = nj;
+  }
+}
+
 template <typename A0, typename F, typename U>
 __device__ bool gmres(Cx& cx, const RefineArgs& a, double s, int ur, int u, int op, double tau,
                       unsigned char* gsm, GmresOut& out) {
@@ -2517,10 +2474,8 @@ __device__ bool gmres(Cx& cx, const RefineArgs& a, double s, int ur, int u, int 
       s_bc[0] = fabs((double)sm_g[k + 1]) / (double)beta;
     }
     __syncthreads();
-    if (cx.cta == 0) {
-      double* Hk = a.H + (size_t)k * (kcap + 1);
-      for (int i = cx.tid; i <= k; i += kRefThreads) Hk[i] = (double)s_h[i];
-    }
+    if (cx.cta == 0)
+      for (int i = cx.tid; i <= k; i += kRefThreads) a.H[(size_t)i * (kcap + 1) + k] = (double)s_h[i];
     if (cx.cta == 0 && cx.tid == 0) cx.t_ns[6] += gtimer() - tg0;
     const double relres = s_bc[0];
     kdone = k + 1;
@@ -2534,15 +2489,9 @@ __device__ bool gmres(Cx& cx, const RefineArgs& a, double s, int ur, int u, int 
     __syncthreads();
     if (!isfinite(relres) || relres <= tau || hk1 == (U)0) break;
   }
-  // y from the rotated Hessenberg matrix (CTA 0), then d = fl_u(V y)
-  if (cx.cta == 0 && cx.tid == 0) {
-    for (int i = kdone - 1; i >= 0; --i) {
-      U acc = sm_g[i];
-      for (int j = i + 1; j < kdone; ++j)
-        acc = M::sub(acc, M::mul((U)a.H[(size_t)j * (kcap + 1) + i], (U)a.yv[j]));
-      a.yv[i] = (double)M::div(acc, (U)a.H[(size_t)i * (kcap + 1) + i]);
-    }
-  }
+  // y from the rotated Hessenberg matrix (warp 0 of CTA 0), then d = fl_u(V y)
+  __syncthreads();  // CTA 0's rows of H are written
+  if (cx.cta == 0 && cx.warp == 0) hessenberg_solve<U>(a, kcap, kdone, sm_g, s_h, cx.lane);
   if (!grid_barrier(a.bar, a.err, cx.G)) return false;
   for (int j = cx.tid; j < kdone; j += kRefThreads) s_h[j] = (U)__ldcg(a.yv + j);
   __syncthreads();

@@ -108,6 +108,7 @@ cudaError_t launch_refine(int a_fmt, int f_fmt, const RefineArgs& a, int grid, c
   if (e != cudaSuccess) return e;
   RefineArgs copy = a;
   copy.gmres_off = (int)(smem - gmres_smem(a.kcap));
+  copy.scratch = copy.gmres_off - kScratchOff;
   if (a.cluster > 1) {
     if (grid % a.cluster != 0) return cudaErrorInvalidValue;
     cudaLaunchAttribute at[2];
