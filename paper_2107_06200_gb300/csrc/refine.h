@@ -71,7 +71,7 @@ constexpr int kRingDeep = 16, kRingFlat = 8;  // steps of the ring of factor val
 // the ring of factor values (16 bytes per thread and step).
 constexpr size_t wide_ring_off(int npad, int G, int vbytes) {
   const size_t rows = (size_t)(kSuper + G - 1) / G, passes = (rows + 3) / 4;  // at least 4 rows of a CTA at a time
-  return ((size_t)npad * vbytes + 2 * (size_t)kSuper * vbytes + 16 * 8 + passes * kRefThreads * 8 + 127) / 128 * 128;
+  return ((size_t)npad * vbytes + 2 * (size_t)kSuper * vbytes + (2 + passes) * kRefThreads * 8 + 127) / 128 * 128;
 }
 constexpr size_t wide_smem(int npad, int G, int vbytes, int ring) {
   return wide_ring_off(npad, G, vbytes) + (size_t)ring * kRefThreads * 16;

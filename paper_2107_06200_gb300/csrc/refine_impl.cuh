@@ -1537,7 +1537,6 @@ __device__ __forceinline__ bool wide_collect(const unsigned long long* p, int nv
   return true;
 }
 
-template <int N> struct Int { static constexpr int value = N; };
 
 // The factor values of one thread of a wide solve, in the order of their
 // use: near(1), far(2), near(2), far(3), ...  A segment is one row's steps
@@ -1610,6 +1609,121 @@ struct WideStream {
   }
 };
 
+// Interleaved sums of a thread: four in fp32 (the chain of a compensated sum
+// is long), one in fp64 (the narrow pipe serves the CTA's warps in turn).
+template <typename ACC> constexpr int kWideAcc = ACC::kW == 1 ? 4 : 1;
+template <typename ACC>
+__device__ __forceinline__ typename ACC::A wide_sum(const typename ACC::A (&acc)[4]) {
+  return ACC::merge(ACC::merge(acc[0], acc[1]), ACC::merge(acc[2], acc[3]));
+}
+template <typename ACC>
+__device__ __forceinline__ typename ACC::A wide_sum(const typename ACC::A (&acc)[1]) {
+  return acc[0];
+}
+
+// U steps of a wide solve's stream: the products of this thread's values with
+// the y at yp, yp + STEP, .., into interleaved sums.
+template <typename ACC, int U, typename F, bool LOWER, int WPR>
+__device__ __forceinline__ void wide_steps(WideStream<F, LOWER, WPR>& q, const typename ACC::V* yp, bool have,
+                                           typename ACC::A (&acc)[kWideAcc<ACC>]) {
+  using V = typename ACC::V;
+  using Lt = typename ACC::L;
+  using Q = WideStream<F, LOWER, WPR>;
+  constexpr int VC = Q::VC;
+  static_assert(U <= 4, "the ring holds depth copies");
+#pragma unroll
+  for (int h = 0; h < U; ++h) q.issue();
+  // depth - 4 + U copies are under way or waiting; the U oldest are due
+  if (q.depth == kRingDeep) cp_async_wait<kRingDeep - 4>();
+  else cp_async_wait<kRingFlat - 4>();
+  uint4 raw[U];
+#pragma unroll
+  for (int h = 0; h < U; ++h) raw[h] = q.take();
+  if (!have) return;
+#pragma unroll
+  for (int h = 0; h < U; ++h) {
+    F f[VC];
+    memcpy(f, &raw[h], 16);
+    V y[VC];
+    if constexpr (VC >= 4) {
+#pragma unroll
+      for (int e = 0; e < VC; e += 4) {
+        V y4[4];
+        lds4(yp + h * Q::STEP + e, y4);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) y[e + i] = y4[i];
+      }
+    } else {
+      y[0] = yp[h * Q::STEP];
+      y[1] = yp[h * Q::STEP + 1];
+    }
+    Lt l[VC];
+    if constexpr (sizeof(Lt) == 8 && sizeof(F) < 8) {
+      // widened by integer instructions (see gemv_rows_n)
+      bool sp = false;
+#pragma unroll
+      for (int e = 0; e < VC; ++e) {
+        const float v = (float)to_f(f[e]);
+        sp |= widen_special(v);
+        l[e] = widen_normal(v);
+      }
+      if (__any_sync(0xffffffffu, sp)) {
+#pragma unroll
+        for (int e = 0; e < VC; ++e) l[e] = (Lt)to_f(f[e]);
+      }
+    } else {
+#pragma unroll
+      for (int e = 0; e < VC; ++e) l[e] = (Lt)to_f(f[e]);
+    }
+#pragma unroll
+    for (int e = 0; e < VC; ++e) acc[e % kWideAcc<ACC>] = ACC::fma(l[e], y[e], acc[e % kWideAcc<ACC>]);
+  }
+}
+
+// Sum over the 32 WPR threads that share a row, for the CTA's 8 / WPR rows at
+// once.  fp32: the total is on lane 0 of the row's first warp.  fp64: an
+// addition by a whole warp holds the SM's pipe for 16 cycles, so the partial
+// sums go through shared memory and warp 0 adds them for all rows (4 WPR
+// lanes per row), instead of five additions on every warp; the total of row
+// r is on warp 0's lane 4 WPR r.  One block barrier (none for fp32 with one
+// warp per row); the buffers of successive calls alternate.
+template <typename ACC, int WPR>
+__device__ __forceinline__ typename ACC::A wide_total(typename ACC::A acc, typename ACC::A* part, int& pbuf, int tid,
+                                                      int lane, int warp) {
+  using A = typename ACC::A;
+  if constexpr (ACC::kW == 1) {
+#pragma unroll
+    for (int m = 16; m > 0; m >>= 1) acc = ACC::merge(acc, ACC::ax(acc, m));
+    if constexpr (WPR > 1) {
+      pbuf ^= 8;
+      if (warp % WPR > 0 && lane == 0) part[pbuf + warp] = acc;
+      __syncthreads();
+      if (warp % WPR == 0) {
+#pragma unroll
+        for (int h = 1; h < WPR; ++h) acc = ACC::merge(acc, part[pbuf + warp + h]);
+      }
+    }
+  } else {
+    pbuf ^= kRefThreads;
+    part[pbuf + tid] = acc;
+    __syncthreads();
+    if (warp == 0) {
+      constexpr int LPR = 4 * WPR, PER = 32 * WPR / LPR;  // lanes per row, partial sums per lane
+      const A* p = part + pbuf + (lane / LPR) * (32 * WPR) + lane % LPR;
+      A s0 = p[0], s1 = p[LPR];
+#pragma unroll
+      for (int h = 2; h < PER; h += 2) {
+        s0 = ACC::merge(s0, p[h * LPR]);
+        s1 = ACC::merge(s1, p[(h + 1) * LPR]);
+      }
+      acc = ACC::merge(s0, s1);
+#pragma unroll
+      for (int m = LPR / 2; m > 0; m >>= 1) acc = ACC::merge(acc, ACC::ax(acc, m));
+    }
+  }
+  return acc;
+}
+
 // One wide triangular solve (LOWER: L y = c; else U x = y).  WPR warps share
 // a row (columns split between them); a CTA takes rpc consecutive rows of
 // every superblock.  Not inlined (see trsv_team).
@@ -1641,6 +1755,7 @@ __device__ __noinline__ bool trsv_wide(Cx& cx, const RefineArgs& a, int store_fm
   constexpr int SPB = SB / STEP;                // steps per superblock
   static_assert(SPB * STEP == SB, "whole steps");
   constexpr bool kPair = sizeof(Z) > sizeof(S);
+  constexpr int kAcc = kWideAcc<ACC>;
   const int n = cx.n, NS = a.npad / SB;
   const int tri = LOWER ? 0 : 1;
   const int rpc = (SB + cx.G - 1) / cx.G;       // rows of each superblock per CTA
@@ -1648,8 +1763,8 @@ __device__ __noinline__ bool trsv_wide(Cx& cx, const RefineArgs& a, int store_fm
   V* ys = (V*)cx.tsm;                           // y, npad values
   S* zh = (S*)(ys + a.npad);                    // z of the superblock
   S* zl = zh + SB;                              // low words (fp32)
-  A* part = (A*)(zl + SB);                      // partial sums of the rows' other warps [2][8]
-  A* facc = part + 16;                          // far sums of the next superblock's rows [npass][256]
+  A* part = (A*)(zl + SB);                      // partial sums of the rows' other warps [2][8] (fp64: of every thread [2][256])
+  A* facc = part + (W == 1 ? 16 : 2 * kRefThreads);  // far sums of the next superblock's rows [npass][256]
   uint4* ring = (uint4*)(cx.tsm + a.ring_off);  // [a.ring][256]
   const size_t llblk = (size_t)kBlk * kLLWords;
   unsigned long long* wy = a.ll + (size_t)tri * cx.nblk * llblk;
@@ -1672,56 +1787,14 @@ __device__ __noinline__ bool trsv_wide(Cx& cx, const RefineArgs& a, int store_fm
 
   WideStream<F, LOWER, WPR> q;
   q.init(LU, a.ldf, n, NS, rpc, npass, r_lo, wp, wrow, cx.lane, cx.tid, ring, a.ring);
-  // U steps: the products of this thread's values with the y at yp, yp +
-  // STEP, .., into four interleaved sums (the chain of a compensated sum is
-  // long)
-  auto consume = [&](auto uc, const V* yp, bool have, A (&acc)[4]) {
-    constexpr int U = decltype(uc)::value;
-#pragma unroll
-    for (int h = 0; h < U; ++h) q.issue();
-    // depth - 4 + U copies are under way or waiting; the U oldest are due
-    static_assert(U <= 4, "the ring holds depth copies");
-    if (q.depth == kRingDeep) cp_async_wait<kRingDeep - 4>();
-    else cp_async_wait<kRingFlat - 4>();
-    uint4 raw[U];
-#pragma unroll
-    for (int h = 0; h < U; ++h) raw[h] = q.take();
-    if (have) {
-#pragma unroll
-      for (int h = 0; h < U; ++h) {
-        F f[VC];
-        memcpy(f, &raw[h], 16);
-        V y[VC];
-        if constexpr (VC >= 4) {
-#pragma unroll
-          for (int e = 0; e < VC; e += 4) lds4(yp + h * STEP + e, *(V(*)[4])(y + e));
-        } else {
-          y[0] = yp[h * STEP];
-          y[1] = yp[h * STEP + 1];
-        }
-#pragma unroll
-        for (int e = 0; e < VC; ++e) acc[e & 3] = ACC::fma((Lt)to_f(f[e]), y[e], acc[e & 3]);
-      }
-    }
-  };
-  auto sum4 = [&](A (&acc)[4]) { return ACC::merge(ACC::merge(acc[0], acc[1]), ACC::merge(acc[2], acc[3])); };
   int pbuf = 0;
-  // sum over the lanes of the warps that share a row; lane 0 of the row's
-  // first warp returns the total.  One block barrier if WPR > 1 (the partial
-  // sums alternate between two buffers).
-  auto row_total = [&](A acc) -> A {
-#pragma unroll
-    for (int m = 16; m > 0; m >>= 1) acc = ACC::merge(acc, ACC::ax(acc, m));
-    if constexpr (WPR > 1) {
-      pbuf ^= 8;
-      if (wp > 0 && cx.lane == 0) part[pbuf + cx.warp] = acc;
-      __syncthreads();
-      if (wp == 0) {
-#pragma unroll
-        for (int q = 1; q < WPR; ++q) acc = ACC::merge(acc, part[pbuf + cx.warp + q]);
-      }
-    }
-    return acc;
+  auto row_total = [&](A acc) -> A { return wide_total<ACC, WPR>(acc, part, pbuf, cx.tid, cx.lane, cx.warp); };
+  // the lane that holds a row's total, and which of the pass's rows (see wide_total)
+  const bool wr_lane = W == 1 ? (wp == 0 && cx.lane == 0) : (cx.warp == 0 && cx.lane % (32 / RG) == 0);
+  const int wr_row = W == 1 ? wrow : cx.lane / (32 / RG);
+  auto out_row = [&](int s, int ps) {  // the row this lane hands on, or -1
+    const int rr = r_lo + ps * RG + wr_row;
+    return wr_lane && rr < min(min(r_lo + rpc, SB), n - s * SB) ? rr : -1;
   };
 
   q.fill();
@@ -1765,16 +1838,20 @@ __device__ __noinline__ bool trsv_wide(Cx& cx, const RefineArgs& a, int store_fm
       fill_z();
       for (int ps = 0; ps < npass; ++ps) {
         const int rr = my_row(s, ps);
-        const V c_in = rr >= 0 ? ACC::load(in_hi, nullptr, R0 + rr) : ACC::zero();
-        A ac[4] = {t > 1 ? facc[ps * kRefThreads + cx.tid] : ACC::azero(), ACC::azero(), ACC::azero(), ACC::azero()};
+        const int ro = out_row(s, ps);
+        const V c_in = ro >= 0 ? ACC::load(in_hi, nullptr, R0 + ro) : ACC::zero();
+        A ac[kAcc];
 #pragma unroll
-        for (int k = 0; k < SPB; ++k) consume(Int<1>(), ys + u * SB + k * STEP + (wp * 32 + cx.lane) * VC, rr >= 0, ac);
-        const A acc = row_total(sum4(ac));
-        if (rr >= 0 && wp == 0 && cx.lane == 0) {
+        for (int e = 0; e < kAcc; ++e) ac[e] = ACC::azero();
+        if (t > 1) ac[0] = facc[ps * kRefThreads + cx.tid];
+#pragma unroll
+        for (int k = 0; k < SPB; ++k) wide_steps<ACC, 1>(q, ys + u * SB + k * STEP + (wp * 32 + cx.lane) * VC, rr >= 0, ac);
+        const A acc = row_total(wide_sum<ACC>(ac));
+        if (ro >= 0) {
           const Z z = WA::zdiff(c_in, acc);
 #pragma unroll
           for (int k = 0; k < ZW; ++k)
-            st_relaxed_u64(wz + (size_t)(R0 + rr) * ZW + k, ((unsigned long long)epoch << 32) | WA::zword(z, k));
+            st_relaxed_u64(wz + (size_t)(R0 + ro) * ZW + k, ((unsigned long long)epoch << 32) | WA::zword(z, k));
         }
       }
     }
@@ -1799,12 +1876,16 @@ __device__ __noinline__ bool trsv_wide(Cx& cx, const RefineArgs& a, int store_fm
     if (t > 0 && t + 1 < NS) {
       for (int ps = 0; ps < npass; ++ps) {
         const bool have = my_row(super(t + 1), ps) >= 0;
-        A ac[4] = {ACC::azero(), ACC::azero(), ACC::azero(), ACC::azero()};
+        A ac[kAcc];
+#pragma unroll
+        for (int e = 0; e < kAcc; ++e) ac[e] = ACC::azero();
         const V* yp = ys + (LOWER ? 0 : super(t - 1) * SB) + (wp * 32 + cx.lane) * VC;
         int k = 0;
-        for (; k + 4 <= t * SPB; k += 4, yp += 4 * STEP) consume(Int<4>(), yp, have, ac);
-        for (; k < t * SPB; ++k, yp += STEP) consume(Int<1>(), yp, have, ac);
-        facc[ps * kRefThreads + cx.tid] = sum4(ac);
+        // (U = 2 in fp64: more widened values would not fit in registers)
+        constexpr int U = W == 1 ? 4 : 2;
+        for (; k + U <= t * SPB; k += U, yp += U * STEP) wide_steps<ACC, U>(q, yp, have, ac);
+        for (; k < t * SPB; ++k, yp += STEP) wide_steps<ACC, 1>(q, yp, have, ac);
+        facc[ps * kRefThreads + cx.tid] = wide_sum<ACC>(ac);
       }
     }
     if (t > 0) {
@@ -1820,7 +1901,9 @@ __device__ __noinline__ bool trsv_wide(Cx& cx, const RefineArgs& a, int store_fm
     for (int ps = 0; ps < npass; ++ps) {
       const int rr = my_row(s, ps);
       if (ps > 0) load_inv(rr);
-      A ac[4] = {ACC::azero(), ACC::azero(), ACC::azero(), ACC::azero()};
+      A ac[kAcc];
+#pragma unroll
+      for (int e = 0; e < kAcc; ++e) ac[e] = ACC::azero();
 #pragma unroll
       for (int q = 0; q < kGrp; ++q) {
         const int c = (q * WPR + wp) * 128 + cx.lane * 4;
@@ -1834,17 +1917,18 @@ __device__ __noinline__ bool trsv_wide(Cx& cx, const RefineArgs& a, int store_fm
           // inside the triangle only (the rest of the array holds other data)
           const bool in = (LOWER ? c + e <= rr : c + e >= rr) && c + e < SBn;
           const S x = in ? xh[e] : (S)0;
-          if constexpr (kPair) ac[e] = ArFF::term(ArFF::V{x, in ? xl[e] : (S)0}, ArFF::V{h4[e], l4[e]}, ac[e]);
-          else ac[e] = __fma_rn(x, h4[e], ac[e]);
+          if constexpr (kPair) ac[e % kAcc] = ArFF::term(ArFF::V{x, in ? xl[e] : (S)0}, ArFF::V{h4[e], l4[e]}, ac[e % kAcc]);
+          else ac[e % kAcc] = __fma_rn(x, h4[e], ac[e % kAcc]);
         }
       }
-      const A acc = row_total(sum4(ac));
-      if (rr >= 0 && wp == 0 && cx.lane == 0) {
+      const A acc = row_total(wide_sum<ACC>(ac));
+      const int ro = out_row(s, ps);
+      if (ro >= 0) {
         const V y = ACC::store(ACC::fin(acc), store_fmt);
 #pragma unroll
         for (int k = 0; k < W; ++k)
-          st_relaxed_u64(wy + (size_t)(R0 + rr) * W + k, ((unsigned long long)epoch << 32) | ACC::word(y, k));
-        ACC::save(out_hi, nullptr, R0 + rr, y);
+          st_relaxed_u64(wy + (size_t)(R0 + ro) * W + k, ((unsigned long long)epoch << 32) | ACC::word(y, k));
+        ACC::save(out_hi, nullptr, R0 + ro, y);
       }
     }
   }
