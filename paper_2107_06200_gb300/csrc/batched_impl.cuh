@@ -254,6 +254,7 @@ __global__ void __launch_bounds__(kBatchThreads, 1) batched_solve_kernel(BatchAr
     cx.nblk = (n + kBlk - 1) / kBlk;
     cx.team_k = 0;
     cx.redbuf = 0;
+    cx.nbar = 0;
     cx.t_ns = S.t_ns;
     // ---- factor, refine, escalate
     int fmt = T.uf, status = MSIR_OK, nfact = 0, scaled = 0, lu_info = 0, nb_used = 0, nbo_used = 0;

@@ -225,11 +225,6 @@ __device__ __forceinline__ unsigned ld_acquire_u32(const unsigned* p) {
 __device__ __forceinline__ void st_release_u32(unsigned* p, unsigned v) {
   asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
-__device__ __forceinline__ unsigned atom_add_release_u32(unsigned* p, unsigned v) {
-  unsigned old;
-  asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(v) : "memory");
-  return old;
-}
 __device__ __forceinline__ int ld_volatile_i32(const int* p) {
   return *(const volatile int*)p;
 }
@@ -252,26 +247,27 @@ __device__ __forceinline__ void record_timeout(int* err, int site, int v0, int v
   }
 }
 
-// Grid-wide barrier for a cooperative launch of G blocks.  `count` grows by
-// G per episode and is zeroed by the host before the launch.  Returns false
-// (after recording the error) on timeout or if another block failed.
-__device__ __forceinline__ bool grid_barrier_for(unsigned* count, int* err, unsigned G,
-                                                 unsigned long long limit_ns) {
+// Grid-wide barrier of a cooperative launch: every block adds 1 to `count`
+// and waits until it reaches `target` (the number of blocks times the
+// barriers so far; count is zeroed by the host before the launch).  The
+// addition is a release without a result, so nothing waits for its round
+// trip to L2 before the polling starts.  Returns false (after recording the
+// error) on timeout or if another block failed.
+static __device__ __noinline__ bool grid_barrier_for(unsigned* count, int* err, unsigned target,
+                                                     unsigned long long limit_ns) {
   __shared__ int s_ok;
   __syncthreads();
   if (threadIdx.x == 0) {
     int ok = 1;
-    __threadfence();
-    unsigned old = atom_add_release_u32(count, 1u);
-    unsigned target = (old / G + 1u) * G;
-    unsigned long long t0 = gtimer();
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(count) : "memory");
+    unsigned long long t0 = 0;
     unsigned spins = 0;
     while ((int)(ld_acquire_u32(count) - target) < 0) {
-      __nanosleep(20);
-      if ((++spins & 63u) == 0u) {
+      if ((++spins & 255u) == 0u) {
+        if (t0 == 0) t0 = gtimer();
         if (ld_volatile_i32(err) != 0) { ok = 0; break; }
         if (gtimer() - t0 > limit_ns) {
-          record_timeout(err, 1, (int)ld_acquire_u32(count), (int)target, (int)G);
+          record_timeout(err, 1, (int)ld_acquire_u32(count), (int)target, 0);
           ok = 0;
           break;
         }
@@ -281,9 +277,6 @@ __device__ __forceinline__ bool grid_barrier_for(unsigned* count, int* err, unsi
   }
   __syncthreads();
   return s_ok != 0;
-}
-__device__ __forceinline__ bool grid_barrier(unsigned* count, int* err, unsigned G) {
-  return grid_barrier_for(count, err, G, kWaitTimeoutNs);
 }
 
 __device__ __forceinline__ unsigned ld_relaxed_u32(const unsigned* p) {

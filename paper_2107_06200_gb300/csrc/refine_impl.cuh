@@ -36,6 +36,7 @@ struct Cx {
   int G, cta, tid, lane, warp, n, nblk;
   int team_k;  // RefineArgs::team_k
   unsigned epoch;
+  unsigned nbar;             // arrivals that complete the latest grid barrier
   int redbuf;
   unsigned long long* t_ns;  // per-phase timers (CTA 0, thread 0), shared memory
   unsigned char* tsm;        // shared scratch of the substitutions (kTrsvSmem bytes)
@@ -44,6 +45,18 @@ struct Cx {
   int C;                     // CTAs per cluster (1: no clusters)
   unsigned long long* inbox; // [kMaxCluster][kBlk][kLLWords] words written by cluster peers
 };
+
+// Barrier of the solve's grid (a block barrier when one block is the grid:
+// nothing else reads its data, and data written during the kernel is never
+// read through the non-coherent path).
+static __device__ __forceinline__ bool grid_barrier(Cx& cx, const RefineArgs& a) {
+  if (cx.G == 1) {
+    __syncthreads();
+    return true;
+  }
+  cx.nbar += cx.G;
+  return grid_barrier_for(a.bar, a.err, cx.nbar, kWaitTimeoutNs);
+}
 
 // Phase timer: CTA 0 / thread 0 accumulates %globaltimer deltas.
 struct PhaseTimer {
@@ -284,7 +297,7 @@ __device__ bool grid_reduce(Cx& cx, const RefineArgs& a, double (&v)[NV], const 
   cx.redbuf ^= 1;
   if (cx.tid == 0)
     for (int i = 0; i < NV; ++i) buf[cx.cta * kRedW + i] = v[i];
-  if (!grid_barrier(a.bar, a.err, cx.G)) return false;
+  if (!grid_barrier(cx, a)) return false;
   if (cx.warp == 0) {
     for (int i = 0; i < NV; ++i) {
       double acc = op[i] ? 0.0 : 0.0;
@@ -352,7 +365,7 @@ template <int N> struct SegLd<float, N> {
   static __device__ __forceinline__ void ld(const float* p, Lt (&v)[N]) {
 #pragma unroll
     for (int m = 0; m < N / 4; ++m) {
-      const float4 f = __ldg((const float4*)p + m);
+      const float4 f = __ldcg((const float4*)p + m);
       v[4 * m] = (Lt)f.x; v[4 * m + 1] = (Lt)f.y; v[4 * m + 2] = (Lt)f.z; v[4 * m + 3] = (Lt)f.w;
     }
   }
@@ -362,7 +375,7 @@ template <int N> struct SegLd<double, N> {
   static __device__ __forceinline__ void ld(const double* p, Lt (&v)[N]) {
 #pragma unroll
     for (int m = 0; m < N / 2; ++m) {
-      const double2 f = __ldg((const double2*)p + m);
+      const double2 f = __ldcg((const double2*)p + m);
       v[2 * m] = (Lt)f.x; v[2 * m + 1] = (Lt)f.y;
     }
   }
@@ -376,11 +389,11 @@ template <typename H, int N> struct SegLdH {
     if (N >= 8) {
 #pragma unroll
       for (int m = 0; m < N / 8; ++m) {
-        const uint4 u = __ldg((const uint4*)p + m);
+        const uint4 u = __ldcg((const uint4*)p + m);
         w[4 * m] = u.x; w[4 * m + 1] = u.y; w[4 * m + 2] = u.z; w[4 * m + 3] = u.w;
       }
     } else {
-      const uint2 u = __ldg((const uint2*)p);
+      const uint2 u = __ldcg((const uint2*)p);
       w[0] = u.x; w[1] = u.y;
     }
 #pragma unroll
@@ -826,7 +839,7 @@ __device__ __noinline__ bool build_inverses(Cx& cx, const RefineArgs& a, bool dd
       }
     }
   }
-  return grid_barrier(a.bar, a.err, cx.G);
+  return grid_barrier(cx, a);
 }
 
 // Scaled off-diagonal blocks M_bj = D_b^{-1} F_bj (j != b; L below the
@@ -896,7 +909,7 @@ __device__ __noinline__ bool build_scaled32(Cx& cx, const RefineArgs& a) {
       }
     }
   }
-  return grid_barrier(a.bar, a.err, cx.G);
+  return grid_barrier(cx, a);
 }
 
 // fp64 and dd (and fp32 with fp64 factors): the inverse of the diagonal block
@@ -976,7 +989,7 @@ __device__ __noinline__ bool build_scaled(Cx& cx, const RefineArgs& a, bool dd) 
       }
     }
   }
-  return grid_barrier(a.bar, a.err, cx.G);
+  return grid_barrier(cx, a);
 }
 
 // Depth of the ring of scaled-block tiles that fp32 / fp64 substitutions
@@ -1480,7 +1493,7 @@ __device__ __noinline__ bool build_wide(Cx& cx, const RefineArgs& a) {
           }
         }
       }
-      if (!grid_barrier(a.bar, a.err, cx.G)) return false;
+      if (!grid_barrier(cx, a)) return false;
     }
   }
   return true;
@@ -1621,15 +1634,12 @@ __device__ __forceinline__ typename ACC::A wide_sum(const typename ACC::A (&acc)
   return acc[0];
 }
 
-// U steps of a wide solve's stream: the products of this thread's values with
-// the y at yp, yp + STEP, .., into interleaved sums.
+// The next U steps of a wide solve's stream, in the solve's precision.
 template <typename ACC, int U, typename F, bool LOWER, int WPR>
-__device__ __forceinline__ void wide_steps(WideStream<F, LOWER, WPR>& q, const typename ACC::V* yp, bool have,
-                                           typename ACC::A (&acc)[kWideAcc<ACC>]) {
-  using V = typename ACC::V;
+__device__ __forceinline__ void wide_fetch(WideStream<F, LOWER, WPR>& q,
+                                           typename ACC::L (&l)[U][WideStream<F, LOWER, WPR>::VC]) {
   using Lt = typename ACC::L;
-  using Q = WideStream<F, LOWER, WPR>;
-  constexpr int VC = Q::VC;
+  constexpr int VC = WideStream<F, LOWER, WPR>::VC;
   static_assert(U <= 4, "the ring holds depth copies");
 #pragma unroll
   for (int h = 0; h < U; ++h) q.issue();
@@ -1639,25 +1649,10 @@ __device__ __forceinline__ void wide_steps(WideStream<F, LOWER, WPR>& q, const t
   uint4 raw[U];
 #pragma unroll
   for (int h = 0; h < U; ++h) raw[h] = q.take();
-  if (!have) return;
 #pragma unroll
   for (int h = 0; h < U; ++h) {
     F f[VC];
     memcpy(f, &raw[h], 16);
-    V y[VC];
-    if constexpr (VC >= 4) {
-#pragma unroll
-      for (int e = 0; e < VC; e += 4) {
-        V y4[4];
-        lds4(yp + h * Q::STEP + e, y4);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) y[e + i] = y4[i];
-      }
-    } else {
-      y[0] = yp[h * Q::STEP];
-      y[1] = yp[h * Q::STEP + 1];
-    }
-    Lt l[VC];
     if constexpr (sizeof(Lt) == 8 && sizeof(F) < 8) {
       // widened by integer instructions (see gemv_rows_n)
       bool sp = false;
@@ -1665,18 +1660,40 @@ __device__ __forceinline__ void wide_steps(WideStream<F, LOWER, WPR>& q, const t
       for (int e = 0; e < VC; ++e) {
         const float v = (float)to_f(f[e]);
         sp |= widen_special(v);
-        l[e] = widen_normal(v);
+        l[h][e] = widen_normal(v);
       }
       if (__any_sync(0xffffffffu, sp)) {
 #pragma unroll
-        for (int e = 0; e < VC; ++e) l[e] = (Lt)to_f(f[e]);
+        for (int e = 0; e < VC; ++e) l[h][e] = (Lt)to_f(f[e]);
       }
     } else {
 #pragma unroll
-      for (int e = 0; e < VC; ++e) l[e] = (Lt)to_f(f[e]);
+      for (int e = 0; e < VC; ++e) l[h][e] = (Lt)to_f(f[e]);
+    }
+  }
+}
+// Their products with the y at yp, yp + STEP, .., into interleaved sums.
+template <typename ACC, int U, int VC, int STEP>
+__device__ __forceinline__ void wide_apply(const typename ACC::L (&l)[U][VC], const typename ACC::V* yp,
+                                           typename ACC::A (&acc)[kWideAcc<ACC>]) {
+  using V = typename ACC::V;
+#pragma unroll
+  for (int h = 0; h < U; ++h) {
+    V y[VC];
+    if constexpr (VC >= 4) {
+#pragma unroll
+      for (int e = 0; e < VC; e += 4) {
+        V y4[4];
+        lds4(yp + h * STEP + e, y4);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) y[e + i] = y4[i];
+      }
+    } else {
+      y[0] = yp[h * STEP];
+      y[1] = yp[h * STEP + 1];
     }
 #pragma unroll
-    for (int e = 0; e < VC; ++e) acc[e % kWideAcc<ACC>] = ACC::fma(l[e], y[e], acc[e % kWideAcc<ACC>]);
+    for (int e = 0; e < VC; ++e) acc[e % kWideAcc<ACC>] = ACC::fma(l[h][e], y[e], acc[e % kWideAcc<ACC>]);
   }
 }
 
@@ -1831,21 +1848,29 @@ __device__ __noinline__ bool trsv_wide(Cx& cx, const RefineArgs& a, int store_fm
       if (__syncthreads_or(!ok)) return false;
     } else {
       const int u = super(t - 1), N0 = u * SB, Nn = min(SB, n - N0);
+      constexpr int PG = SPB < 4 ? SPB : 4;
+      Lt ln[PG][VC];
+      wide_fetch<ACC, PG>(q, ln);  // ahead of y
       const bool ok = wide_collect<W>(wy + (size_t)N0 * W, Nn, epoch, cx.tid, a.err, where,
                                       [&](int i, const unsigned* w) { ys[N0 + i] = ACC::unword(w); });
       for (int i = N0 + Nn + cx.tid; i < N0 + SB; i += kRefThreads) ys[i] = ACC::zero();
       if (__syncthreads_or(!ok)) return false;
       fill_z();
       for (int ps = 0; ps < npass; ++ps) {
-        const int rr = my_row(s, ps);
+        if (ps > 0) wide_fetch<ACC, PG>(q, ln);
         const int ro = out_row(s, ps);
         const V c_in = ro >= 0 ? ACC::load(in_hi, nullptr, R0 + ro) : ACC::zero();
         A ac[kAcc];
 #pragma unroll
         for (int e = 0; e < kAcc; ++e) ac[e] = ACC::azero();
         if (t > 1) ac[0] = facc[ps * kRefThreads + cx.tid];
+        const V* yp = ys + u * SB + (wp * 32 + cx.lane) * VC;
+        wide_apply<ACC, PG, VC, STEP>(ln, yp, ac);
 #pragma unroll
-        for (int k = 0; k < SPB; ++k) wide_steps<ACC, 1>(q, ys + u * SB + k * STEP + (wp * 32 + cx.lane) * VC, rr >= 0, ac);
+        for (int g = PG; g < SPB; g += PG) {
+          wide_fetch<ACC, PG>(q, ln);
+          wide_apply<ACC, PG, VC, STEP>(ln, yp + g * STEP, ac);
+        }
         const A acc = row_total(wide_sum<ACC>(ac));
         if (ro >= 0) {
           const Z z = WA::zdiff(c_in, acc);
@@ -1883,8 +1908,16 @@ __device__ __noinline__ bool trsv_wide(Cx& cx, const RefineArgs& a, int store_fm
         int k = 0;
         // (U = 2 in fp64: more widened values would not fit in registers)
         constexpr int U = W == 1 ? 4 : 2;
-        for (; k + U <= t * SPB; k += U, yp += U * STEP) wide_steps<ACC, U>(q, yp, have, ac);
-        for (; k < t * SPB; ++k, yp += STEP) wide_steps<ACC, 1>(q, yp, have, ac);
+        for (; k + U <= t * SPB; k += U, yp += U * STEP) {
+          Lt l[U][VC];
+          wide_fetch<ACC, U>(q, l);
+          if (have) wide_apply<ACC, U, VC, STEP>(l, yp, ac);
+        }
+        for (; k < t * SPB; ++k, yp += STEP) {
+          Lt l[1][VC];
+          wide_fetch<ACC, 1>(q, l);
+          if (have) wide_apply<ACC, 1, VC, STEP>(l, yp, ac);
+        }
         facc[ps * kRefThreads + cx.tid] = wide_sum<ACC>(ac);
       }
     }
@@ -1969,14 +2002,14 @@ __device__ bool msolve(Cx& cx, const RefineArgs& a, int store_fmt, bool synced) 
         if (!build_wide<F, k32>(cx, a)) return false;
         cx.mready |= need;
       }
-      if (!synced && !grid_barrier(a.bar, a.err, cx.G)) return false;
+      if (!synced && !grid_barrier(cx, a)) return false;
       {
         PhaseTimer pt(cx, 1);
         if (!trsv_wide_any<F, ACC, true>(cx, a, store_fmt)) return false;
       }
       PhaseTimer pt(cx, 2);
       if (!trsv_wide_any<F, ACC, false>(cx, a, store_fmt)) return false;
-      return synced || grid_barrier(a.bar, a.err, cx.G);
+      return synced || grid_barrier(cx, a);
     }
   }
   // inverses and scaled blocks of the current factors in this precision, once
@@ -1996,14 +2029,14 @@ __device__ bool msolve(Cx& cx, const RefineArgs& a, int store_fmt, bool synced) 
   // team of K > 1 CTAs spreads them over other CTAs, so c must be visible
   // grid-wide before the forward solve and z after the backward solve.
   const bool team = !synced && team_size<ACC>(cx) > 1;
-  if (team && !grid_barrier(a.bar, a.err, cx.G)) return false;
+  if (team && !grid_barrier(cx, a)) return false;
   {
     PhaseTimer pt(cx, 1);
     if (!trsv<F, ACC, true>(cx, a, store_fmt)) return false;
   }
   PhaseTimer pt(cx, 2);
   if (!trsv<F, ACC, false>(cx, a, store_fmt)) return false;
-  return !team || grid_barrier(a.bar, a.err, cx.G);
+  return !team || grid_barrier(cx, a);
 }
 
 template <typename F>
@@ -2166,7 +2199,7 @@ __device__ __noinline__ bool apply_A(Cx& cx, const RefineArgs& a, const U* v, in
       gemv_rows<A0, U, MSIR_FP64>(cx, a, v, [&](int i, int ar, double t) { a.c_hi[i] = t * rscale(a, ar); });
     }
   }
-  return grid_barrier(a.bar, a.err, cx.G);
+  return grid_barrier(cx, a);
 }
 
 // GMRES's vector work (Gram-Schmidt, norms, basis updates) uses a flat
@@ -2184,7 +2217,7 @@ __device__ __forceinline__ void flat_rows(const Cx& cx, int& r0, int& r1) {
 // are visible grid-wide)
 template <typename U>
 __device__ bool finish_solve(Cx& cx, const RefineArgs& a, U* out, int arith) {
-  if (!grid_barrier(a.bar, a.err, cx.G)) return false;
+  if (!grid_barrier(cx, a)) return false;
   int r0, r1;
   flat_rows(cx, r0, r1);
   for (int i = r0 + cx.tid; i < r1; i += kRefThreads) out[i] = UA<U>::rnd(get_z(a, arith, i) * cscale(a, i));
@@ -2197,14 +2230,14 @@ __device__ bool finish_solve(Cx& cx, const RefineArgs& a, U* out, int arith) {
 template <typename U>
 __device__ bool cgs_reduce(Cx& cx, const RefineArgs& a, int kp1, U* s_h) {
   PhaseTimer pt(cx, 3);
-  if (!grid_barrier(a.bar, a.err, cx.G)) return false;
+  if (!grid_barrier(cx, a)) return false;
   for (int j = cx.cta * 8 + cx.warp; j < kp1; j += cx.G * 8) {
     double acc = 0.0;
     for (int c = cx.lane; c < cx.G; c += 32) acc = __dadd_rn(acc, __ldcg(a.hred + (size_t)c * (a.kcap + 1) + j));
     acc = warp_sum_d(acc);
     if (cx.lane == 0) a.hvec[j] = (double)UA<U>::rnd(acc);
   }
-  if (!grid_barrier(a.bar, a.err, cx.G)) return false;
+  if (!grid_barrier(cx, a)) return false;
   for (int j = cx.tid; j < kp1; j += kRefThreads) s_h[j] = (U)__ldcg(a.hvec + j);
   __syncthreads();
   return true;
@@ -2282,11 +2315,10 @@ __device__ __noinline__ void cgs_partials(Cx& cx, const RefineArgs& a, const U* 
 // independent, so their latencies overlap.  Lane q < kRows returns row
 // i0+q's sum as a compensated pair (u = fp32: Dot2 in fp32, the pair's sum
 // is the value; u = fp64: an fp64 sum in .s, .c = 0).
-constexpr int kRows = 8;
 struct RowSum {
   double s, c;
 };
-template <typename U>
+template <typename U, int kRows>
 __device__ __forceinline__ RowSum basis_rows_dot(const RefineArgs& a, const U* V, int i0, int r1, int kp1,
                                                  const U* c, int lane) {
   constexpr int kVec = 16 / (int)sizeof(U);
@@ -2340,38 +2372,45 @@ __device__ __forceinline__ RowSum basis_rows_dot(const RefineArgs& a, const U* V
   return mine;
 }
 
+// rows per warp: the CTA's rows over its 8 warps
+template <typename U, typename Epi>
+__device__ __forceinline__ void basis_rows(const Cx& cx, const RefineArgs& a, const U* V, int kp1, const U* c, Epi epi) {
+  int r0, r1;
+  flat_rows(cx, r0, r1);
+  auto run = [&](auto rows) {
+    constexpr int kRows = decltype(rows)::value;
+    for (int i0 = r0 + cx.warp * kRows; i0 < r1; i0 += (kRefThreads / 32) * kRows) {
+      const RowSum acc = basis_rows_dot<U, kRows>(a, V, i0, r1, kp1, c, cx.lane);
+      const int i = i0 + cx.lane;
+      if (cx.lane < kRows && i < r1) epi(i, acc);
+    }
+  };
+  const int per = (r1 - r0 + kRefThreads / 32 - 1) / (kRefThreads / 32);
+  if (per <= 2) run(std::integral_constant<int, 2>());
+  else if (per <= 4) run(std::integral_constant<int, 4>());
+  else run(std::integral_constant<int, 8>());
+}
+
 // w_i = fl_u(w_i - sum_j V_j[i] h_j) with the difference taken from the
-// accurate sum (fp32: w - (s + c) by ff_sub_from); flat rows, kRows rows
-// per warp at a time
+// accurate sum (fp32: w - (s + c) by ff_sub_from); flat rows
 template <typename U>
 __device__ __noinline__ void cgs_update(Cx& cx, const RefineArgs& a, const U* V, U* w, int kp1, const U* s_h) {
   PhaseTimer pt(cx, 3);
-  int r0, r1;
-  flat_rows(cx, r0, r1);
-  for (int i0 = r0 + cx.warp * kRows; i0 < r1; i0 += (kRefThreads / 32) * kRows) {
-    const RowSum acc = basis_rows_dot<U>(a, V, i0, r1, kp1, s_h, cx.lane);
-    const int i = i0 + cx.lane;
-    if (cx.lane < kRows && i < r1) {
-      if constexpr (sizeof(U) == 4)
-        w[i] = ff_sub_from(w[i], ff_t{(float)acc.s, (float)acc.c});
-      else
-        w[i] = UA<U>::rnd(__dsub_rn((double)w[i], acc.s));
-    }
-  }
+  basis_rows<U>(cx, a, V, kp1, s_h, [&](int i, RowSum acc) {
+    if constexpr (sizeof(U) == 4)
+      w[i] = ff_sub_from(w[i], ff_t{(float)acc.s, (float)acc.c});
+    else
+      w[i] = UA<U>::rnd(__dsub_rn((double)w[i], acc.s));
+  });
   __syncthreads();
 }
 
 // d_i = fl_u(sum_j V_j[i] y_j) over the flat rows (the GMRES correction)
 template <typename U>
 __device__ __noinline__ void basis_combine(Cx& cx, const RefineArgs& a, const U* V, int kdone, const U* y) {
-  int f0, f1;
-  flat_rows(cx, f0, f1);
-  for (int i0 = f0 + cx.warp * kRows; i0 < f1; i0 += (kRefThreads / 32) * kRows) {
-    const RowSum acc = basis_rows_dot<U>(a, V, i0, f1, kdone, y, cx.lane);
-    const int i = i0 + cx.lane;
-    if (cx.lane < kRows && i < f1)
-      a.d[i] = sizeof(U) == 4 ? (double)ff_fin(ff_t{(float)acc.s, (float)acc.c}) : (double)UA<U>::rnd(acc.s);
-  }
+  basis_rows<U>(cx, a, V, kdone, y, [&](int i, RowSum acc) {
+    a.d[i] = sizeof(U) == 4 ? (double)ff_fin(ff_t{(float)acc.s, (float)acc.c}) : (double)UA<U>::rnd(acc.s);
+  });
 }
 
 template <typename U>
@@ -2463,7 +2502,7 @@ __device__ bool gmres(Cx& cx, const RefineArgs& a, double s, int ur, int u, int 
   flat_rows(cx, f0, f1);
   if (beta == (U)0) {
     for (int i = f0 + cx.tid; i < f1; i += kRefThreads) a.d[i] = 0.0;
-    return grid_barrier(a.bar, a.err, cx.G);  // d is read by the block partition
+    return grid_barrier(cx, a);  // d is read by the block partition
   }
   for (int i = f0 + cx.tid; i < f1; i += kRefThreads) {
     const U v = M::div(w[i], beta);
@@ -2475,7 +2514,7 @@ __device__ bool gmres(Cx& cx, const RefineArgs& a, double s, int ur, int u, int 
   int kdone = 0;
   for (int k = 0; k < kcap; ++k) {
     // full V_k needed by the matrix-vector product
-    if (!grid_barrier(a.bar, a.err, cx.G)) return false;
+    if (!grid_barrier(cx, a)) return false;
     if (!apply_A<A0, U>(cx, a, vk, op)) return false;
     if (!msolve_arith<F>(cx, a, op, op, true)) return false;
     if (!finish_solve<U>(cx, a, w, op)) return false;
@@ -2495,47 +2534,42 @@ __device__ bool gmres(Cx& cx, const RefineArgs& a, double s, int ur, int u, int 
     const U hk1 = M::sqrt_(M::rnd(ww));
     // Givens rotations (every CTA computes the same numbers)
     unsigned long long tg0 = (cx.cta == 0 && cx.tid == 0) ? gtimer() : 0;
-    // the entry carried from one rotation to the next stays in a register
+    // The rotations are a chain from entry to entry: carry = -sn carry + cs x.
+    // The products cs x and sn x do not depend on it and are formed by all
+    // threads first (into the upper half of s_h, and in x's place), so the
+    // chain is one multiplication and one addition per rotation (an fp64
+    // operation takes about 130 cycles on GB300), its operands loaded four
+    // rotations ahead.
+    for (int i = cx.tid; i < k; i += kRefThreads) {
+      const U x = s_h[i + 1];
+      s_h[kcap + 1 + i] = M::mul(sm_cs[i], x);
+      s_h[i + 1] = M::mul(sm_sn[i], x);
+    }
+    __syncthreads();
     U carry = (U)0;
-    if constexpr (sizeof(U) == 8) {
-      // fp64: the four products of a rotation on lanes 0-3 of warp 0 (lane
-      // q: cs x0, sn x1, -sn x0, cs x1), then lanes 0 and 2 add their pairs:
-      // two fp64 instructions on the chain per rotation instead of six
-      if (cx.warp == 0) {
-        const int q = cx.lane & 3;
-        carry = s_h[0];
-        for (int i = 0; i < k; ++i) {
-          const U cs = sm_cs[i], sn = sm_sn[i], x1 = s_h[i + 1];
-          const U ml = q == 1 ? sn : (q == 2 ? -sn : cs);
-          const U p = M::mul(ml, (q & 1) ? x1 : carry);
-          const U t = M::add(p, __shfl_down_sync(0xffffffffu, p, 1));
-          if (cx.lane == 0) s_h[i] = t;
-          carry = __shfl_sync(0xffffffffu, t, 2);
-        }
-      }
-    } else if (cx.tid == 0) {
-      // the operands of four rotations are loaded ahead of their use
+    if (cx.tid == 0) {
       carry = s_h[0];
       int i = 0;
       for (; i + 4 <= k; i += 4) {
-        U cs[4], sn[4], x1[4];
+        U cs[4], sn[4], p1[4], p2[4];
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
           cs[q] = sm_cs[i + q];
           sn[q] = sm_sn[i + q];
-          x1[q] = s_h[i + q + 1];
+          p1[q] = s_h[kcap + 1 + i + q];
+          p2[q] = s_h[i + q + 1];
         }
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
           const U x0 = carry;
-          s_h[i + q] = M::add(M::mul(cs[q], x0), M::mul(sn[q], x1[q]));
-          carry = M::add(M::mul(-sn[q], x0), M::mul(cs[q], x1[q]));
+          carry = M::add(M::mul(-sn[q], x0), p1[q]);
+          s_h[i + q] = M::add(M::mul(cs[q], x0), p2[q]);
         }
       }
       for (; i < k; ++i) {
-        const U x0 = carry, x1 = s_h[i + 1];
-        s_h[i] = M::add(M::mul(sm_cs[i], x0), M::mul(sm_sn[i], x1));
-        carry = M::add(M::mul(-sm_sn[i], x0), M::mul(sm_cs[i], x1));
+        const U x0 = carry, p2 = s_h[i + 1];
+        carry = M::add(M::mul(-sm_sn[i], x0), s_h[kcap + 1 + i]);
+        s_h[i] = M::add(M::mul(sm_cs[i], x0), p2);
       }
     }
     if (cx.tid == 0) {
@@ -2576,12 +2610,12 @@ __device__ bool gmres(Cx& cx, const RefineArgs& a, double s, int ur, int u, int 
   // y from the rotated Hessenberg matrix (warp 0 of CTA 0), then d = fl_u(V y)
   __syncthreads();  // CTA 0's rows of H are written
   if (cx.cta == 0 && cx.warp == 0) hessenberg_solve<U>(a, kcap, kdone, sm_g, s_h, cx.lane);
-  if (!grid_barrier(a.bar, a.err, cx.G)) return false;
+  if (!grid_barrier(cx, a)) return false;
   for (int j = cx.tid; j < kdone; j += kRefThreads) s_h[j] = (U)__ldcg(a.yv + j);
   __syncthreads();
   basis_combine<U>(cx, a, V, kdone, s_h);
   out.k = kdone;
-  return grid_barrier(a.bar, a.err, cx.G);  // d is read by the block partition
+  return grid_barrier(cx, a);  // d is read by the block partition
 }
 
 // -------------------------------------------------------------- kernel
@@ -2681,7 +2715,7 @@ __device__ __forceinline__ bool refine_msir(Cx& cx, const RefineArgs& a, RefStat
         a.xbest[i] = a.x0[i];
       }
     }
-    if (!(ok = grid_barrier(a.bar, a.err, cx.G))) return false;
+    if (!(ok = grid_barrier(cx, a))) return false;
     if (!(ok = residual<A0>(cx, a, a.x, S.ur, s, xnorm))) return false;
     nbe = s / (a.normA * xnorm + a.normb);
     if (cx.tid == 0) {
@@ -2695,7 +2729,7 @@ __device__ __forceinline__ bool refine_msir(Cx& cx, const RefineArgs& a, RefStat
     }
     __syncthreads();
   } else if (S.phase == PH_ESCALATED) {
-    if (!(ok = grid_barrier(a.bar, a.err, cx.G))) return false;
+    if (!(ok = grid_barrier(cx, a))) return false;
     if (!(ok = residual<A0>(cx, a, a.x, S.ur, s, xnorm))) return false;
     nbe = s / (a.normA * xnorm + a.normb);
     if (cx.tid == 0) {
@@ -2782,7 +2816,7 @@ __device__ __forceinline__ bool refine_msir(Cx& cx, const RefineArgs& a, RefStat
     }
     const double s_old = s, xnorm_old = mx;
     FOR_MY_ROWS(cx, i) a.x[i] = a.xn[i];
-    if (!(ok = grid_barrier(a.bar, a.err, cx.G))) break;
+    if (!(ok = grid_barrier(cx, a))) break;
     double ferr = 0.0;
     if (!(ok = residual<A0>(cx, a, a.x, ur, s, xnorm, &ferr))) break;
     nbe = s / (a.normA * xnorm + a.normb);
@@ -2830,7 +2864,7 @@ __device__ __forceinline__ bool refine_msir(Cx& cx, const RefineArgs& a, RefStat
       }
       __syncthreads();
       if (reset) {
-        if (!(ok = grid_barrier(a.bar, a.err, cx.G))) break;
+        if (!(ok = grid_barrier(cx, a))) break;
         if (!(ok = residual<A0>(cx, a, a.x, ur, s, xnorm))) break;
         nbe = s / (a.normA * xnorm + a.normb);
         const bool b2 = nbe < S.best_nbe;
@@ -2877,6 +2911,7 @@ __global__ void __launch_bounds__(kRefThreads, 1) refine_kernel(RefineArgs a) {
   cx.nblk = (a.n + kBlk - 1) / kBlk;
   cx.team_k = a.team_k;
   cx.redbuf = 0;
+  cx.nbar = 0;
   cx.inbox = (unsigned long long*)smem_raw;
   cx.C = 1;
   if (a.cluster > 1) {
@@ -2898,7 +2933,7 @@ __global__ void __launch_bounds__(kRefThreads, 1) refine_kernel(RefineArgs a) {
   bool ok = true;
   if (a.mode == MODE_RESIDUAL) {
     double s = 0.0, xn = 0.0;
-    ok = grid_barrier(a.bar, a.err, cx.G) && residual<A0>(cx, a, a.x, a.ap_arith, s, xn);
+    ok = grid_barrier(cx, a) && residual<A0>(cx, a, a.x, a.ap_arith, s, xn);
     if (ok && cx.cta == 0 && cx.tid == 0) *a.res_s = s;
   } else if (a.mode == MODE_APPLY) {
     for (int b = cx.cta; b < cx.nblk; b += cx.G)
