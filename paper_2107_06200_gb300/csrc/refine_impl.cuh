@@ -2231,6 +2231,11 @@ template <typename U>
 __device__ bool cgs_reduce(Cx& cx, const RefineArgs& a, int kp1, U* s_h) {
   PhaseTimer pt(cx, 3);
   if (!grid_barrier(cx, a)) return false;
+  if (cx.G == 1) {  // one block's partial sums are the sums
+    for (int j = cx.tid; j < kp1; j += kRefThreads) s_h[j] = UA<U>::rnd(a.hred[j]);
+    __syncthreads();
+    return true;
+  }
   for (int j = cx.cta * 8 + cx.warp; j < kp1; j += cx.G * 8) {
     double acc = 0.0;
     for (int c = cx.lane; c < cx.G; c += 32) acc = __dadd_rn(acc, __ldcg(a.hred + (size_t)c * (a.kcap + 1) + j));
@@ -2254,141 +2259,183 @@ __device__ bool cgs_reduce(Cx& cx, const RefineArgs& a, int kp1, U* s_h) {
 // The phase is bound by load latency, not bandwidth: each thread takes
 // kVec consecutive basis vectors (one 16-byte load per row; the basis is
 // row-major with ldv a multiple of 32) and loads kChunk rows ahead of the
-// sums, so a CTA keeps about 50 KB of loads in flight.
+// sums.  While there are few basis vectors, groups of gw threads (a power of
+// two) take every 256 / gw-th row each, and their sums are added by
+// shuffles and through shared memory.
 template <typename U>
 __device__ __noinline__ void cgs_partials(Cx& cx, const RefineArgs& a, const U* V, const U* w, int kp1) {
   PhaseTimer pt(cx, 3);
   constexpr int kVec = 16 / (int)sizeof(U);
   constexpr int kChunk = 12;
-  using Vec = typename std::conditional<sizeof(U) == 4, float4, double2>::type;
+  constexpr bool kF = sizeof(U) == 4;
+  using Vec = typename std::conditional<kF, float4, double2>::type;
+  using Acc = typename std::conditional<kF, ff_t, double>::type;
   int r0, r1;
   flat_rows(cx, r0, r1);
   const int nq = (kp1 + kVec - 1) / kVec;
-  for (int jq = cx.tid; jq < nq; jq += kRefThreads) {
-    const int j0 = jq * kVec;
+  int gw = 4;
+  while (gw < nq && gw < kRefThreads) gw *= 2;
+  const int ngrp = kRefThreads / gw;
+  Acc* part = (Acc*)cx.tsm;  // [warp][column of the warp's groups]
+  for (int jq = cx.tid & (gw - 1); jq < (nq + gw - 1) / gw * gw; jq += gw) {
+    const int j0 = min(jq, nq - 1) * kVec;
     // columns j0 .. j0 + kVec - 1 (those past k are summed and not stored)
-    ff_t af[kVec];
-    double ad[kVec];
+    Acc acc[kVec];
 #pragma unroll
     for (int e = 0; e < kVec; ++e) {
-      af[e] = ff_t{0.0f, 0.0f};
-      ad[e] = 0.0;
+      if constexpr (kF) acc[e] = ff_t{0.0f, 0.0f};
+      else acc[e] = 0.0;
     }
-    for (int i0 = r0; i0 < r1; i0 += kChunk) {
+    for (int i0 = r0 + cx.tid / gw; i0 < r1; i0 += kChunk * ngrp) {
       U vv[kChunk][kVec], wv[kChunk];
 #pragma unroll
       for (int c = 0; c < kChunk; ++c) {
-        const int i = i0 + c;
-        if (i < r1) {
-          const Vec t = __ldcg((const Vec*)(V + (size_t)i * a.ldv + j0));
-          const U* tp = (const U*)&t;
+        const int i = min(i0 + c * ngrp, r1 - 1);
+        const Vec t = __ldcg((const Vec*)(V + (size_t)i * a.ldv + j0));
+        const U* tp = (const U*)&t;
 #pragma unroll
-          for (int e = 0; e < kVec; ++e) vv[c][e] = tp[e];
-          wv[c] = __ldcg(w + i);
-        } else {
-#pragma unroll
-          for (int e = 0; e < kVec; ++e) vv[c][e] = (U)0;
-          wv[c] = (U)0;
-        }
+        for (int e = 0; e < kVec; ++e) vv[c][e] = tp[e];
+        wv[c] = __ldcg(w + i);
       }
 #pragma unroll
-      for (int c = 0; c < kChunk; ++c)
+      for (int c = 0; c < kChunk; ++c) {
+        if (i0 + c * ngrp < r1) {
+#pragma unroll
+          for (int e = 0; e < kVec; ++e) {
+            if constexpr (kF) acc[e] = ff_fma(vv[c][e], wv[c], acc[e]);
+            else acc[e] = __fma_rn(vv[c][e], wv[c], acc[e]);
+          }
+        }
+      }
+    }
+    auto add = [](Acc x, Acc y) {
+      if constexpr (kF) return ff_merge(x, y);
+      else return __dadd_rn(x, y);
+    };
+    for (int m = gw; m < 32; m *= 2) {
+#pragma unroll
+      for (int e = 0; e < kVec; ++e) {
+        if constexpr (kF) acc[e] = ff_merge(acc[e], ff_shfl_xor(acc[e], m));
+        else acc[e] = __dadd_rn(acc[e], __shfl_xor_sync(0xffffffffu, acc[e], m));
+      }
+    }
+    if (ngrp > 1) {
+#pragma unroll
+      for (int e = 0; e < kVec; ++e) part[cx.tid * kVec + e] = acc[e];
+      __syncthreads();
+      // the threads of the first group (of each warp: of its first one) hold
+      // the sums' columns; with gw < 32 a warp holds all of them
+      const int hop = gw < 32 ? 32 : gw;
+      if (cx.tid < gw) {
 #pragma unroll
         for (int e = 0; e < kVec; ++e) {
-          if constexpr (sizeof(U) == 4) af[e] = ff_fma(vv[c][e], wv[c], af[e]);
-          else ad[e] = __fma_rn(vv[c][e], wv[c], ad[e]);
-        }
-    }
+          Acc s[kRefThreads / 32];
 #pragma unroll
-    for (int e = 0; e < kVec; ++e) {
-      if (j0 + e >= kp1) break;
-      a.hred[(size_t)cx.cta * (a.kcap + 1) + j0 + e] =
-          sizeof(U) == 4 ? __dadd_rn((double)af[e].s, (double)af[e].c) : ad[e];
+          for (int g = 0; g < kRefThreads / 32; ++g) {
+            if constexpr (kF) s[g] = ff_t{0.0f, 0.0f};
+            else s[g] = 0.0;
+            if (g * hop < kRefThreads) s[g] = part[(cx.tid + g * hop) * kVec + e];
+          }
+          acc[e] = add(add(add(s[0], s[1]), add(s[2], s[3])), add(add(s[4], s[5]), add(s[6], s[7])));
+        }
+      }
+    }
+    if (cx.tid < gw && jq < nq) {
+#pragma unroll
+      for (int e = 0; e < kVec; ++e) {
+        if (j0 + e >= kp1) break;
+        double v;
+        if constexpr (kF) v = __dadd_rn((double)acc[e].s, (double)acc[e].c);
+        else v = acc[e];
+        a.hred[(size_t)cx.cta * (a.kcap + 1) + j0 + e] = v;
+      }
     }
   }
 }
 
-// sum_j V_j[i] c_j for the rows i0 .. i0+kRows-1 (those below r1) by one
-// warp: lane l sums the columns 4l .. 4l+3 (fp64: 2l, 2l+1) of every
-// 128-column (64) step, in order, with 16-byte loads two steps ahead, then a
-// butterfly over the lanes.  The rows' loads and reductions are
-// independent, so their latencies overlap.  Lane q < kRows returns row
-// i0+q's sum as a compensated pair (u = fp32: Dot2 in fp32, the pair's sum
-// is the value; u = fp64: an fp64 sum in .s, .c = 0).
+// sum_j V_j[i] c_j for the CTA's flat rows, handed to epi(i, pre(i), sum):
+// gw lanes (a power of two, 32 from 128 columns on; fp64: 64) share a row,
+// each summing groups of kVec consecutive columns by 16-byte loads, then a
+// butterfly over them; a warp has kRows rows per group of lanes in flight,
+// and what epi reads beside the sum (pre) is loaded with them.  The sum is a
+// compensated pair (u = fp32: Dot2 in fp32, the pair's sum is the value;
+// u = fp64: an fp64 sum in .s, .c = 0).
 struct RowSum {
   double s, c;
 };
-template <typename U, int kRows>
-__device__ __forceinline__ RowSum basis_rows_dot(const RefineArgs& a, const U* V, int i0, int r1, int kp1,
-                                                 const U* c, int lane) {
+template <typename U, int kRows, typename Pre, typename Epi>
+__device__ __forceinline__ void basis_rows_n(const Cx& cx, const RefineArgs& a, const U* V, int kp1, const U* c,
+                                             int gw, int r0, int r1, Pre pre, Epi epi) {
   constexpr int kVec = 16 / (int)sizeof(U);
-  constexpr int kStep = 32 * kVec;
-  using Vec = typename std::conditional<sizeof(U) == 4, float4, double2>::type;
-  ff_t af[kRows];
-  double ad[kRows];
-#pragma unroll
-  for (int q = 0; q < kRows; ++q) {
-    af[q] = ff_t{0.0f, 0.0f};
-    ad[q] = 0.0;
-  }
-  const int nr = min(kRows, r1 - i0);
-#pragma unroll 2
-  for (int j0 = lane * kVec; j0 < kp1; j0 += kStep) {
-    U vv[kRows][kVec], cj[kVec];
-#pragma unroll
-    for (int e = 0; e < kVec; ++e) cj[e] = j0 + e < kp1 ? c[j0 + e] : (U)0;
+  constexpr bool kF = sizeof(U) == 4;
+  using Vec = typename std::conditional<kF, float4, double2>::type;
+  const int l = cx.lane & (gw - 1), sub = cx.lane / gw, spw = 32 / gw;
+  for (int i0 = r0 + cx.warp * kRows * spw; i0 < r1; i0 += (kRefThreads / 32) * kRows * spw) {
+    ff_t af[kRows];
+    double ad[kRows];
+    U pv[kRows];
+    size_t row[kRows];
 #pragma unroll
     for (int q = 0; q < kRows; ++q) {
-      if (q < nr) {
-        const Vec t = __ldcg((const Vec*)(V + (size_t)(i0 + q) * a.ldv + j0));
+      const int i = min(i0 + q * spw + sub, r1 - 1);
+      row[q] = (size_t)i * a.ldv;
+      pv[q] = pre(i);
+      af[q] = ff_t{0.0f, 0.0f};
+      ad[q] = 0.0;
+    }
+    auto step = [&](int j0, bool full) {
+      U vv[kRows][kVec], cj[kVec];
+#pragma unroll
+      for (int e = 0; e < kVec; ++e) cj[e] = full || j0 + e < kp1 ? c[j0 + e] : (U)0;
+#pragma unroll
+      for (int q = 0; q < kRows; ++q) {
+        const Vec t = __ldcg((const Vec*)(V + row[q] + j0));
         const U* tp = (const U*)&t;
 #pragma unroll
-        for (int e = 0; e < kVec; ++e) vv[q][e] = j0 + e < kp1 ? tp[e] : (U)0;  // columns past k may hold anything
-      } else {
+        for (int e = 0; e < kVec; ++e) vv[q][e] = full || j0 + e < kp1 ? tp[e] : (U)0;  // past k: anything
+      }
 #pragma unroll
-        for (int e = 0; e < kVec; ++e) vv[q][e] = (U)0;
+      for (int q = 0; q < kRows; ++q)
+#pragma unroll
+        for (int e = 0; e < kVec; ++e) {
+          if constexpr (kF) af[q] = ff_fma(vv[q][e], cj[e], af[q]);
+          else ad[q] = __fma_rn(vv[q][e], cj[e], ad[q]);
+        }
+    };
+    int j0 = l * kVec;
+#pragma unroll 2
+    for (; j0 + kVec <= kp1; j0 += gw * kVec) step(j0, true);
+    if (j0 < kp1) step(j0, false);
+    __syncwarp();
+    for (int m = gw / 2; m > 0; m >>= 1) {
+#pragma unroll
+      for (int q = 0; q < kRows; ++q) {
+        if constexpr (kF) af[q] = ff_merge(af[q], ff_shfl_xor(af[q], m));
+        else ad[q] = __dadd_rn(ad[q], __shfl_xor_sync(0xffffffffu, ad[q], m));
       }
     }
 #pragma unroll
-    for (int q = 0; q < kRows; ++q)
-#pragma unroll
-      for (int e = 0; e < kVec; ++e) {
-        if constexpr (sizeof(U) == 4) af[q] = ff_fma(vv[q][e], cj[e], af[q]);
-        else ad[q] = __fma_rn(vv[q][e], cj[e], ad[q]);
-      }
-  }
-  RowSum mine{0.0, 0.0};
-#pragma unroll
-  for (int q = 0; q < kRows; ++q) {
-    if constexpr (sizeof(U) == 4) {
-#pragma unroll
-      for (int m = 16; m > 0; m >>= 1) af[q] = ff_merge(af[q], ff_shfl_xor(af[q], m));
-      if (lane == q) mine = RowSum{(double)af[q].s, (double)af[q].c};
-    } else {
-      const double t = warp_sum_d(ad[q]);
-      if (lane == q) mine.s = t;
+    for (int q = 0; q < kRows; ++q) {
+      const int i = i0 + q * spw + sub;
+      if (l == (q & (gw - 1)) && i < r1)
+        epi(i, pv[q], kF ? RowSum{(double)af[q].s, (double)af[q].c} : RowSum{ad[q], 0.0});
     }
   }
-  return mine;
 }
-
-// rows per warp: the CTA's rows over its 8 warps
-template <typename U, typename Epi>
-__device__ __forceinline__ void basis_rows(const Cx& cx, const RefineArgs& a, const U* V, int kp1, const U* c, Epi epi) {
+template <typename U, typename Pre, typename Epi>
+__device__ __forceinline__ void basis_rows(const Cx& cx, const RefineArgs& a, const U* V, int kp1, const U* c, Pre pre,
+                                           Epi epi) {
+  constexpr int kVec = 16 / (int)sizeof(U);
   int r0, r1;
   flat_rows(cx, r0, r1);
-  auto run = [&](auto rows) {
-    constexpr int kRows = decltype(rows)::value;
-    for (int i0 = r0 + cx.warp * kRows; i0 < r1; i0 += (kRefThreads / 32) * kRows) {
-      const RowSum acc = basis_rows_dot<U, kRows>(a, V, i0, r1, kp1, c, cx.lane);
-      const int i = i0 + cx.lane;
-      if (cx.lane < kRows && i < r1) epi(i, acc);
-    }
-  };
-  const int per = (r1 - r0 + kRefThreads / 32 - 1) / (kRefThreads / 32);
-  if (per <= 2) run(std::integral_constant<int, 2>());
-  else if (per <= 4) run(std::integral_constant<int, 4>());
-  else run(std::integral_constant<int, 8>());
+  int gw = 4;
+  while (gw < 32 && gw * kVec < kp1) gw *= 2;
+  const int spw = 32 / gw;
+  // rows per group of lanes that let all warps work
+  const int per = (r1 - r0 + kRefThreads / 32 * spw - 1) / (kRefThreads / 32 * spw);
+  if (per <= 2) basis_rows_n<U, 2>(cx, a, V, kp1, c, gw, r0, r1, pre, epi);
+  else if (per <= 4) basis_rows_n<U, 4>(cx, a, V, kp1, c, gw, r0, r1, pre, epi);
+  else basis_rows_n<U, 8>(cx, a, V, kp1, c, gw, r0, r1, pre, epi);
 }
 
 // w_i = fl_u(w_i - sum_j V_j[i] h_j) with the difference taken from the
@@ -2396,11 +2443,11 @@ __device__ __forceinline__ void basis_rows(const Cx& cx, const RefineArgs& a, co
 template <typename U>
 __device__ __noinline__ void cgs_update(Cx& cx, const RefineArgs& a, const U* V, U* w, int kp1, const U* s_h) {
   PhaseTimer pt(cx, 3);
-  basis_rows<U>(cx, a, V, kp1, s_h, [&](int i, RowSum acc) {
+  basis_rows<U>(cx, a, V, kp1, s_h, [&](int i) { return w[i]; }, [&](int i, U wi, RowSum acc) {
     if constexpr (sizeof(U) == 4)
-      w[i] = ff_sub_from(w[i], ff_t{(float)acc.s, (float)acc.c});
+      w[i] = ff_sub_from(wi, ff_t{(float)acc.s, (float)acc.c});
     else
-      w[i] = UA<U>::rnd(__dsub_rn((double)w[i], acc.s));
+      w[i] = UA<U>::rnd(__dsub_rn((double)wi, acc.s));
   });
   __syncthreads();
 }
@@ -2408,7 +2455,7 @@ __device__ __noinline__ void cgs_update(Cx& cx, const RefineArgs& a, const U* V,
 // d_i = fl_u(sum_j V_j[i] y_j) over the flat rows (the GMRES correction)
 template <typename U>
 __device__ __noinline__ void basis_combine(Cx& cx, const RefineArgs& a, const U* V, int kdone, const U* y) {
-  basis_rows<U>(cx, a, V, kdone, y, [&](int i, RowSum acc) {
+  basis_rows<U>(cx, a, V, kdone, y, [](int) { return (U)0; }, [&](int i, U, RowSum acc) {
     a.d[i] = sizeof(U) == 4 ? (double)ff_fin(ff_t{(float)acc.s, (float)acc.c}) : (double)UA<U>::rnd(acc.s);
   });
 }
