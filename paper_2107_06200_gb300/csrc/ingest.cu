@@ -10,7 +10,11 @@
 //    with power-of-two R, S, mu (the two-sided scaling of Sec. 2.1.2).
 //  * vector rounding b_u = fl_u0(b) and infinity norms.
 #include "common.cuh"
+#include "factor_io.cuh"
 #include "ingest.h"
+
+#include <algorithm>
+#include <type_traits>
 
 namespace msir {
 
@@ -30,22 +34,41 @@ __global__ void ingest_matrix_kernel(const double* __restrict__ Ain, int lda, in
   }
 }
 
-template <typename U0>
-__global__ void row_stats_kernel(const U0* Au, int ldu, int n, double* rowsum, double* rowmax) {
+// One warp per row, lane l summing columns l, l + 32, .. in order.  fp32
+// rows are widened by integer instructions (see common.cuh) and the maximum,
+// three fp64-pipe operations of its own, is formed only where it is wanted:
+// GB300's fp64 pipe takes 2 operations a cycle and SM.
+template <typename U0, bool MAX>
+__global__ void row_stats_kernel(const U0* __restrict__ Au, int ldu, int n, double* rowsum, double* rowmax) {
   const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (warp >= n) return;
   const U0* row = Au + (size_t)warp * ldu;
+  constexpr int kAhead = 8;
   double s = 0.0, m = 0.0;
-  for (int j = lane; j < n; j += 32) {
-    const double v = fabs((double)row[j]);
-    s = __dadd_rn(s, v);
-    m = nanmax(m, v);
+  for (int j0 = lane; j0 < n; j0 += 32 * kAhead) {
+    U0 v[kAhead];
+#pragma unroll
+    for (int q = 0; q < kAhead; ++q) v[q] = j0 + 32 * q < n ? row[j0 + 32 * q] : (U0)0;
+#pragma unroll
+    for (int q = 0; q < kAhead; ++q) {
+      double d;
+      if constexpr (sizeof(U0) == 4) {
+        const float f = fabsf(v[q]);
+        d = widen_special(f) ? (double)f : widen_normal(f);
+      } else {
+        d = fabs(v[q]);
+      }
+      if (j0 + 32 * q < n) {
+        s = __dadd_rn(s, d);
+        if (MAX) m = nanmax(m, d);
+      }
+    }
   }
   s = warp_sum_d(s);
-  m = warp_nanmax_d(m);
+  if (MAX) m = warp_nanmax_d(m);
   if (lane == 0) {
     if (rowsum) rowsum[warp] = s;
-    if (rowmax) rowmax[warp] = m;
+    if (MAX) rowmax[warp] = m;
   }
 }
 
@@ -71,14 +94,17 @@ __global__ void col_max_scaled_kernel(const U0* Au, int ldu, int n, const double
   colmax[j] = m;
 }
 
+// A block of kFactorThreads threads per row piece, kFactorVec consecutive
+// entries each with 16-byte loads and stores (rows start on 64-entry
+// boundaries; what lies past column n is not written).  Bound by memory;
+// one entry a thread through fp64 took 0.6 ms at n = 8192 (fp32 to fp16).
+constexpr int kFactorThreads = 256;
 template <typename U0, typename F>
-__global__ void make_factor_kernel(const U0* Au, int ldu, int n, F* Af, int ldf, const double* R,
-                                   const double* S, double mu) {
-  const int j = blockIdx.x * blockDim.x + threadIdx.x, i = blockIdx.y;
+__global__ void make_factor_kernel(const U0* __restrict__ Au, int ldu, int n, F* __restrict__ Af, int ldf,
+                                   const double* R, const double* S, double mu) {
+  const int j = (blockIdx.x * kFactorThreads + threadIdx.x) * kFactorVec, i = blockIdx.y;
   if (j >= n) return;
-  double v = (double)Au[(size_t)i * ldu + j];
-  if (R) v = v * R[i] * S[j] * mu;
-  Af[(size_t)i * ldf + j] = from_d<F>(v);
+  factor_piece<U0, F>(Au + (size_t)i * ldu, i, j, n, Af + (size_t)i * ldf, R, S, mu);
 }
 
 __global__ void round_vec_kernel(const double* in, int n, int fmt, double* out) {
@@ -106,26 +132,9 @@ __global__ void copy_strided_kernel(const double* src, int n, double* dst) {
   if (i < n) dst[i] = src[i];
 }
 
-// The interchanges are sequential by nature: one thread applies them to a
-// permutation held in shared memory (the block stages ipiv and perm).
-__global__ void ipiv_to_perm_kernel(const int* ipiv, int n, int* perm) {
+__global__ void ipiv_to_perm_kernel(const int* ipiv, int n, int* perm, int runs) {
   extern __shared__ int sm[];
-  int* sp = sm;
-  int* si = sm + n;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) { sp[i] = i; si[i] = ipiv[i]; }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int j = 0; j < n; ++j) {
-      const int p = si[j];
-      if (p != j) {
-        const int t = sp[j];
-        sp[j] = sp[p];
-        sp[p] = t;
-      }
-    }
-  }
-  __syncthreads();
-  for (int i = threadIdx.x; i < n; i += blockDim.x) perm[i] = sp[i];
+  perm_of_pivots(ipiv, n, perm, runs, sm);
 }
 
 __global__ void iota_kernel(int* p, int n) {
@@ -147,10 +156,17 @@ cudaError_t ingest_matrix(const double* Ain, int lda, int n, int u0, void* Au, i
 cudaError_t row_stats(const void* Au, int ldu, int n, int u0, double* rowsum, double* rowmax,
                       cudaStream_t st) {
   const int threads = 256, blocks = (n * 32 + threads - 1) / threads;
-  if (u0 == MSIR_FP32)
-    row_stats_kernel<float><<<blocks, threads, 0, st>>>((const float*)Au, ldu, n, rowsum, rowmax);
-  else
-    row_stats_kernel<double><<<blocks, threads, 0, st>>>((const double*)Au, ldu, n, rowsum, rowmax);
+  auto run = [&](auto* A, auto max) {
+    using U0 = typename std::remove_cv<typename std::remove_pointer<decltype(A)>::type>::type;
+    row_stats_kernel<U0, decltype(max)::value><<<blocks, threads, 0, st>>>(A, ldu, n, rowsum, rowmax);
+  };
+  if (u0 == MSIR_FP32) {
+    if (rowmax) run((const float*)Au, std::true_type());
+    else run((const float*)Au, std::false_type());
+  } else {
+    if (rowmax) run((const double*)Au, std::true_type());
+    else run((const double*)Au, std::false_type());
+  }
   return cudaGetLastError();
 }
 
@@ -170,12 +186,13 @@ cudaError_t squeeze_scalings(const void* Au, int ldu, int n, int u0, double* row
 template <typename U0>
 static cudaError_t make_factor_u0(const U0* Au, int ldu, int n, int uf, void* Af, int ldf,
                                   const double* R, const double* S, double mu, cudaStream_t st) {
-  dim3 grid((n + 255) / 256, n);
+  constexpr int kRow = kFactorThreads * kFactorVec;
+  dim3 grid((n + kRow - 1) / kRow, n);
   switch (uf) {
-    case MSIR_FP16: make_factor_kernel<U0, __half><<<grid, 256, 0, st>>>(Au, ldu, n, (__half*)Af, ldf, R, S, mu); break;
-    case MSIR_BF16: make_factor_kernel<U0, __nv_bfloat16><<<grid, 256, 0, st>>>(Au, ldu, n, (__nv_bfloat16*)Af, ldf, R, S, mu); break;
-    case MSIR_FP32: make_factor_kernel<U0, float><<<grid, 256, 0, st>>>(Au, ldu, n, (float*)Af, ldf, R, S, mu); break;
-    case MSIR_FP64: make_factor_kernel<U0, double><<<grid, 256, 0, st>>>(Au, ldu, n, (double*)Af, ldf, R, S, mu); break;
+    case MSIR_FP16: make_factor_kernel<U0, __half><<<grid, kFactorThreads, 0, st>>>(Au, ldu, n, (__half*)Af, ldf, R, S, mu); break;
+    case MSIR_BF16: make_factor_kernel<U0, __nv_bfloat16><<<grid, kFactorThreads, 0, st>>>(Au, ldu, n, (__nv_bfloat16*)Af, ldf, R, S, mu); break;
+    case MSIR_FP32: make_factor_kernel<U0, float><<<grid, kFactorThreads, 0, st>>>(Au, ldu, n, (float*)Af, ldf, R, S, mu); break;
+    case MSIR_FP64: make_factor_kernel<U0, double><<<grid, kFactorThreads, 0, st>>>(Au, ldu, n, (double*)Af, ldf, R, S, mu); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();
@@ -198,11 +215,15 @@ cudaError_t max_abs(const double* v, int n, int absval, double* out, cudaStream_
 }
 
 cudaError_t ipiv_to_perm(const int* ipiv, int n, int* perm, cudaStream_t st) {
-  const size_t smem = (size_t)2 * n * sizeof(int);
+  // as many runs as shared memory holds beside the interchanges, two at
+  // least (8 bytes a row: n up to 29056)
+  constexpr size_t kRoom = 226 * 1024;
+  const int runs = (int)std::min<size_t>(kPermRuns, std::max<size_t>(2, kRoom / n < 4 ? 0 : (kRoom / n - 4) / 2));
+  const size_t smem = (size_t)n * (sizeof(int) + runs * sizeof(unsigned short));
   cudaError_t e = cudaFuncSetAttribute(ipiv_to_perm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)smem);
   if (e != cudaSuccess) return e;
-  ipiv_to_perm_kernel<<<1, 1024, smem, st>>>(ipiv, n, perm);
+  ipiv_to_perm_kernel<<<1, 1024, smem, st>>>(ipiv, n, perm, runs);
   return cudaGetLastError();
 }
 
