@@ -10,7 +10,7 @@ void* batched_solve_entry_f32();
 void* batched_solve_entry_f64();
 
 size_t batch_smem_bytes(int kcap) {
-  const size_t lu = std::max(cta_lu_smem<float>(32), cta_lu_smem<double>(16));
+  const size_t lu = std::max(cta_lu_smem<float>(), cta_lu_smem<double>());
   const size_t refine = refine_smem_bytes(kcap);
   return std::max(lu, refine);
 }
@@ -62,7 +62,7 @@ size_t batched_factor_ws_bytes(int fmt) {
 template <typename F>
 static cudaError_t launch_factor_t(const BatchFactorTask* tasks, int count, char* ws, size_t ws_stride, int nb,
                                    int nbo, int grid, cudaStream_t st) {
-  const size_t smem = cta_lu_smem<F>(nb);
+  const size_t smem = cta_lu_smem<F>();
   cudaError_t e = cudaFuncSetAttribute(batched_factor_kernel<F>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)smem);
   if (e != cudaSuccess) return e;

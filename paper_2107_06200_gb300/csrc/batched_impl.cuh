@@ -15,6 +15,7 @@
 #include <cuda_bf16.h>
 
 #include "batched.h"
+#include "factor_io.cuh"
 #include "lu_cta.cuh"
 #include "refine_impl.cuh"
 
@@ -57,22 +58,25 @@ __device__ __forceinline__ void batch_lu_fmt(int fmt, void* A, int lda, int n, i
 }
 // A_f = fl_f(A_u), or fl_f(mu R_i a_ij S_j) when squeezed (the same
 // product order as the single-system path)
+template <typename A0, typename F>
+__device__ void batch_make_factor_t(const A0* Au, int ldu, int n, F* Af, const double* R, const double* S,
+                                    double mu) {
+  const int lane = threadIdx.x & 31;
+  for (int i = threadIdx.x >> 5; i < n; i += kBatchThreads / 32)
+#pragma unroll 2
+    for (int j = lane * kFactorVec; j < n; j += 32 * kFactorVec)
+      factor_piece<A0, F>(Au + (size_t)i * ldu, i, j, n, Af + (size_t)i * ldu, R, S, mu);
+  __syncthreads();
+}
 template <typename A0>
 __device__ void batch_make_factor(int fmt, const A0* Au, int ldu, int n, void* Af, const double* R,
                                   const double* S, double mu) {
-  for (int e = threadIdx.x; e < n * n; e += kBatchThreads) {
-    const int i = e / n, j = e % n;
-    double v = (double)Au[(size_t)i * ldu + j];
-    if (R) v = v * R[i] * S[j] * mu;
-    const size_t o = (size_t)i * ldu + j;
-    switch (fmt) {
-      case MSIR_FP16: ((__half*)Af)[o] = from_d<__half>(v); break;
-      case MSIR_BF16: ((__nv_bfloat16*)Af)[o] = from_d<__nv_bfloat16>(v); break;
-      case MSIR_FP32: ((float*)Af)[o] = from_d<float>(v); break;
-      default: ((double*)Af)[o] = v; break;
-    }
+  switch (fmt) {
+    case MSIR_FP16: batch_make_factor_t<A0, __half>(Au, ldu, n, (__half*)Af, R, S, mu); break;
+    case MSIR_BF16: batch_make_factor_t<A0, __nv_bfloat16>(Au, ldu, n, (__nv_bfloat16*)Af, R, S, mu); break;
+    case MSIR_FP32: batch_make_factor_t<A0, float>(Au, ldu, n, (float*)Af, R, S, mu); break;
+    default: batch_make_factor_t<A0, double>(Au, ldu, n, (double*)Af, R, S, mu); break;
   }
-  __syncthreads();
 }
 
 // scale = 2^-e where m = f 2^e, f in [1/2, 1) (1 for m == 0 or non-finite)
@@ -99,22 +103,6 @@ __device__ void batch_squeeze(const A0* Au, int ldu, int n, double* R, double* S
     double m = 0.0;
     for (int i = 0; i < n; ++i) m = nanmax(m, fabs((double)Au[(size_t)i * ldu + j] * R[i]));
     S[j] = batch_pow2_inv(m);
-  }
-  __syncthreads();
-}
-
-// permutation of a LAPACK-style ipiv: (P A)[i] = A[perm[i]]
-static __device__ void batch_perm(const int* ipiv, int n, int* perm) {
-  if (threadIdx.x == 0) {
-    for (int i = 0; i < n; ++i) perm[i] = i;
-    for (int j = 0; j < n; ++j) {
-      const int p = ipiv[j];
-      if (p != j) {
-        const int t = perm[j];
-        perm[j] = perm[p];
-        perm[p] = t;
-      }
-    }
   }
   __syncthreads();
 }
@@ -154,9 +142,21 @@ __global__ void __launch_bounds__(kBatchThreads, 1) batched_solve_kernel(BatchAr
     const BatchTask T = B.tasks[t];
     const int n = T.n, ldu = L.ldu, u0 = T.u;
     // ---- ingest: A_u = fl_u0(A) row-major, b_u, norms
-    for (int e = tid; e < n * n; e += kBatchThreads) {
-      const int j = e / n, i = e % n;  // column-major reads, coalesced
-      Au[(size_t)i * ldu + j] = (A0)T.A[(size_t)j * n + i];
+    // (32 x 32 tiles through shared memory, one per warp at a time)
+    {
+      A0* tile = (A0*)smem_raw + warp * 32 * 33;
+      const int nt = (n + 31) / 32;
+      for (int q = warp; q < nt * nt; q += kBatchThreads / 32) {
+        const int bi = q / nt * 32, bj = q % nt * 32;
+#pragma unroll 16
+        for (int c = 0; c < 32; ++c)
+          tile[c * 33 + lane] = bj + c < n && bi + lane < n ? (A0)T.A[(size_t)(bj + c) * n + bi + lane] : (A0)0;
+        __syncwarp();
+#pragma unroll 8
+        for (int r = 0; r < 32; ++r)
+          if (bi + r < n && bj + lane < n) Au[(size_t)(bi + r) * ldu + bj + lane] = tile[lane * 33 + r];
+        __syncwarp();
+      }
     }
     for (int i = tid; i < n; i += kBatchThreads) b_u[i] = round_to(T.b[i], u0);
     if (tid < 32) iflags[tid] = 0;
@@ -301,7 +301,7 @@ __global__ void __launch_bounds__(kBatchThreads, 1) batched_solve_kernel(BatchAr
       }
       lu_info = 0;
       scaled = squeeze ? 1 : 0;
-      batch_perm(ipiv, n, perm);
+      perm_of_pivots(ipiv, n, perm, kPermRuns, (int*)smem_raw);
       t_factor += 1e-6 * (double)(gtimer() - tf0);
       if (tid == 0 && fmt != S.uf) {  // precision raised (Algorithm 4's escalation)
         S.uf = fmt;
@@ -385,18 +385,19 @@ __global__ void __launch_bounds__(kBatchThreads, 1)
     batched_factor_kernel(const BatchFactorTask* tasks, int count, char* ws, size_t ws_stride, int nb, int nbo) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ int s_info, s_nonfinite;
-  F* Af = (F*)(ws + (size_t)blockIdx.x * ws_stride);
+  F* Af = (F*)(ws + (size_t)blockIdx.x * ws_stride);  // kBatchMaxN rows of kBatchMaxN entries at most
   int* ipiv = (int*)(ws + (size_t)blockIdx.x * ws_stride + (size_t)kBatchMaxN * kBatchMaxN * sizeof(F));
   for (int t = blockIdx.x; t < count; t += gridDim.x) {
     const BatchFactorTask T = tasks[t];
-    const int n = T.n;
+    const int n = T.n, lda = (n + 63) / 64 * 64;
     for (int e = threadIdx.x; e < n * n; e += kBatchThreads) {
       const int j = e / n, i = e % n;
-      Af[(size_t)i * n + j] = from_d<F>(T.A[(size_t)j * n + i]);
+      Af[(size_t)i * lda + j] = from_d<F>(T.A[(size_t)j * n + i]);
     }
     __syncthreads();
-    cta_lu<F>(Af, n, n, nb, nbo, ipiv, &s_info, &s_nonfinite, smem_raw);
-    for (int e = threadIdx.x; e < n * n; e += kBatchThreads) T.F_out[e] = (double)to_f(Af[e]);
+    cta_lu<F>(Af, lda, n, nb, nbo, ipiv, &s_info, &s_nonfinite, smem_raw);
+    for (int e = threadIdx.x; e < n * n; e += kBatchThreads)
+      T.F_out[e] = (double)to_f(Af[(size_t)(e / n) * lda + e % n]);
     for (int i = threadIdx.x; i < n; i += kBatchThreads) T.ipiv_out[i] = ipiv[i];
     if (threadIdx.x == 0) {
       T.flags_out[0] = s_info;

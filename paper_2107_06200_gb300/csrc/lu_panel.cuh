@@ -15,45 +15,6 @@ namespace cg = cooperative_groups;
 
 namespace msir {
 
-// Panel width limit per arithmetic precision (also the register arrays).
-template <typename T> struct PanelNB { static constexpr int v = 32; };
-template <> struct PanelNB<double> { static constexpr int v = 16; };
-
-// Pivot order: larger |a| first; NaN only if nothing else; equal magnitudes
-// -> smaller row index.
-// Pivot keys: monotone in |a|, 0 for "no candidate", 1 for NaN (chosen only
-// if nothing else is left), else the bits of |a| plus 2 (the bits of a
-// non-negative IEEE number order like its value).
-template <typename T> struct PivKey;
-template <> struct PivKey<float> {
-  using K = unsigned;
-  static __device__ __forceinline__ K of(float v) {
-    const unsigned b = __float_as_uint(v) & 0x7fffffffu;
-    return b > 0x7f800000u ? 1u : b + 2u;
-  }
-};
-template <> struct PivKey<double> {
-  using K = unsigned long long;
-  static __device__ __forceinline__ K of(double v) {
-    const unsigned long long b = (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
-    return b > 0x7ff0000000000000ull ? 1ull : b + 2ull;
-  }
-};
-// Largest key of the warp and the smallest index among the lanes holding it.
-__device__ __forceinline__ void warp_argmax(unsigned& key, int& i) {
-  const unsigned mk = __reduce_max_sync(0xffffffffu, key);
-  i = __reduce_min_sync(0xffffffffu, key == mk ? i : INT_MAX);
-  key = mk;
-}
-__device__ __forceinline__ void warp_argmax(unsigned long long& key, int& i) {
-  const unsigned hi = (unsigned)(key >> 32);
-  const unsigned mh = __reduce_max_sync(0xffffffffu, hi);
-  const unsigned ml = __reduce_max_sync(0xffffffffu, hi == mh ? (unsigned)key : 0u);
-  const unsigned long long mk = ((unsigned long long)mh << 32) | ml;
-  i = __reduce_min_sync(0xffffffffu, key == mk ? i : INT_MAX);
-  key = mk;
-}
-
 // ------------------------------------------------------------------ panel
 
 // Optional section timers (rank 0, thread 0): 0 column loop, 4 panel store
@@ -64,29 +25,6 @@ __device__ __forceinline__ void warp_argmax(unsigned long long& key, int& i) {
 #define PT_BEGIN(id) unsigned long long _t##id = (a.tdbg && rank == 0 && tid == 0) ? gtimer() : 0
 #define PT_END(id) \
   if (a.tdbg && rank == 0 && tid == 0) s_tacc[id] += gtimer() - _t##id
-
-// N consecutive values of T in 16-byte loads / stores (16-byte aligned).
-template <typename T, int N>
-__device__ __forceinline__ void ld_vec(const T* p, T (&v)[N]) {
-  constexpr int E = 16 / (int)sizeof(T);
-  static_assert(N % E == 0, "whole 16-byte loads");
-#pragma unroll
-  for (int m = 0; m < N / E; ++m) {
-    const uint4 u = reinterpret_cast<const uint4*>(p)[m];
-    memcpy(&v[m * E], &u, 16);
-  }
-}
-template <typename T, int N>
-__device__ __forceinline__ void st_vec(T* p, const T (&v)[N]) {
-  constexpr int E = 16 / (int)sizeof(T);
-  static_assert(N % E == 0, "whole 16-byte stores");
-#pragma unroll
-  for (int m = 0; m < N / E; ++m) {
-    uint4 u;
-    memcpy(&u, &v[m * E], 16);
-    reinterpret_cast<uint4*>(p)[m] = u;
-  }
-}
 
 // Pivot exchange between the CTAs of a cluster: each sends its candidate's
 // row (kCandRow bytes) and key / position (16 bytes) into a slot of every
@@ -133,9 +71,6 @@ static __device__ __noinline__ void cand_wait_slow(unsigned mbar, unsigned parit
     }
   }
 }
-
-// One step of applying the interchange (j, q) to the position of a row.
-__device__ __forceinline__ int swap_step(int pos, int j, int q) { return pos == j ? q : (pos == q ? j : pos); }
 
 // The column loop is a chain: a pivot search over all rows, one exchange
 // across the cluster, one rank-1 update, w times per panel.  What bounds it
