@@ -266,7 +266,7 @@ __global__ void __launch_bounds__(256) lu_outer_swap_trsm(SwapTrsmArgs a) {
 // while the current one is used, and shared memory holds two slices, so a
 // slice costs one block barrier.
 template <typename T, int BM, int BN>
-__global__ void __launch_bounds__(256) lu_update_simt(UpdateArgs a) {
+__global__ void __launch_bounds__(256, BM * BN > 64 * 64 ? 2 : sizeof(T) == 8 ? 3 : 4) lu_update_simt(UpdateArgs a) {
   constexpr int BK = 16;
   constexpr int E = 16 / (int)sizeof(T);       // values per 16-byte load
   constexpr int TM = BM / 16, TN = BN / 16;    // elements per thread
@@ -285,11 +285,25 @@ __global__ void __launch_bounds__(256) lu_update_simt(UpdateArgs a) {
   const int ty = tid / 16, tx = tid % 16;
   // 16-byte loads need aligned columns (rows start on 64-element boundaries)
   const bool vecA = (k % E) == 0, vecB = (c0 % E) == 0;
-  T acc[TM][TN];
+  // C is read at the end: bring its lines to L2 meanwhile
+  {
+    constexpr int kLine = 128 / (int)sizeof(T);
+    for (int l = tid; l < BM * (BN / kLine); l += 256) {
+      const int i = tm + l / (BN / kLine), j = tn + l % (BN / kLine) * kLine;
+      if (i < M && j < NC)
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(A + (size_t)(r0 + i) * lda + c0 + j));
+    }
+  }
+  // fp32: two neighbouring columns per accumulator (one instruction for the
+  // two fused multiply-adds, each rounded as usual)
+  constexpr bool kPair = std::is_same<T, float>::value;
+  using Acc = typename std::conditional<kPair, unsigned long long, T>::type;
+  constexpr int NA = kPair ? TN / 2 : TN;
+  Acc acc2[TM][NA];
 #pragma unroll
   for (int i = 0; i < TM; ++i)
 #pragma unroll
-    for (int j = 0; j < TN; ++j) acc[i][j] = 0;
+    for (int j = 0; j < NA; ++j) acc2[i][j] = 0;
   // slice loads: L21 values kq = E (idx % (BK / E)) .. of row idx / (BK / E);
   // U12 columns E (idx % (BN / E)) .. of row idx / (BN / E)
   T ra[LA], rb[LB];
@@ -335,19 +349,29 @@ __global__ void __launch_bounds__(256) lu_update_simt(UpdateArgs a) {
     }
   };
   auto step = [&](int buf, int kq) {
-    T av[TM], bv[TN];
+    T av[TM];
+    Acc bv[NA];
 #pragma unroll
     for (int h = 0; h < HM; ++h)
 #pragma unroll
       for (int i = 0; i < VM; ++i) av[h * VM + i] = As[buf][kq][h * (BM / HM) + ty * VM + i];
+    constexpr int NV = NA / HN;
 #pragma unroll
     for (int h = 0; h < HN; ++h)
+      memcpy(&bv[h * NV], __builtin_assume_aligned(&Bs[buf][kq][h * (BN / HN) + tx * VN], VN * sizeof(T)), VN * sizeof(T));
 #pragma unroll
-      for (int j = 0; j < VN; ++j) bv[h * VN + j] = Bs[buf][kq][h * (BN / HN) + tx * VN + j];
+    for (int i = 0; i < TM; ++i) {
+      if constexpr (kPair) {
+        unsigned long long a2;
+        asm("mov.b64 %0, {%1, %1};" : "=l"(a2) : "f"(av[i]));
 #pragma unroll
-    for (int i = 0; i < TM; ++i)
+        for (int j = 0; j < NA; ++j)
+          asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc2[i][j]) : "l"(a2), "l"(bv[j]));
+      } else {
 #pragma unroll
-      for (int j = 0; j < TN; ++j) acc[i][j] = fma_rn(av[i], bv[j], acc[i][j]);
+        for (int j = 0; j < NA; ++j) acc2[i][j] = fma_rn(av[i], bv[j], acc2[i][j]);
+      }
+    }
   };
   load(0);
   put(0);
@@ -366,6 +390,8 @@ __global__ void __launch_bounds__(256) lu_update_simt(UpdateArgs a) {
     __syncthreads();
   }
   const bool vecC = vecB && VN == E;
+  T acc[TM][TN];
+  memcpy(acc, acc2, sizeof(acc));
 #pragma unroll
   for (int i = 0; i < TM; ++i) {
     const int row = tm + (i / VM) * (BM / HM) + ty * VM + i % VM;
