@@ -143,6 +143,12 @@ template <> struct RowAcc<MSIR_DD> {
     s = v.hi;
     c = v.lo;
   }
+  // as a term of the sum: five fp64 operations instead of 26
+  __device__ __forceinline__ void merge_term(const RowAcc& o) {
+    const dd_t t = two_sum_ord(s, o.s);
+    s = t.hi;
+    c = __dadd_rn(c, __dadd_rn(t.lo, o.c));
+  }
   __device__ __forceinline__ RowAcc peer(int m) const {
     return RowAcc{__shfl_xor_sync(0xffffffffu, s, m), __shfl_xor_sync(0xffffffffu, c, m)};
   }
@@ -259,28 +265,40 @@ __device__ __forceinline__ void gemv_rows_n(Cx& cx, const RefineArgs& a, const X
           for (int r = 0; r < NR; ++r) acc[r][q & 1].add(av[r][q], xv[q]);
       }
     }
+    // Double-double: a lane's sums as terms of the row's from kTermMerge
+    // columns on.  n = 8192: 1.29 -> 1.22 ms, largest error against exact
+    // sums 0.94 -> 0.34 x 2^-106 sum |a x|; for rows of a few terms a lane,
+    // the sum of renormalised pairs has the smaller one (n = 100: 0.27 and 0.47).
+    constexpr int kTermMerge = 2048;
+    auto merge = [&](Acc& d, const Acc& o) {
+      if constexpr (OP == MSIR_DD) {
+        if (n >= kTermMerge) d.merge_term(o);
+        else d.merge(o);
+      } else {
+        d.merge(o);
+      }
+    };
 #pragma unroll
-    for (int r = 0; r < NR; ++r) acc[r][0].merge(acc[r][1]);
+    for (int r = 0; r < NR; ++r) merge(acc[r][0], acc[r][1]);
 #pragma unroll
     for (int m = 16; m > 0; m >>= 1)
 #pragma unroll
-      for (int r = 0; r < NR; ++r) acc[r][0].merge(acc[r][0].peer(m));
+      for (int r = 0; r < NR; ++r) merge(acc[r][0], acc[r][0].peer(m));
+    Acc mine = acc[0][0];
 #pragma unroll
-    for (int r = 0; r < NR; ++r)
-      if (lane == r && i0 + r < n) epi(i0 + r, a.perm[i0 + r], acc[r][0].fin());
+    for (int r = 1; r < NR; ++r)
+      if (lane == r) mine = acc[r][0];
+    if (lane < NR && i0 + lane < n) epi(i0 + lane, a.perm[i0 + lane], mine.fin());
   }
   cp_async_wait<0>();  // (empty groups: every copy has been waited for)
 }
 
-// All rows: the fewest rows per warp (of 1, 2, 4, 7, 8) that take one round;
-// one at a time in double-double, which the fp64 pipe bounds (n = 8192: 7
-// rounds of one row 1.26 ms, 2 rounds of four 1.47 ms).
+// All rows: the fewest rows per warp (of 1, 2, 4, 7, 8) that take one round.
 template <typename A0, typename X, int OP, typename Epi>
 __device__ __forceinline__ void gemv_rows(Cx& cx, const RefineArgs& a, const X* x, Epi epi) {
   const int nwarps = cx.G * (kRefThreads / 32);
   const int rpw = (cx.n + nwarps - 1) / nwarps;
-  if (rpw <= 1 || OP == MSIR_DD) gemv_rows_n<A0, X, OP, 1>(cx, a, x, epi);
-  else if constexpr (OP == MSIR_DD) return;
+  if (rpw <= 1) gemv_rows_n<A0, X, OP, 1>(cx, a, x, epi);
   else if (rpw <= 2) gemv_rows_n<A0, X, OP, 2>(cx, a, x, epi);
   else if (rpw <= 4) gemv_rows_n<A0, X, OP, 4>(cx, a, x, epi);
   else if (rpw <= 7) gemv_rows_n<A0, X, OP, 7>(cx, a, x, epi);
