@@ -1287,9 +1287,116 @@ __device__ __forceinline__ int team_size(const Cx& cx) {
   return cx.C > 1 ? min(k, cx.C) : k;  // a team stays inside one cluster
 }
 
+// The same solve by a grid of one block (the batched engine) of at most
+// kOneBlocks row blocks: the hand-offs are block barriers and y stays in
+// shared memory, all w_b are formed first, and the tiles stream through one
+// ring over all row blocks.  A row's four threads take alternate 16-byte
+// pieces of it, so that the reads of y fall in different banks.  Bound by
+// the fp64 pipe of its SM in fp64 solves (131k multiply-adds at n = 512: 32
+// of 52 us).  n = 511, forward + backward, fp64: 197 us with a wait on
+// published words and a tile fetched per dependency, 104 us so.
+constexpr int kOneBlocks = 8;
+template <typename ACC, bool LOWER>
+__device__ __noinline__ bool trsv_one(Cx& cx, const RefineArgs& a, int store_fmt) {
+  using V = typename ACC::V;
+  using Tm = typename ACC::Tm;
+  constexpr int EPC = 16 / (int)sizeof(Tm);      // values per 16-byte piece
+  constexpr int NCH = kBlk / EPC / 4;            // pieces per thread and tile
+  constexpr int kTile = kBlk * kBlk * (int)sizeof(Tm);
+  constexpr int kFit = (kPhaseSmem - kTrsvSmem) / kTile, D = kFit < 6 ? kFit : 6;
+  static_assert(D >= 2 && 2 * kOneBlocks * kBlk * sizeof(V) <= kTrsvSmem, "shared scratch");
+  static_assert(NCH * kRefThreads * 16 == kTile, "four threads per row");
+  V* ys = (V*)cx.tsm;                 // c (backward: y of the forward solve), then the solved values
+  V* ws = ys + kOneBlocks * kBlk;
+  uint4* ring = (uint4*)cx.ssm + cx.tid;
+  const Tm* Mat = ACC::mat(a);
+  const double* in_hi = LOWER ? a.c_hi : a.y_hi;
+  const double* in_lo = LOWER ? a.c_lo : a.y_lo;
+  double* out_hi = LOWER ? a.y_hi : a.z_hi;
+  double* out_lo = LOWER ? a.y_lo : a.z_lo;
+  const int n = cx.n, nblk = cx.nblk, rr = cx.tid >> 2, seg = cx.tid & 3, tri = LOWER ? 0 : 1;
+  // row blocks in order q = 0, 1, ..; the q-th has q tiles
+  int iq = 1, it = 0, islot = 0;
+  auto issue = [&]() {
+    if (iq < nblk) {
+      const int row = (LOWER ? iq : nblk - 1 - iq) * kBlk + rr, c0 = (LOWER ? it : nblk - 1 - it) * kBlk;
+#pragma unroll
+      for (int c = 0; c < NCH; ++c) {
+        const int col = c0 + (c * 4 + seg) * EPC;
+        const int valid = row < n ? max(0, min(EPC, n - col)) : 0;
+        cp_async16(ring + (islot * NCH + c) * kRefThreads, Mat + (valid > 0 ? (size_t)row * a.ldf + col : 0),
+                   valid * (int)sizeof(Tm));
+      }
+      if (++it == iq) {
+        it = 0;
+        ++iq;
+      }
+    }
+    islot = islot + 1 == D ? 0 : islot + 1;
+    cp_async_commit();
+  };
+#pragma unroll
+  for (int q = 0; q < D - 1; ++q) issue();
+  __syncthreads();  // c (y) of every row
+  for (int i = cx.tid; i < nblk * kBlk; i += kRefThreads) ys[i] = i < n ? ACC::load(in_hi, in_lo, i) : ACC::zero();
+  __syncthreads();
+#pragma unroll 2
+  for (int b = 0; b < nblk; ++b) {
+    typename ACC::A wa = ACC::azero(), wb = ACC::azero();
+    const size_t inv_row = (((size_t)tri * nblk + b) * kBlk + rr) * kBlk + seg;
+#pragma unroll
+    for (int k = 0; k < 16; k += 2) {
+      wa = ACC::ifma(ACC::inv(a, inv_row + k * 4), ys[b * kBlk + k * 4 + seg], wa);
+      wb = ACC::ifma(ACC::inv(a, inv_row + k * 4 + 4), ys[b * kBlk + k * 4 + 4 + seg], wb);
+    }
+    wa = ACC::merge(wa, wb);
+    wa = ACC::merge(wa, ACC::ax(wa, 1));
+    wa = ACC::merge(wa, ACC::ax(wa, 2));
+    if (seg == 0) ws[b * kBlk + rr] = ACC::fin(wa);
+  }
+  __syncthreads();
+  int slot = 0;
+  for (int q = 0; q < nblk; ++q) {
+    const int b = LOWER ? q : nblk - 1 - q, row = b * kBlk + rr;
+    typename ACC::A acc = ACC::azero(), acc2 = ACC::azero();
+    for (int t = 0; t < q; ++t) {
+      issue();
+      cp_async_wait<D - 1>();
+      const V* y = ys + (LOWER ? t : nblk - 1 - t) * kBlk + seg * EPC;
+      const uint4* src = ring + slot * NCH * kRefThreads;
+      slot = slot + 1 == D ? 0 : slot + 1;
+#pragma unroll
+      for (int c = 0; c < NCH; ++c) {
+        const uint4 u = src[c * kRefThreads];
+        Tm m[EPC];
+        memcpy(m, &u, 16);
+#pragma unroll
+        for (int e = 0; e < EPC; e += 2) {
+          acc = ACC::tfma(m[e], y[c * 4 * EPC + e], acc);
+          acc2 = ACC::tfma(m[e + 1], y[c * 4 * EPC + e + 1], acc2);
+        }
+      }
+    }
+    acc = ACC::merge(acc, acc2);
+    acc = ACC::merge(acc, ACC::ax(acc, 1));
+    acc = ACC::merge(acc, ACC::ax(acc, 2));
+    V y = ACC::store(ACC::wsub(ws[row], acc), store_fmt);
+    if (row >= n) y = ACC::zero();
+    if (seg == 0) {
+      ys[row] = y;
+      if (row < n) ACC::save(out_hi, out_lo, row, y);
+    }
+    __syncthreads();
+  }
+  cp_async_wait<0>();
+  return true;
+}
+
 template <typename F, typename ACC, bool LOWER>
 __device__ __forceinline__ bool trsv(Cx& cx, const RefineArgs& a, int store_fmt) {
   const unsigned epoch = ++cx.epoch;
+  if constexpr (ACC::kW <= 2)
+    if (cx.G == 1 && cx.nblk <= kOneBlocks) return trsv_one<ACC, LOWER>(cx, a, store_fmt);
   const int K = team_size<ACC>(cx);
   if (ACC::kW > 1 && K == 8) return trsv_team<F, ACC, LOWER, 8>(cx, a, store_fmt, epoch);
   if (ACC::kW > 1 && K == 4) return trsv_team<F, ACC, LOWER, 4>(cx, a, store_fmt, epoch);
