@@ -804,14 +804,20 @@ static void fill_args(msir_ctx* ctx, Slot& s, RefineArgs& a, int mode) {
   // deep ring if that fits too.  MSIR_WIDE_MIN overrides the smallest n
   // (tuning only).
   static const int wide_min = env_int("MSIR_WIDE_MIN", kWideMin, kWideMin, 1 << 30);
-  if (mode != MODE_RESIDUAL && j.n >= wide_min && w.D32h) {
+  const bool kept = mode == MODE_APPLY || mode == MODE_PREP;  // (the two agree: one builds what the other uses)
+  if ((mode == MODE_SOLVE || kept) && j.n >= wide_min && w.D32h) {
     a.npad = (int)round_up((size_t)j.n, kSuper);
     a.D32h = w.D32h;
     a.D32l = w.D32l;
     a.D64 = w.D64;
     const size_t room = (size_t)ctx->max_dyn_smem - 1024;
     for (int vb : {4, 8}) {
-      if (vb == 8 && j.n < kWideMin64) break;
+      if (vb == 8 && j.n < (kept ? kWideApply64 : kWideMin64)) break;
+      // An fp32 apply returns the solve's own rounding errors: in superblocks
+      // they are an order of magnitude smaller, i.e. other ones (2e-5 to 4e-5
+      // of the result from n = 3500 on).  What a program has computed with
+      // its factors stays what it was; a refined solution does not show it.
+      if (vb == 4 && kept) continue;
       for (int ring : {kRingDeep, kRingFlat})
         if (refine_smem_bytes(a.kcap, wide_smem(a.npad, s.G, vb, ring)) <= room) {
           a.wide |= vb == 4 ? 1 : 2;
@@ -1427,6 +1433,21 @@ msir_status msir_factor(msir_ctx* ctx, int n, const double* A_dev, int lda, int 
   L.valid = true;
   s.cur = s.try_level;
   if (s.h_flags[2]) { int e = s.h_flags[2]; slot_destroy(s); delete f; return (msir_status)e; }
+  if (L.info == 0 && L.nonfinite == 0) {
+    // the diagonal blocks' inverses belong to the factors that the caller
+    // keeps; an apply builds what its precision needs beside them, once
+    RefineArgs a;
+    fill_args(ctx, s, a, MODE_PREP);
+    RefState st0;
+    memset(&st0, 0, sizeof(st0));
+    cudaMemcpyAsync(s.w.st, &st0, sizeof(st0), cudaMemcpyHostToDevice, s.st);
+    cudaMemsetAsync(s.w.bar, 0, 64, s.st);
+    r = cuda_status(launch_refine(s.u0, L.fmt, a, s.G, s.st));
+    if (r == MSIR_OK) r = cuda_status(cudaStreamSynchronize(s.st));
+    if (r != MSIR_OK) { slot_destroy(s); delete f; return r; }
+    s.w.m_serial = L.serial;
+    s.w.m_ready = RDY_INV;
+  }
   if (info) *info = L.info;
   if (nonfinite) *nonfinite = L.nonfinite;
   *out = f;
@@ -1509,6 +1530,8 @@ msir_status msir_factors_apply(msir_ctx* ctx, const msir_factors* fc, int nrhs, 
   CK(cudaMemsetAsync(s.w.ll, 0, ll_bytes(n), s.st));
   RefState st0;
   memset(&st0, 0, sizeof(st0));
+  // inverses and scaled blocks are the factors', built once per handle
+  if (s.w.m_serial == s.lv[s.cur].serial) st0.mready = s.w.m_ready;
   for (int c = 0; c < nrhs; ++c) {
     RefineArgs a;
     fill_args(ctx, s, a, MODE_APPLY);
@@ -1517,21 +1540,20 @@ msir_status msir_factors_apply(msir_ctx* ctx, const msir_factors* fc, int nrhs, 
     a.ap_in = B_dev + (size_t)c * ldb;
     a.ap_out = X_dev + (size_t)c * ldx;
     st0.epoch = (unsigned)(2 * c);
-    if (s.w.m_serial != s.lv[s.cur].serial) {
-      st0.mready = 0;
-      s.w.m_serial = s.lv[s.cur].serial;
-    }
     CK(cudaMemcpyAsync(s.w.st, &st0, sizeof(st0), cudaMemcpyHostToDevice, s.st));
     CK(cudaMemsetAsync(s.w.bar, 0, 64, s.st));
     CK(launch_refine(s.u0, s.lv[s.cur].fmt, a, s.G, s.st));
     CK(cudaStreamSynchronize(s.st));
     RefState back;
     CK(cudaMemcpy(&back, s.w.st, sizeof(back), cudaMemcpyDeviceToHost));
-    st0.mready = back.mready;  // scaled blocks built by this launch stay valid
+    st0.mready = back.mready;  // blocks built by this launch stay valid
+    if (back.phase == PH_ERROR) st0.mready = 0;
   }
   int flags[16];
   CK(cudaMemcpy(flags, s.w.iflags, sizeof(flags), cudaMemcpyDeviceToHost));
   if (flags[2]) return (msir_status)flags[2];
+  s.w.m_serial = s.lv[s.cur].serial;
+  s.w.m_ready = st0.mready;
   return MSIR_OK;
 }
 

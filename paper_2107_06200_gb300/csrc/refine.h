@@ -65,6 +65,10 @@ enum ReadyBits : unsigned {
 constexpr int kSuper = 512;
 constexpr int kWideMin = 1024;
 constexpr int kWideMin64 = 1792;
+// Smallest matrix whose factors' fp64 applies are wide: below, the first
+// apply of a handle would pay more for the superblocks (n = 2000: 1.1 ms)
+// than for the scaled blocks (0.7 ms); n = 5000: 2.4 and 3.7 ms.
+constexpr int kWideApply64 = 3072;
 constexpr int kRingDeep = 16, kRingFlat = 8;  // steps of the ring of factor values
 // Shared memory of a wide solve in values of `vbytes` on a grid of G CTAs:
 // y of every row, z of a superblock (high and low words), partial sums; then
@@ -77,7 +81,9 @@ constexpr size_t wide_smem(int npad, int G, int vbytes, int ring) {
   return wide_ring_off(npad, G, vbytes) + (size_t)ring * kRefThreads * 16;
 }
 
-enum RefMode { MODE_SOLVE = 0, MODE_APPLY = 1, MODE_RESIDUAL = 2 };
+// MODE_PREP: the double-double inverses of the diagonal blocks alone (a
+// factorisation that is handed out)
+enum RefMode { MODE_SOLVE = 0, MODE_APPLY = 1, MODE_RESIDUAL = 2, MODE_PREP = 3 };
 enum RefPhase {
   PH_START = 0,      // compute x0, then refine
   PH_ESCALATED = 1,  // factors replaced by a finer u_f: recompute r, start SIR

@@ -1423,7 +1423,7 @@ __device__ __forceinline__ bool trsv(Cx& cx, const RefineArgs& a, int store_fmt)
 // to 17 times; fp64: up to 12 times).
 //
 // Measured (forward + backward, alone on the GPU): n = 2000 94 -> 42 us
-// (fp32), 112 -> 64 us (fp64); n = 8192 390 -> 270 us (fp32), 740 -> 480 us
+// (fp32), 112 -> 49 us (fp64); n = 8192 390 -> 200 us (fp32), 740 -> 350 us
 // (fp64).  What bounds it now: two hand-offs of about 1 us per superblock
 // (an L2 round trip alone is 0.4 us) and, at n = 8192, the compensated sums
 // of the far products.
@@ -3109,6 +3109,9 @@ __global__ void __launch_bounds__(kRefThreads, 1) refine_kernel(RefineArgs a) {
     double s = 0.0, xn = 0.0;
     ok = grid_barrier(cx, a) && residual<A0>(cx, a, a.x, a.ap_arith, s, xn);
     if (ok && cx.cta == 0 && cx.tid == 0) *a.res_s = s;
+  } else if (a.mode == MODE_PREP) {
+    ok = build_inverses<F>(cx, a, true, false);
+    cx.mready |= RDY_INV;
   } else if (a.mode == MODE_APPLY) {
     for (int b = cx.cta; b < cx.nblk; b += cx.G)
       for (int i = b * kBlk + cx.tid; i < min((b + 1) * kBlk, cx.n); i += kRefThreads) {

@@ -79,3 +79,26 @@ def test_wide_solve_edges(ctx, n, uf):
     A, _, _ = randsvd_system(n, 1e3, 50 + n)
     u = OF.FP64 if uf in (OF.FP32, OF.FP64) else OF.FP32
     _check(ctx, A, u, uf, [(OF.FP32, OF.FP32), (OF.FP64, OF.FP64), (OF.FP32, OF.FP16)])
+
+
+@pytest.mark.parametrize("n", [3071, 3072, 3073, 3585])
+def test_wide_apply_edges(ctx, n):
+    """fp64 applies around the smallest size of the superblock solves, with a
+    last superblock of one row and of all but one."""
+    A, _, _ = randsvd_system(n, 1e3, 50 + n)
+    _check(ctx, A, OF.FP32, OF.FP16, [(OF.FP64, OF.FP64)])
+
+
+@pytest.mark.parametrize("n", [1023, 1024, 1025, 1535, 1793])
+def test_wide_refinement_edges(ctx, n):
+    """Solves around the smallest sizes of the fp32 superblock solves: the
+    refinement stops when its correction is below u = 2^-24, so the backward
+    error is at most 4 u."""
+    A, _, _ = randsvd_system(n, 1e2, 60 + n)
+    A = A.astype(np.float32).astype(np.float64)
+    b = (A @ np.random.default_rng(n).standard_normal(n)).astype(np.float32).astype(np.float64)
+    X, reps, st = ctx.solve(to_dev(A), to_dev(b), "fp16,fp32,fp64")
+    x = X.cpu().numpy().reshape(-1)
+    r = np.abs(b - A @ x).max()
+    assert st == 0
+    assert r <= 4 * 2.0 ** -24 * (np.abs(A).sum(1).max() * np.abs(x).max() + np.abs(b).max())
