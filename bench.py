@@ -333,7 +333,8 @@ def engine_fp64_flops(rep, n):
     diagonal blocks (64^3/6 compensated terms of about 11 fp64 operations
     each) and the fp64 scaled blocks (64 fused multiply-adds per element of
     the n^2 off-diagonal part, 2 flops each); then the refinement's fp64
-    work (refine_fp64_flops)."""
+    work (refine_fp64_flops).  An upper count: a factorisation whose solves
+    all run in fp32 builds its inverses and scaled blocks on the fp32 pipe."""
     nf = max(1, rep["n_factorizations"])
     nblk = -(-n // 64)
     inv = 2 * nblk * (64 ** 3 / 6.0) * 11.0
@@ -355,7 +356,7 @@ def engine_roofline(reps, ns, dur_s):
     return {"bound": "alu", "pipe": "fp64", "achieved": ach64, "peak": pk64, "unit": "TFLOP/s", "frac": ach64 / pk64,
             "peak_source": "measured (msir_probe_fma_rate, fp64 fma chains on every SM)",
             "kernel": "batched_solve_kernel (batched engine, one launch per step)",
-            "work": "fp64-pipe flops as executed: dd diagonal-block inverses, fp64 scaled blocks, refinement",
+            "work": "fp64-pipe flops (upper count): dd diagonal-block inverses, fp64 scaled blocks, refinement",
             "fp32": {"achieved": ach32, "peak": pk32, "unit": "TFLOP/s", "frac": ach32 / pk32,
                      "work": "2/3 n^3 per fp32-pipe factorisation + 4 n^2 per GMRES iteration or step + 8 n k"},
             "traffic": None, "traffic_unit": "bytes per launch (ncu)", "concurrency": 1.0}
