@@ -178,6 +178,14 @@ __device__ __forceinline__ void gemv_rows_n(Cx& cx, const RefineArgs& a, const X
   static_assert(VC * sizeof(X) >= 16, "a lane's x fills whole pieces");
   static_assert(2 * UNIT * 16 <= kPhaseSmem, "the scratch holds two steps");
   using Acc = RowAcc<OP>;
+  // fp64 sums on fp32 rows with an fp64 vector (the residual): one sum per
+  // lane, columns ascending, the columns past the last multiple of 4 one per
+  // lane at the end.  A residual is what its sums leave after cancellation,
+  // so their order shows in it (1e-9 of it); with several rows per warp it
+  // costs nothing on the fp64 pipe, which bounds this product.
+  constexpr bool kAscending = OP == MSIR_FP64 && sizeof(A0) == 4 && sizeof(X) == 8;
+  constexpr int kOdd = kAscending ? 0 : 1;
+  const int nv = kAscending ? cx.n & ~3 : cx.n;  // columns of the steps
   const A0* A = (const A0*)a.A;
   const int n = cx.n, lane = cx.lane, nwarps = cx.G * (kRefThreads / 32), gw = cx.cta * (kRefThreads / 32) + cx.warp;
   const int depth = min(4, a.scratch / (UNIT * 16));     // 2, 3 or 4
@@ -191,19 +199,19 @@ __device__ __forceinline__ void gemv_rows_n(Cx& cx, const RefineArgs& a, const X
     // each warp starts at columns of its own and wraps around: in step, the
     // warps would all read the same few lines of x at once, and the L2 slices
     // that hold them would serve one after another
-    int ist = (int)((long long)gw * nsteps / nwarps), islot = 0;
+    int ist = kAscending ? 0 : (int)((long long)gw * nsteps / nwarps), islot = 0;
     auto issue = [&](int st) {
       if (st < nsteps) {
         const int col = ist * STEP + lane * VC;
         ist = ist + 1 == nsteps ? 0 : ist + 1;
-        const int valid = min(VC, max(0, n - col)), c = valid > 0 ? col : 0;  // zeros past n
+        const int valid = min(VC, max(0, nv - col)), c = valid > 0 ? col : 0;  // zeros past nv
         uint4* dst = ring + islot * UNIT;
 #pragma unroll
         for (int r = 0; r < NR; ++r) cp_async16(dst + r * kRefThreads, row[r] + c, valid * (int)sizeof(A0));
 #pragma unroll
         for (int q = 0; q < XS; ++q) {
           constexpr int XC = 16 / (int)sizeof(X);
-          const int xc = col + q * XC, xv = min(XC, max(0, n - xc));
+          const int xc = col + q * XC, xv = min(XC, max(0, nv - xc));
           cp_async16(dst + (NR + q) * kRefThreads, x + (xv > 0 ? xc : 0), xv * (int)sizeof(X));
         }
       }
@@ -251,19 +259,26 @@ __device__ __forceinline__ void gemv_rows_n(Cx& cx, const RefineArgs& a, const X
 #pragma unroll
           for (int q = 0; q < VC; ++q)
 #pragma unroll
-            for (int r = 0; r < NR; ++r) acc[r][q & 1].add((double)av[r][q], (double)xv[q]);
+            for (int r = 0; r < NR; ++r) acc[r][q & kOdd].add((double)av[r][q], (double)xv[q]);
         } else {
 #pragma unroll
           for (int q = 0; q < VC; ++q)
 #pragma unroll
-            for (int r = 0; r < NR; ++r) acc[r][q & 1].add(widen_normal(av[r][q]), xd[q]);
+            for (int r = 0; r < NR; ++r) acc[r][q & kOdd].add(widen_normal(av[r][q]), xd[q]);
         }
       } else {
 #pragma unroll
         for (int q = 0; q < VC; ++q)
 #pragma unroll
-          for (int r = 0; r < NR; ++r) acc[r][q & 1].add(av[r][q], xv[q]);
+          for (int r = 0; r < NR; ++r) acc[r][q & kOdd].add(av[r][q], xv[q]);
       }
+    }
+    if constexpr (kAscending) {
+      if (nv + lane < n) {
+#pragma unroll
+        for (int r = 0; r < NR; ++r) acc[r][0].add((double)row[r][nv + lane], (double)__ldcg(x + nv + lane));
+      }
+      __syncwarp();
     }
     // Double-double: a lane's sums as terms of the row's from kTermMerge
     // columns on.  n = 8192: 1.29 -> 1.22 ms, largest error against exact
@@ -279,7 +294,8 @@ __device__ __forceinline__ void gemv_rows_n(Cx& cx, const RefineArgs& a, const X
       }
     };
 #pragma unroll
-    for (int r = 0; r < NR; ++r) merge(acc[r][0], acc[r][1]);
+    for (int r = 0; r < NR; ++r)
+      if (kOdd) merge(acc[r][0], acc[r][1]);
 #pragma unroll
     for (int m = 16; m > 0; m >>= 1)
 #pragma unroll
