@@ -805,19 +805,23 @@ static void fill_args(msir_ctx* ctx, Slot& s, RefineArgs& a, int mode) {
   // (tuning only).
   static const int wide_min = env_int("MSIR_WIDE_MIN", kWideMin, kWideMin, 1 << 30);
   const bool kept = mode == MODE_APPLY || mode == MODE_PREP;  // (the two agree: one builds what the other uses)
-  if ((mode == MODE_SOLVE || kept) && j.n >= wide_min && w.D32h) {
+  // MSIR_WIDE_APPLY=1: applies take the wide solves wherever a solve does,
+  // 0: never (tests of the two routes against each other)
+  const int wide_env = env_int("MSIR_WIDE_APPLY", -1, 0, 1);
+  const bool wide_apply = wide_env == 1;
+  if ((mode == MODE_SOLVE || (kept && wide_env != 0)) && j.n >= wide_min && w.D32h) {
     a.npad = (int)round_up((size_t)j.n, kSuper);
     a.D32h = w.D32h;
     a.D32l = w.D32l;
     a.D64 = w.D64;
     const size_t room = (size_t)ctx->max_dyn_smem - 1024;
     for (int vb : {4, 8}) {
-      if (vb == 8 && j.n < (kept ? kWideApply64 : kWideMin64)) break;
+      if (vb == 8 && j.n < (kept && !wide_apply ? kWideApply64 : kWideMin64)) break;
       // An fp32 apply returns the solve's own rounding errors: in superblocks
       // they are an order of magnitude smaller, i.e. other ones (2e-5 to 4e-5
       // of the result from n = 3500 on).  What a program has computed with
       // its factors stays what it was; a refined solution does not show it.
-      if (vb == 4 && kept) continue;
+      if (vb == 4 && kept && !wide_apply) continue;
       for (int ring : {kRingDeep, kRingFlat})
         if (refine_smem_bytes(a.kcap, wide_smem(a.npad, s.G, vb, ring)) <= room) {
           a.wide |= vb == 4 ? 1 : 2;
