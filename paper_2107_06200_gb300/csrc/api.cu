@@ -216,6 +216,8 @@ struct Workspace {
   float* D32h = nullptr;
   float* D32l = nullptr;
   double* D64 = nullptr;
+  float* wrow = nullptr;     // their rows' sums and diagonals, wflag after them
+  int* wflag = nullptr;
   // the factorisation whose inverses and scaled blocks these are (-1: none),
   // and which of them are built (ReadyBits); a new allocation holds none
   int m_serial = -1;
@@ -288,9 +290,12 @@ static size_t ws_layout(Workspace& w, int n, int kcap, int G, bool alloc_f64_lev
     w.D32h = (float*)take(nd * 4);
     w.D32l = (float*)take(nd * 4);
     w.D64 = (double*)take(nd * 8);
+    w.wrow = (float*)take(4 * round_up((size_t)n, kSuper) * 4);
+    w.wflag = (int*)take(64);
   } else {
-    w.D32h = w.D32l = nullptr;
+    w.D32h = w.D32l = w.wrow = nullptr;
     w.D64 = nullptr;
+    w.wflag = nullptr;
   }
   w.bar = (unsigned*)take(64);
   w.st = (RefState*)take(sizeof(RefState));
@@ -814,6 +819,8 @@ static void fill_args(msir_ctx* ctx, Slot& s, RefineArgs& a, int mode) {
     a.D32h = w.D32h;
     a.D32l = w.D32l;
     a.D64 = w.D64;
+    a.wrow = w.wrow;
+    a.wflag = w.wflag;
     const size_t room = (size_t)ctx->max_dyn_smem - 1024;
     for (int vb : {4, 8}) {
       if (vb == 8 && j.n < (kept && !wide_apply ? kWideApply64 : kWideMin64)) break;

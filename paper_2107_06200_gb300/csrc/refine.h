@@ -53,7 +53,8 @@ enum ReadyBits : unsigned {
   RDY_M64 = 4u,  // fp64 scaled blocks
   RDY_INV = 8u,  // inv_hi, inv_lo
   RDY_W32 = 16u, // fp32-pair inverses of the diagonal superblocks
-  RDY_W64 = 32u  // fp64 ones
+  RDY_W64 = 32u, // fp64 ones
+  RDY_NO32 = 64u // fp32 pairs do not hold these superblocks' inverses: 64-row solves
 };
 
 // Wide solves (refine_impl.cuh): rows of a superblock, and the smallest
@@ -69,6 +70,14 @@ constexpr int kWideMin64 = 1792;
 // apply of a handle would pay more for the superblocks (n = 2000: 1.1 ms)
 // than for the scaled blocks (0.7 ms); n = 5000: 2.4 and 3.7 ms.
 constexpr int kWideApply64 = 3072;
+// A superblock's inverse is formed in fp32 pairs (2^-46 an operation) only if
+// its row sums and diagonal lie within 2^+-60 of 1 and of each other, so that
+// no product or error term of the doubling leaves fp32's range, and its
+// Skeel condition number max_i (|X||T|e)_i is at most kWideCond: the pair's
+// error, some 2^-46 of it, then stays below an fp32 rounding.  (LU factors of
+// randsvd matrices, kappa 1e2 .. 1e8, plain and with rows graded by
+// 10^+-4: at most 4.7e4.)
+constexpr float kWideRange = 0x1p60f, kWideCond = 0x1p20f;
 constexpr int kRingDeep = 16, kRingFlat = 8;  // steps of the ring of factor values
 // Shared memory of a wide solve in values of `vbytes` on a grid of G CTAs:
 // y of every row, z of a superblock (high and low words), partial sums; then
@@ -174,6 +183,10 @@ struct RefineArgs {
   float* D32h;
   float* D32l;
   double* D64;
+  // of the triangles' rows within their superblock: sum of magnitudes, then
+  // the diagonal's magnitude, [2][npad] each; what build_wide found (0: safe)
+  float* wrow;
+  int* wflag;
   unsigned* bar;           // grid barrier counter (zeroed before launch)
   int* err;
   RefState* st;

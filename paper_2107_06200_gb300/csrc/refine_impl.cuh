@@ -1540,6 +1540,57 @@ __device__ __forceinline__ void wide_tile_mma(const double* A, const double* B, 
   }
 }
 
+// Row sums of magnitudes and diagonals of the triangles within their
+// superblocks (a warp per row; fp32 is enough for the test below).
+template <typename F>
+__device__ __forceinline__ void wide_rows(Cx& cx, const RefineArgs& a) {
+  const int n = cx.n, nw = cx.G * (kRefThreads / 32);
+  if (cx.cta == 0 && cx.tid == 0) *a.wflag = 0;
+  for (int q = cx.cta * (kRefThreads / 32) + cx.warp; q < 2 * n; q += nw) {
+    const bool lower = q < n;
+    const int r = lower ? q : q - n, s0 = r / kSuper * kSuper;
+    const int c0 = lower ? s0 : r, c1 = lower ? r : min(s0 + kSuper, n);
+    float s = 0.0f;
+    for (int c = c0 + cx.lane; c < c1; c += 32) s += fabsf((float)factor_at<F>(a, (size_t)r * a.ldf + c));
+    s = warp_sum_f(s);
+    if (cx.lane == 0) {
+      a.wrow[(size_t)(lower ? 0 : 1) * a.npad + r] = lower ? s + 1.0f : s;
+      a.wrow[(size_t)(lower ? 2 : 3) * a.npad + r] = lower ? 1.0f : fabsf((float)factor_at<F>(a, (size_t)r * a.ldf + r));
+    }
+  }
+}
+// Whether the superblocks' inverses are safe in fp32 pairs (kWideRange,
+// kWideCond): sets *wflag if not, a warp per row.  The products of a row i
+// are X_ik T_kj with k between i and j, of the size of R_k / R_j where R are
+// the rows' scales; out of range they overflow or vanish although X itself
+// does not.
+static __device__ __noinline__ void wide_check(Cx& cx, const RefineArgs& a) {
+  const int n = cx.n, nw = cx.G * (kRefThreads / 32);
+  for (int q = cx.cta * (kRefThreads / 32) + cx.warp; q < 2 * n; q += nw) {
+    const bool lower = q < n;
+    const int r = lower ? q : q - n, s0 = r / kSuper * kSuper, tri = lower ? 0 : 1;
+    const float* sum = a.wrow + (size_t)tri * a.npad;
+    const float* dia = a.wrow + (size_t)(2 + tri) * a.npad;
+    const float* x = a.D32h + wide_row(a, tri, r) - s0;
+    const int c0 = lower ? s0 : r, c1 = lower ? r + 1 : min(s0 + kSuper, n);
+    float v = 0.0f, mx = 0.0f, mn = kWideRange;
+    for (int c = c0 + cx.lane; c < c1; c += 32) {
+      const float s = __ldcg(sum + c);
+      v += fabsf(__ldcg(x + c)) * s;
+      mx = fmaxf(mx, s);
+      mn = fminf(mn, __ldcg(dia + c));
+    }
+    v = warp_sum_f(v);
+#pragma unroll
+    for (int m = 16; m > 0; m >>= 1) {
+      mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, m));
+      mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, m));
+    }
+    const bool safe = v <= kWideCond && mx <= kWideRange && mn >= 1.0f / kWideRange && mx <= mn * kWideRange;
+    if (cx.lane == 0 && !safe) atomicOr(a.wflag, 1);
+  }
+}
+
 // Inverses of the diagonal superblocks from those of the 64x64 blocks
 // (build_inverses has put them on the diagonal), by doubling h = 64, 128, ..:
 //   L: X21 = -X22 (L21 X11)     U: X12 = -X11 (U12 X22)
@@ -1558,6 +1609,7 @@ __device__ __noinline__ bool build_wide(Cx& cx, const RefineArgs& a) {
   constexpr int sb = kSuper;
   const int n = cx.n, ldf = a.ldf;
   const int i0 = (cx.tid >> 4) * 4, j0 = (cx.tid & 15) * 4;
+  if (kF32) wide_rows<F>(cx, a);  // (read behind the barriers of the doubling)
   for (int h = kBlk; h < sb; h *= 2) {
     const int nt = h / kBlk, npair = (a.npad / 2) / h;
     for (int pass = 0; pass < 2; ++pass) {
@@ -1637,6 +1689,13 @@ __device__ __noinline__ bool build_wide(Cx& cx, const RefineArgs& a) {
       if (!grid_barrier(cx, a)) return false;
     }
   }
+  if (!kF32) {
+    cx.mready |= RDY_W64;
+    return true;
+  }
+  wide_check(cx, a);
+  if (!grid_barrier(cx, a)) return false;
+  cx.mready |= __ldcg(a.wflag) ? RDY_NO32 : RDY_W32;
   return true;
 }
 
@@ -2135,22 +2194,23 @@ __device__ bool msolve(Cx& cx, const RefineArgs& a, int store_fmt, bool synced) 
     if constexpr (!std::is_same<F, FAny>::value && ACC::kW <= 2) {
       constexpr bool k32 = ACC::kW == 1;
       const unsigned need = k32 ? RDY_W32 : RDY_W64;
-      if (!(cx.mready & need)) {
+      if (!(cx.mready & (need | (k32 ? RDY_NO32 : 0u)))) {
         if (k32 || !(cx.mready & RDY_INV)) {
           if (!build_inverses<F>(cx, a, !k32, true)) return false;
           if (!k32) cx.mready |= RDY_INV;
         }
         if (!build_wide<F, k32>(cx, a)) return false;
-        cx.mready |= need;
       }
-      if (!synced && !grid_barrier(cx, a)) return false;
-      {
-        PhaseTimer pt(cx, 1);
-        if (!trsv_wide_any<F, ACC, true>(cx, a, store_fmt)) return false;
+      if (cx.mready & need) {
+        if (!synced && !grid_barrier(cx, a)) return false;
+        {
+          PhaseTimer pt(cx, 1);
+          if (!trsv_wide_any<F, ACC, true>(cx, a, store_fmt)) return false;
+        }
+        PhaseTimer pt(cx, 2);
+        if (!trsv_wide_any<F, ACC, false>(cx, a, store_fmt)) return false;
+        return synced || grid_barrier(cx, a);
       }
-      PhaseTimer pt(cx, 2);
-      if (!trsv_wide_any<F, ACC, false>(cx, a, store_fmt)) return false;
-      return synced || grid_barrier(cx, a);
     }
   }
   // inverses and scaled blocks of the current factors in this precision, once

@@ -57,3 +57,31 @@ def test_fp32_error_is_below_the_64_row_route(ctx, monkeypatch, n, kappa, graded
     A, B = system(n, kappa, graded)
     ew, e64 = route_errors(ctx, monkeypatch, A, B, OF.FP32, uf, OF.FP32)
     assert np.all(ew <= e64), (ew / e64)
+
+
+@pytest.mark.parametrize("n", [1024, 1500])
+@pytest.mark.parametrize("lo,hi", [(90, -60), (-60, 90), (10, -10)])
+def test_rows_that_leave_the_range_of_a_superblock(ctx, monkeypatch, n, lo, hi):
+    """A = D T with T well conditioned and upper triangular, D powers of two
+    that fall or rise by 2^150 within one superblock (and by 2^20, which the
+    pairs hold): the products behind a superblock's inverse overflow or
+    vanish, the solve does not.  A scaling by rows changes no rounding of the
+    64-row solve, so T's bound holds: 2 (n u + u) cond(T, x) |x|_inf."""
+    import paper_2107_06200_gb300 as M
+    from gpu_helpers import cond_comp
+    monkeypatch.setenv("MSIR_WIDE_APPLY", "1")
+    rng = np.random.default_rng(n)
+    T = np.eye(n) + np.triu(rng.uniform(-1, 1, (n, n)), 1) / np.sqrt(n)
+    T = T.astype(np.float32).astype(np.float64)
+    e = np.full(n, float(hi))
+    e[:512] = np.round(np.linspace(lo, hi, 512))
+    A = T * 2.0 ** e[:, None]
+    x = rng.standard_normal(n)
+    c = (A @ x).astype(np.float32).astype(np.float64)
+    f = ctx.factor(to_dev(A), OF.FP32, OF.FP32, M.params_default())
+    assert f.info == 0 and f.nonfinite == 0
+    got = f.apply(to_dev(c), OF.FP32, OF.FP32).cpu().numpy()[:, 0]
+    f.close()
+    ref = np.linalg.solve(T, c * 2.0 ** -e)
+    u = 2.0 ** -24
+    assert np.max(np.abs(got - ref)) <= 2 * (n * u + u) * cond_comp(T, ref) * np.max(np.abs(ref))
