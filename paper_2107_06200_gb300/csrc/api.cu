@@ -809,7 +809,7 @@ static void fill_args(msir_ctx* ctx, Slot& s, RefineArgs& a, int mode) {
   // deep ring if that fits too.  MSIR_WIDE_MIN overrides the smallest n
   // (tuning only).
   static const int wide_min = env_int("MSIR_WIDE_MIN", kWideMin, kWideMin, 1 << 30);
-  const bool kept = mode == MODE_APPLY || mode == MODE_PREP;  // (the two agree: one builds what the other uses)
+  const bool kept = mode == MODE_APPLY;
   // MSIR_WIDE_APPLY=1: applies take the wide solves wherever a solve does,
   // 0: never (tests of the two routes against each other)
   const int wide_env = env_int("MSIR_WIDE_APPLY", -1, 0, 1);

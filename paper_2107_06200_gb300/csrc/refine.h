@@ -54,30 +54,36 @@ enum ReadyBits : unsigned {
   RDY_INV = 8u,  // inv_hi, inv_lo
   RDY_W32 = 16u, // fp32-pair inverses of the diagonal superblocks
   RDY_W64 = 32u, // fp64 ones
-  RDY_NO32 = 64u // fp32 pairs do not hold these superblocks' inverses: 64-row solves
+  RDY_NO32 = 64u, // fp32 pairs do not hold these superblocks' inverses: 64-row solves
+  RDY_NO64 = 128u // nor the fp64 ones made from them
 };
 
 // Wide solves (refine_impl.cuh): rows of a superblock, and the smallest
 // matrices that take them.  fp32: from two superblocks on (n = 1024 .. 2000:
-// 20-40 us for a pair of solves against 45-95).  fp64: from 1792 rows on;
-// below, the error of a solve was up to 1.2 times that of the 64-row solve
-// (n = 1500, kappa = 1e2: 5.0e-13 against 4.1e-13 of |x|), above it is
-// smaller (n = 2000 .. 5000: 0.97 to 0.08 times).
+// 20-40 us for a pair of solves against 45-95).  fp64: from 1792 rows on
+// (n = 2000: 49 us against 112; below, the superblocks' construction, 1 ms,
+// takes the solves of a short run to earn).  Errors against double-double
+// solves, mean over n = 1300 .. 7237 and kappa = 1e2 .. 1e8, relative to the
+// 64-row solves': fp32 0.08 (right-hand sides A x) and 0.09 (random ones),
+// fp64 0.14 and 0.27.
 constexpr int kSuper = 512;
 constexpr int kWideMin = 1024;
 constexpr int kWideMin64 = 1792;
 // Smallest matrix whose factors' fp64 applies are wide: below, the first
 // apply of a handle would pay more for the superblocks (n = 2000: 1.1 ms)
-// than for the scaled blocks (0.7 ms); n = 5000: 2.4 and 3.7 ms.
+// than for the scaled blocks (0.7 ms); n = 5000: 2.7 and 3.7 ms.
 constexpr int kWideApply64 = 3072;
 // A superblock's inverse is formed in fp32 pairs (2^-46 an operation) only if
 // its row sums and diagonal lie within 2^+-60 of 1 and of each other, so that
 // no product or error term of the doubling leaves fp32's range, and its
 // Skeel condition number max_i (|X||T|e)_i is at most kWideCond: the pair's
-// error, some 2^-46 of it, then stays below an fp32 rounding.  (LU factors of
-// randsvd matrices, kappa 1e2 .. 1e8, plain and with rows graded by
-// 10^+-4: at most 4.7e4.)
-constexpr float kWideRange = 0x1p60f, kWideCond = 0x1p20f;
+// error is some 2^-46 of it.  (LU factors of randsvd matrices, kappa 1e2 ..
+// 1e8, plain and with rows graded by 10^+-4, stay below 4.7e4; random
+// triangles of 2^18 gave one solve of four 1.17 times the error of the
+// 64-row one.)
+// kWideResid: the largest scaled residual of a pair that one Newton step
+// takes to fp64 (build_wide64).
+constexpr float kWideRange = 0x1p60f, kWideCond = 0x1p17f, kWideResid = 0x1p-32f;
 constexpr int kRingDeep = 16, kRingFlat = 8;  // steps of the ring of factor values
 // Shared memory of a wide solve in values of `vbytes` on a grid of G CTAs:
 // y of every row, z of a superblock (high and low words), partial sums; then
@@ -184,7 +190,8 @@ struct RefineArgs {
   float* D32l;
   double* D64;
   // of the triangles' rows within their superblock: sum of magnitudes, then
-  // the diagonal's magnitude, [2][npad] each; what build_wide found (0: safe)
+  // the diagonal's magnitude, [2][npad] each; what build_wide and
+  // build_wide64 found (0: safe)
   float* wrow;
   int* wflag;
   unsigned* bar;           // grid barrier counter (zeroed before launch)

@@ -817,8 +817,7 @@ __device__ __forceinline__ size_t wide_row(const RefineArgs& a, int tri, int r) 
 // Inverses of the diagonal blocks of L and U by all CTAs of the grid, once
 // per factorisation: as fp32 pairs (dd = false; inv32, inv32l) or in
 // double-double (inv_hi, inv_lo, and for fp64 factors inv32, inv32l too);
-// `wide`: the fp32 pairs go into the superblocks' array (the fp64 ones
-// always go there too).  An
+// `wide`: the fp32 pairs go into the superblocks' array.  An
 // fp32 pair keeps its 2^-46 as long as the block's diagonal is far from
 // fp32's range ends; other blocks take the double-double arithmetic.
 template <typename F>
@@ -847,8 +846,8 @@ __device__ __noinline__ bool build_inverses(Cx& cx, const RefineArgs& a, bool dd
     const size_t base = ((size_t)(lower ? 0 : 1) * cx.nblk + b) * kBlk * kBlk;
     const int nr = min(kBlk, cx.n - b * kBlk);
     // for wide solves the blocks go on the diagonals of the superblocks
-    const size_t wbase = a.wide ? wide_row(a, lower ? 0 : 1, b * kBlk) + (b * kBlk) % kSuper : 0;
-    const bool w32 = wide && !dd, w64 = (a.wide & 2) != 0;
+    const size_t wbase = wide ? wide_row(a, lower ? 0 : 1, b * kBlk) + (b * kBlk) % kSuper : 0;
+    const bool w32 = wide && !dd;
     float* o32h = w32 ? a.D32h + wbase : a.inv32 + base;
     float* o32l = w32 ? a.D32l + wbase : a.inv32l + base;
     const int ld32 = w32 ? kSuper : kBlk;
@@ -860,7 +859,6 @@ __device__ __noinline__ bool build_inverses(Cx& cx, const RefineArgs& a, bool dd
         if (dd) {
           a.inv_hi[base + e] = h;
           a.inv_lo[base + e] = l;
-          if (w64) a.D64[wbase + (size_t)i * kSuper + k] = h;
         }
         if (want32) {
           const float r = dd_to_f32(h, l);
@@ -1434,9 +1432,9 @@ __device__ __forceinline__ bool trsv(Cx& cx, const RefineArgs& a, int store_fmt)
 //
 // Rounding: the inverse of a diagonal superblock and z are kept as pairs in
 // fp32 solves (sums compensated), so the only fp32-sized error of a
-// component is its final rounding; fp64 solves use fp64 throughout.
-// Against the 64-row solve the error is smaller (fp32, n = 2000 .. 5000: 10
-// to 17 times; fp64: up to 12 times).
+// component is its final rounding.  fp64 solves use fp64 values: the inverse
+// is the exact one rounded (build_wide64), so that a solve's error stays
+// within |X||T||y| 2^-53 as on the 64-row route (figures: see kWideMin64).
 //
 // Measured (forward + backward, alone on the GPU): n = 2000 94 -> 42 us
 // (fp32), 112 -> 49 us (fp64); n = 8192 390 -> 200 us (fp32), 740 -> 350 us
@@ -1494,16 +1492,16 @@ __device__ __forceinline__ void lds4(const double* p, double (&v)[4]) {
 
 template <typename ACC, typename F>
 __device__ __forceinline__ bool use_wide(const RefineArgs& a) {
-  if constexpr (std::is_same<F, FAny>::value || ACC::kW == 4) return false;
-  else if constexpr (ACC::kW == 1) return (a.wide & 1) && !std::is_same<F, double>::value;
-  else return (a.wide & 2) != 0;
+  // (fp64 factors are not exact in the fp32 words of the inverses)
+  if constexpr (std::is_same<F, FAny>::value || std::is_same<F, double>::value || ACC::kW == 4) return false;
+  else return (a.wide & (ACC::kW == 1 ? 1 : 2)) != 0;
 }
 
 // Products of 64x64 tiles for the doubling of the superblock inverses: acc
 // (4 x 4 per thread: rows 4 (tid / 16) .., columns 4 (tid % 16) ..) +=
-// A B over 64 inner terms; A staged transposed ([k][i]), B as [k][j].
+// A B over 64 inner terms; A staged transposed ([k][i]), B as [k][j].  fp32
+// pairs; A values or pairs (kPairA).
 constexpr int kWtLd = kBlk + 4;
-// fp32 pairs: A values or pairs (Al null: values)
 template <bool kPairA>
 __device__ __forceinline__ void wide_tile_mma(const float* Ah, const float* Al, const float* Bh, const float* Bl,
                                               int i0, int j0, ff_t (&acc)[4][4]) {
@@ -1524,28 +1522,13 @@ __device__ __forceinline__ void wide_tile_mma(const float* Ah, const float* Al, 
       }
   }
 }
-__device__ __forceinline__ void wide_tile_mma(const double* A, const double* B, int i0, int j0, double (&acc)[4][4]) {
-#pragma unroll 2
-  for (int k = 0; k < kBlk; ++k) {
-    double a4[4], b4[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      a4[q] = A[k * kWtLd + i0 + q];
-      b4[q] = B[k * kWtLd + j0 + q];
-    }
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) acc[i][j] = __fma_rn(a4[i], b4[j], acc[i][j]);
-  }
-}
 
 // Row sums of magnitudes and diagonals of the triangles within their
 // superblocks (a warp per row; fp32 is enough for the test below).
 template <typename F>
 __device__ __forceinline__ void wide_rows(Cx& cx, const RefineArgs& a) {
   const int n = cx.n, nw = cx.G * (kRefThreads / 32);
-  if (cx.cta == 0 && cx.tid == 0) *a.wflag = 0;
+  if (cx.cta == 0 && cx.tid == 0) a.wflag[0] = a.wflag[1] = 0;
   for (int q = cx.cta * (kRefThreads / 32) + cx.warp; q < 2 * n; q += nw) {
     const bool lower = q < n;
     const int r = lower ? q : q - n, s0 = r / kSuper * kSuper;
@@ -1594,22 +1577,21 @@ static __device__ __noinline__ void wide_check(Cx& cx, const RefineArgs& a) {
 // Inverses of the diagonal superblocks from those of the 64x64 blocks
 // (build_inverses has put them on the diagonal), by doubling h = 64, 128, ..:
 //   L: X21 = -X22 (L21 X11)     U: X12 = -X11 (U12 X22)
-// in 64x64 tiles over all CTAs.  The inner product T waits in the opposite
-// off-diagonal block of the same array, which the inverse does not use (its
-// readers stay inside the triangle).
-template <typename F, bool kF32>
+// as fp32 pairs, in 64x64 tiles over all CTAs.  The inner product T waits in
+// the opposite off-diagonal block of the same arrays, which the inverse does
+// not use (its readers stay inside the triangle).
+template <typename F>
 __device__ __noinline__ bool build_wide(Cx& cx, const RefineArgs& a) {
-  using S = typename std::conditional<kF32, float, double>::type;
-  S* D0 = kF32 ? (S*)a.D32h : (S*)a.D64;
-  S* D1 = kF32 ? (S*)a.D32l : nullptr;
-  S* As = (S*)cx.tsm;                 // [k][i], high words
-  S* Bs = As + kBlk * kWtLd;          // [k][j]
-  S* Al = Bs + kBlk * kWtLd;          // low words (fp32)
-  S* Bl = Al + kBlk * kWtLd;
+  float* D0 = a.D32h;
+  float* D1 = a.D32l;
+  float* As = (float*)cx.tsm;         // [k][i], high words
+  float* Bs = As + kBlk * kWtLd;      // [k][j]
+  float* Al = Bs + kBlk * kWtLd;      // low words
+  float* Bl = Al + kBlk * kWtLd;
   constexpr int sb = kSuper;
   const int n = cx.n, ldf = a.ldf;
   const int i0 = (cx.tid >> 4) * 4, j0 = (cx.tid & 15) * 4;
-  if (kF32) wide_rows<F>(cx, a);  // (read behind the barriers of the doubling)
+  wide_rows<F>(cx, a);  // (read behind the barriers of the doubling)
   for (int h = kBlk; h < sb; h *= 2) {
     const int nt = h / kBlk, npair = (a.npad / 2) / h;
     for (int pass = 0; pass < 2; ++pass) {
@@ -1626,44 +1608,37 @@ __device__ __noinline__ bool build_wide(Cx& cx, const RefineArgs& a) {
         const int yk0 = lower ? 0 : ti, yk1 = lower ? ti + 1 : nt;      // pass 1
         const int tr = lower ? o : o + h, tc = lower ? oc + h : oc;     // where T waits
         const int k0 = pass ? yk0 : xk0, k1 = pass ? yk1 : xk1;
-        typename std::conditional<kF32, ff_t, double>::type acc[4][4];
+        ff_t acc[4][4];
 #pragma unroll
         for (int i = 0; i < 4; ++i)
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            if constexpr (kF32) acc[i][j] = ff_t{0.0f, 0.0f};
-            else acc[i][j] = 0.0;
-          }
+          for (int j = 0; j < 4; ++j) acc[i][j] = ff_t{0.0f, 0.0f};
         for (int kt = k0; kt < k1; ++kt) {
           __syncthreads();  // the previous staging is no longer read
           for (int e = cx.tid; e < kBlk * kBlk; e += kRefThreads) {
             const int r = e / kBlk, c = e % kBlk;
             if (pass == 0) {
               const int frow = fr + ti * kBlk + r, fcol = xr + kt * kBlk + c;
-              As[c * kWtLd + r] = (frow < n && fcol < n) ? (S)factor_at<F>(a, (size_t)frow * ldf + fcol) : (S)0;
+              As[c * kWtLd + r] = (frow < n && fcol < n) ? (float)factor_at<F>(a, (size_t)frow * ldf + fcol) : 0.0f;
               const int xrow = xr + kt * kBlk + r;
               const size_t x = wide_row(a, tri, xrow) + (xr - o) + oc + tj * kBlk + c;
-              Bs[r * kWtLd + c] = xrow < n ? __ldcg(D0 + x) : (S)0;
-              if (kF32) Bl[r * kWtLd + c] = xrow < n ? __ldcg(D1 + x) : (S)0;
+              Bs[r * kWtLd + c] = xrow < n ? __ldcg(D0 + x) : 0.0f;
+              Bl[r * kWtLd + c] = xrow < n ? __ldcg(D1 + x) : 0.0f;
             } else {
               const int xrow = fr + ti * kBlk + r;
               const size_t x = wide_row(a, tri, xrow) + (fr - o) + oc + kt * kBlk + c;
-              As[c * kWtLd + r] = xrow < n ? __ldcg(D0 + x) : (S)0;
-              if (kF32) Al[c * kWtLd + r] = xrow < n ? __ldcg(D1 + x) : (S)0;
+              As[c * kWtLd + r] = xrow < n ? __ldcg(D0 + x) : 0.0f;
+              Al[c * kWtLd + r] = xrow < n ? __ldcg(D1 + x) : 0.0f;
               const int trow = kt * kBlk + r;  // inner index of T
               const size_t y = wide_row(a, tri, tr + trow) + tc + tj * kBlk + c;
               const bool in = fr + trow < n;   // rows of T past the matrix were not formed
-              Bs[r * kWtLd + c] = in ? __ldcg(D0 + y) : (S)0;
-              if (kF32) Bl[r * kWtLd + c] = in ? __ldcg(D1 + y) : (S)0;
+              Bs[r * kWtLd + c] = in ? __ldcg(D0 + y) : 0.0f;
+              Bl[r * kWtLd + c] = in ? __ldcg(D1 + y) : 0.0f;
             }
           }
           __syncthreads();
-          if constexpr (kF32) {
-            if (pass == 0) wide_tile_mma<false>(As, Al, Bs, Bl, i0, j0, acc);
-            else wide_tile_mma<true>(As, Al, Bs, Bl, i0, j0, acc);
-          } else {
-            wide_tile_mma(As, Bs, i0, j0, acc);
-          }
+          if (pass == 0) wide_tile_mma<false>(As, Al, Bs, Bl, i0, j0, acc);
+          else wide_tile_mma<true>(As, Al, Bs, Bl, i0, j0, acc);
         }
         // T to its waiting place (row index: inner index of the second
         // product), X_off negated
@@ -1675,27 +1650,155 @@ __device__ __noinline__ bool build_wide(Cx& cx, const RefineArgs& a) {
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
             const size_t y = x + tj * kBlk + j0 + j;
-            if constexpr (kF32) {
-              ArFF::V v = ArFF::fin(acc[i][j]);
-              if (pass) v = ArFF::neg(v);
-              D0[y] = v.h;
-              D1[y] = v.l;
-            } else {
-              D0[y] = pass ? -acc[i][j] : acc[i][j];
-            }
+            ArFF::V v = ArFF::fin(acc[i][j]);
+            if (pass) v = ArFF::neg(v);
+            D0[y] = v.h;
+            D1[y] = v.l;
           }
         }
       }
       if (!grid_barrier(cx, a)) return false;
     }
   }
-  if (!kF32) {
-    cx.mready |= RDY_W64;
-    return true;
-  }
   wide_check(cx, a);
   if (!grid_barrier(cx, a)) return false;
   cx.mready |= __ldcg(a.wflag) ? RDY_NO32 : RDY_W32;
+  return true;
+}
+
+// Running sum of fp32 products f (h + l) in three words: the first two take
+// their terms by TwoSum, the third collects what those round off (Ogita,
+// Rump and Oishi's K-fold summation, K = 3: about 2^-70 of the magnitudes).
+struct ff3_t {
+  float s0, s1, s2;
+};
+__device__ __forceinline__ void ff3_term(ff3_t& a, float f, float h, float l) {
+  const float p = __fmul_rn(f, h), pe = __fmaf_rn(f, h, -p);
+  const float q = __fmul_rn(f, l), qe = __fmaf_rn(f, l, -q);
+  float t, u1, u2, u3;
+  two_sum_f(a.s0, p, a.s0, t);
+  two_sum_f(a.s1, t, a.s1, u1);
+  two_sum_f(a.s1, pe, a.s1, u2);
+  two_sum_f(a.s1, q, a.s1, u3);
+  a.s2 = __fadd_rn(a.s2, __fadd_rn(__fadd_rn(u1, u2), __fadd_rn(u3, qe)));
+}
+
+// fp64 inverses of the diagonal superblocks from the fp32 pairs X by one
+// Newton step, X (2 I - T X) = X + X R with the residual R = I - T X.  The
+// factor's values are exact in fp32, so T X is summed on the fp32 pipe in
+// three words; R is then known to some 2^-60 of its terms, and its own
+// rounding to fp32 and the plain fp32 product X R are a correction's.  What
+// is left is R^2 and the final rounding: the result is the inverse to about
+// one fp64 rounding.  (Doubled up in plain fp64 instead, the inverses carry
+// the superblock's Skeel condition number, some 1e4 for LU factors, times
+// 2^-53, and a solve with random right-hand sides was up to 2.6 times, with
+// graded rows 13 times, as inaccurate as the 64-row one.)
+//
+// R waits in M64, whose scaled blocks belong to the 64-row route (their bit
+// is cleared).  R scaled by the row sums s of |T|, R_ij s_j / s_i, has to
+// stay below kWideResid, so that R^2 (512 terms) is below 2^-54; otherwise
+// RDY_NO64 is set and the solves keep the 64-row route.
+//
+// The tiles of a superblock with the most inner tiles come first.
+template <typename F>
+__device__ __noinline__ bool build_wide64(Cx& cx, const RefineArgs& a) {
+  constexpr int NT = kSuper / kBlk, NP = NT * (NT + 1) / 2;
+  float* R = (float*)a.M64;
+  float* As = (float*)cx.tsm;     // [k][i]
+  float* Bs = As + kBlk * kWtLd;  // [k][j]
+  float* Bl = Bs + kBlk * kWtLd;
+  const int n = cx.n, ldf = a.ldf, NS = a.npad / kSuper;
+  const int i0 = (cx.tid >> 4) * 4, j0 = (cx.tid & 15) * 4;
+  cx.mready &= ~RDY_M64;
+  for (int pass = 0; pass < 2; ++pass) {
+    bool bad = false;
+    for (int t = cx.cta; t < 2 * NS * NP; t += cx.G) {
+      const int tri = t % 2, s0 = (t / 2) % NS * kSuper;
+      // the q-th pair of tiles, distance NT - 1 first
+      int q = t / (2 * NS), d = NT - 1;
+      for (int cnt = 1; q >= cnt; ++cnt, --d) q -= cnt;
+      const bool lower = tri == 0;
+      const int ti = lower ? q + d : q, tj = lower ? q : q + d;
+      const int r0 = s0 + ti * kBlk, c0 = s0 + tj * kBlk;  // first row and column of the tile
+      if (max(r0, c0) >= n) continue;
+      ff3_t acc[4][4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = ff3_t{0.0f, 0.0f, 0.0f};
+      for (int kt = min(ti, tj); kt <= max(ti, tj); ++kt) {
+        const int k0 = s0 + kt * kBlk;
+        __syncthreads();  // the previous staging is no longer read
+        for (int e = cx.tid; e < kBlk * kBlk; e += kRefThreads) {
+          const int r = e / kBlk, c = e % kBlk;
+          const int arow = r0 + r, acol = k0 + c, brow = k0 + r;
+          float av = 0.0f, bh = 0.0f, bl = 0.0f;
+          if (pass == 0) {
+            if (arow < n && acol < n && (lower ? acol < arow : acol >= arow))
+              av = (float)factor_at<F>(a, (size_t)arow * ldf + acol);
+            else if (lower && acol == arow)
+              av = 1.0f;
+          } else if (arow < n) {
+            av = __ldcg(a.D32h + wide_row(a, tri, arow) + kt * kBlk + c);
+          }
+          if (brow < n) {
+            const size_t x = wide_row(a, tri, brow) + tj * kBlk + c;
+            bh = pass == 0 ? __ldcg(a.D32h + x) : __ldcg(R + x);
+            if (pass == 0) bl = __ldcg(a.D32l + x);
+          }
+          As[c * kWtLd + r] = av;
+          Bs[r * kWtLd + c] = bh;
+          Bl[r * kWtLd + c] = bl;
+        }
+        __syncthreads();
+#pragma unroll 2
+        for (int k = 0; k < kBlk; ++k) {
+          const float4 f = *(const float4*)(As + k * kWtLd + i0);
+          const float4 bh = *(const float4*)(Bs + k * kWtLd + j0);
+          const float F4[4] = {f.x, f.y, f.z, f.w}, H4[4] = {bh.x, bh.y, bh.z, bh.w};
+          if (pass == 0) {
+            const float4 bl = *(const float4*)(Bl + k * kWtLd + j0);
+            const float L4[4] = {bl.x, bl.y, bl.z, bl.w};
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+              for (int j = 0; j < 4; ++j) ff3_term(acc[i][j], F4[i], H4[j], L4[j]);
+          } else {
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+              for (int j = 0; j < 4; ++j) acc[i][j].s0 = __fmaf_rn(F4[i], H4[j], acc[i][j].s0);
+          }
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int row = r0 + i0 + i;
+        if (row >= n) continue;
+        const size_t x = wide_row(a, tri, row) + tj * kBlk + j0;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const int col = c0 + j0 + j;
+          const ff3_t v = acc[i][j];
+          if (pass == 0) {
+            float h, l;
+            two_sum_f(__fsub_rn(v.s0, row == col ? 1.0f : 0.0f), v.s1, h, l);
+            const float r = -__fadd_rn(h, __fadd_rn(l, v.s2));
+            R[x + j] = r;
+            if (col < n)
+              bad |= !(fabsf(r) * __ldcg(a.wrow + (size_t)tri * a.npad + col) <=
+                       kWideResid * __ldcg(a.wrow + (size_t)tri * a.npad + row));
+          } else {
+            a.D64[x + j] = __dadd_rn((double)__ldcg(a.D32h + x + j),
+                                     __dadd_rn((double)__ldcg(a.D32l + x + j), (double)v.s0));
+          }
+        }
+      }
+    }
+    if (bad) atomicOr(a.wflag + 1, 1);
+    if (!grid_barrier(cx, a)) return false;
+  }
+  cx.mready |= __ldcg(a.wflag + 1) ? RDY_NO64 : RDY_W64;
   return true;
 }
 
@@ -2191,16 +2294,13 @@ __device__ bool msolve(Cx& cx, const RefineArgs& a, int store_fmt, bool synced) 
   // one superblock would not see each other's rounding, which doubles the
   // error of the result)
   if (use_wide<ACC, F>(a) && (ACC::kW == 2 || store_fmt >= MSIR_FP32)) {
-    if constexpr (!std::is_same<F, FAny>::value && ACC::kW <= 2) {
+    if constexpr (!std::is_same<F, FAny>::value && !std::is_same<F, double>::value && ACC::kW <= 2) {
       constexpr bool k32 = ACC::kW == 1;
       const unsigned need = k32 ? RDY_W32 : RDY_W64;
-      if (!(cx.mready & (need | (k32 ? RDY_NO32 : 0u)))) {
-        if (k32 || !(cx.mready & RDY_INV)) {
-          if (!build_inverses<F>(cx, a, !k32, true)) return false;
-          if (!k32) cx.mready |= RDY_INV;
-        }
-        if (!build_wide<F, k32>(cx, a)) return false;
-      }
+      if (!(cx.mready & (RDY_W32 | RDY_NO32)))
+        if (!build_inverses<F>(cx, a, false, true) || !build_wide<F>(cx, a)) return false;
+      if (!k32 && (cx.mready & RDY_W32) && !(cx.mready & (RDY_W64 | RDY_NO64)))
+        if (!build_wide64<F>(cx, a)) return false;
       if (cx.mready & need) {
         if (!synced && !grid_barrier(cx, a)) return false;
         {

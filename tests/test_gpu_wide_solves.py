@@ -85,3 +85,50 @@ def test_rows_that_leave_the_range_of_a_superblock(ctx, monkeypatch, n, lo, hi):
     ref = np.linalg.solve(T, c * 2.0 ** -e)
     u = 2.0 ** -24
     assert np.max(np.abs(got - ref)) <= 2 * (n * u + u) * cond_comp(T, ref) * np.max(np.abs(ref))
+
+
+@pytest.mark.parametrize("n,kappa,graded", [(1793, 1e2, False), (2100, 1e8, False), (2560, 1e4, True), (3100, 1e6, False)])
+@pytest.mark.parametrize("uf", [OF.FP16, OF.FP32])
+def test_fp64_error_is_below_the_64_row_route(ctx, monkeypatch, n, kappa, graded, uf):
+    """fp64: the superblocks' inverses are the exact ones rounded to fp64, as
+    the 64-row blocks' are, so the error of a solve is bounded by |X||T||x|
+    on both routes and fewer roundings are left on the wide one.  (Rows
+    graded by 10^+-4: right-hand sides of the same grading.)"""
+    A, B = system(n, kappa, graded)
+    if graded:
+        B = B[:, :2]
+    ew, e64 = route_errors(ctx, monkeypatch, A, B, OF.FP32, uf, OF.FP64)
+    assert np.all(ew <= e64), (ew / e64)
+
+
+@pytest.mark.parametrize("c", [0.15, 0.3, 0.4])
+@pytest.mark.parametrize("arith", [OF.FP32, OF.FP64])
+def test_ill_conditioned_superblocks(ctx, monkeypatch, c, arith):
+    """U = I + c N, N uniform in [-1, 1] above the diagonal: the Skeel
+    condition number of its 512-row blocks is 2^10.8, 2^18.1 and 2^25.5, on
+    both sides of what the pairs and the Newton step are used for."""
+    n = 1900
+    rng = np.random.default_rng(1)
+    A = (np.eye(n) + c * np.triu(rng.uniform(-1, 1, (n, n)), 1)).astype(np.float32).astype(np.float64)
+    ew, e64 = route_errors(ctx, monkeypatch, A, rng.standard_normal((n, 4)).astype(np.float32).astype(np.float64),
+                           OF.FP32, OF.FP32, arith)
+    assert np.all(ew <= e64), (ew / e64)
+
+
+def test_routes_share_a_workspace(ctx, monkeypatch):
+    """The wide route's construction uses the 64-row route's scaled blocks as
+    scratch: each route gives the same bits before and after the other, in
+    either order of first use."""
+    import paper_2107_06200_gb300 as M
+    n = 1793
+    A, B = system(n, 1e3, False)
+    x = {}
+    for order in ("01010", "10101"):
+        f = ctx.factor(to_dev(A), OF.FP32, OF.FP16, M.params_default())
+        for route in order:
+            monkeypatch.setenv("MSIR_WIDE_APPLY", route)
+            for arith in (OF.FP64, OF.FP32):
+                got = f.apply(to_dev(B), arith, arith).cpu().numpy()
+                assert np.array_equal(got, x.setdefault((route, arith), got))
+        f.close()
+    assert not np.array_equal(x["0", OF.FP64], x["1", OF.FP64])
