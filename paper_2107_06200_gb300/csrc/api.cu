@@ -198,6 +198,7 @@ struct Workspace {
   float* inv32l = nullptr;
   double* inv_hi = nullptr;
   double* inv_lo = nullptr;
+  int* inv_hard = nullptr;
   void* Ut = nullptr;
   int* map = nullptr;       // map_pos | map_val | map_cnt
   int* iflags = nullptr;    // info, nonfinite, err
@@ -267,6 +268,7 @@ static size_t ws_layout(Workspace& w, int n, int kcap, int G, bool alloc_f64_lev
   w.inv32l = (float*)take(ninv * 4);
   w.inv_hi = (double*)take(ninv * 8);
   w.inv_lo = (double*)take(ninv * 8);
+  w.inv_hard = (int*)take(ninv / (kBlk * kBlk) * 4);
   w.Ut = take((size_t)n * 256 * 2);
   w.map = (int*)take(2 * kMapInts * 4);  // two outer blocks' maps (look-ahead)
   w.iflags = (int*)take(32 * 4);
@@ -787,6 +789,7 @@ static void fill_args(msir_ctx* ctx, Slot& s, RefineArgs& a, int mode) {
   a.H = w.H; a.yv = w.yv; a.red = w.red; a.hred = w.hred; a.hvec = w.hvec;
   a.ll = w.ll; a.bar = w.bar;
   a.inv32 = w.inv32; a.inv32l = w.inv32l; a.inv_hi = w.inv_hi; a.inv_lo = w.inv_lo;
+  a.inv_hard = w.inv_hard;
   a.M32 = w.M32; a.M64 = w.M64; a.Mdh = w.Mdh; a.Mdl = w.Mdl; a.err = w.iflags + 2; a.st = w.st; a.rep = w.rep;
   a.tsv = trsv_timers_enabled() ? w.tsv : nullptr;
   a.i_max = j.p.i_max;
@@ -1446,7 +1449,8 @@ msir_status msir_factor(msir_ctx* ctx, int n, const double* A_dev, int lda, int 
   if (s.h_flags[2]) { int e = s.h_flags[2]; slot_destroy(s); delete f; return (msir_status)e; }
   if (L.info == 0 && L.nonfinite == 0) {
     // the diagonal blocks' inverses belong to the factors that the caller
-    // keeps; an apply builds what its precision needs beside them, once
+    // keeps: every apply starts from them (in fp32 rounded to pairs) and
+    // builds what else its precision needs, once
     RefineArgs a;
     fill_args(ctx, s, a, MODE_PREP);
     RefState st0;
@@ -1715,6 +1719,7 @@ static BatchLayout batch_layout(int nmax, int kcap) {
   L.d = off(w.d); L.w = off(w.w); L.vk = off(w.vk);
   L.V = off(w.V); L.H = off(w.H); L.yv = off(w.yv); L.red = off(w.red); L.hred = off(w.hred);
   L.inv32 = off(w.inv32); L.inv32l = off(w.inv32l); L.inv_hi = off(w.inv_hi); L.inv_lo = off(w.inv_lo);
+  L.inv_hard = off(w.inv_hard);
   L.hvec = off(w.hvec); L.ll = off(w.ll); L.M32 = off(w.M32); L.M64 = off(w.M64); L.Mdh = off(w.Mdh);
   L.Mdl = off(w.Mdl); L.bar = off(w.bar); L.iflags = off(w.iflags);
   L.ldu = w.ldu;

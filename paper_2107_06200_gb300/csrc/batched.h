@@ -16,7 +16,7 @@ namespace msir {
 struct BatchLayout {
   size_t Au, b_u, rowsum, rowmax, colmax;
   size_t F[3], ipiv[3], perm[3], R[3], S[3];
-  size_t inv32, inv32l, inv_hi, inv_lo;
+  size_t inv32, inv32l, inv_hi, inv_lo, inv_hard;
   size_t x, xn, x0, xbest, r_hi, r_lo, c_hi, c_lo, y_hi, y_lo, z_hi, z_lo, d, w, vk;
   size_t V, H, yv, red, hred, hvec, ll, M32, M64, Mdh, Mdl, bar, iflags;
   int ldu, ldv, kcap, nmax;

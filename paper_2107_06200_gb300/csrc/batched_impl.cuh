@@ -223,6 +223,7 @@ __global__ void __launch_bounds__(kBatchThreads, 1) batched_solve_kernel(BatchAr
     a.ll = (unsigned long long*)(ws + L.ll);
     a.inv32 = (float*)(ws + L.inv32); a.inv32l = (float*)(ws + L.inv32l);
     a.inv_hi = (double*)(ws + L.inv_hi); a.inv_lo = (double*)(ws + L.inv_lo);
+    a.inv_hard = (int*)(ws + L.inv_hard);
     a.M32 = (float*)(ws + L.M32); a.M64 = (double*)(ws + L.M64);
     a.Mdh = (double*)(ws + L.Mdh); a.Mdl = (double*)(ws + L.Mdl);
     a.bar = (unsigned*)(ws + L.bar);

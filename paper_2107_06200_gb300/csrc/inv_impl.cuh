@@ -13,7 +13,9 @@
 // Oishi's Dot2, with the low words of pair operands added), results are
 // unevaluated pairs h + l:
 //   ArFF  pairs of fp32 (about 2^-46 per operation, all work on the fp32
-//         pipe): for fp32 solves, whose inverse is the pair rounded to fp32;
+//         pipe): for fp32 solves, whose inverse is the pair rounded to fp32,
+//         while the block's Skeel condition number (inv_cond) leaves some
+//         2^-30 of that, as it does for LU factors; other blocks take ArDD;
 //   ArDD  pairs of fp64 (about 2^-104): for fp64 solves (the high word) and
 //         double-double ones.
 #pragma once
@@ -218,6 +220,27 @@ __device__ __forceinline__ void inv_triangle(bool lower, typename AR::S* sm) {
   inv_double<AR, 8>(lower, B, Xh, Xl, Th, Tl);
   inv_double<AR, 16>(lower, B, Xh, Xl, Th, Tl);
   inv_double<AR, 32>(lower, B, Xh, Xl, Th, Tl);
+}
+
+// Whether the Skeel condition number max_i (|X||B|e)_i of the triangle and
+// its inverse in sm (inv_triangle's arrangement) is at most `limit`: the
+// relative error of the pairs is that times their 2^-46.  Unlike the norms'
+// product it does not see how the rows are scaled.  False if X is not finite.
+__device__ __forceinline__ bool inv_cond_below(float* sm, float limit) {
+  const float* X = sm + kIB * kXld;
+  float* sum = sm + kInvValues - kIB;  // (the reciprocals' low words are no longer read)
+  const int row = threadIdx.x >> 2, part = threadIdx.x & 3;
+  float s = 0.0f;
+  for (int k = part; k < kIB; k += 4) s += fabsf(sm[row * kXld + k]);
+  s += __shfl_xor_sync(0xffffffffu, s, 1);
+  s += __shfl_xor_sync(0xffffffffu, s, 2);
+  if (part == 0) sum[row] = s;
+  __syncthreads();
+  float v = 0.0f;
+  for (int k = part; k < kIB; k += 4) v += fabsf(X[row * kXld + k]) * sum[k];
+  v += __shfl_xor_sync(0xffffffffu, v, 1);
+  v += __shfl_xor_sync(0xffffffffu, v, 2);
+  return __syncthreads_and(v <= limit) != 0;
 }
 
 // Diagonal block b of triangle `lower` (get(i, k): the packed factor's entry

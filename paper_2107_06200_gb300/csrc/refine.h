@@ -172,6 +172,7 @@ struct RefineArgs {
   float* inv32l;
   double* inv_hi;
   double* inv_lo;
+  int* inv_hard;           // [2][ceil(n/kBlk)]: block kept out of the fp32 pairs' sums
   // scaled off-diagonal blocks D_b^{-1} F_bj (j != b) of L (j < b) and U
   // (j > b), row-major with leading dimension ldf, built in the kernel when a
   // solve in that precision first needs them (RefState::mready)

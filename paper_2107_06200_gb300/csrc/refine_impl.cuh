@@ -817,34 +817,59 @@ __device__ __forceinline__ size_t wide_row(const RefineArgs& a, int tri, int r) 
 // Inverses of the diagonal blocks of L and U by all CTAs of the grid, once
 // per factorisation: as fp32 pairs (dd = false; inv32, inv32l) or in
 // double-double (inv_hi, inv_lo, and for fp64 factors inv32, inv32l too);
-// `wide`: the fp32 pairs go into the superblocks' array.  An
-// fp32 pair keeps its 2^-46 as long as the block's diagonal is far from
-// fp32's range ends; other blocks take the double-double arithmetic.
+// `wide`: the fp32 pairs go into the superblocks' array.
+//
+// The fp32 pairs of a block are formed in pair arithmetic if its diagonal is
+// far from fp32's range ends and its Skeel condition number is at most
+// kInvCond: their error of 2^-46 times that is then below 2^-32, so that the
+// inverse's fp32 rounding is the exact inverse's but for near ties.  (LU
+// factors of randsvd matrices, kappa 1e2 .. 1e8, plain and with rows graded
+// by 10^+-4: at most 1.3e3.  Solves with such inverses and scaled blocks
+// against double-double ones, n = 1024 .. 7237: 1.000 times the error of
+// those formed in double-double and fp64.)  Other blocks are formed in
+// double-double and marked inv_hard.  Where double-double inverses are there
+// already (kept factors), they are rounded to pairs instead.
+constexpr float kInvCond = 0x1p14f;
 template <typename F>
 __device__ __noinline__ bool build_inverses(Cx& cx, const RefineArgs& a, bool dd, bool wide) {
   float* smf = (float*)cx.tsm;
   double* smd = (double*)cx.tsm;
   const bool want32 = !dd || factor_fmt<F>(a) == MSIR_FP64;
+  const bool have = !dd && (cx.mready & RDY_INV);
   for (int q = cx.cta; q < 2 * cx.nblk; q += cx.G) {
     const int b = q % cx.nblk;
     const bool lower = q < cx.nblk;
     const size_t f0 = (size_t)b * kBlk * a.ldf + (size_t)b * kBlk;
+    const size_t base = ((size_t)(lower ? 0 : 1) * cx.nblk + b) * kBlk * kBlk;
+    const int nr = min(kBlk, cx.n - b * kBlk);
     auto get = [&](int i, int k) { return factor_at<F>(a, f0 + (size_t)i * a.ldf + k); };
     bool pair64 = dd;
     __syncthreads();  // the scratch is no longer read
     if (!dd) {
       inv_load<float>(smf, cx.n, b, lower, get);
       const float d = cx.tid < kBlk ? fabsf(smf[cx.tid * kXld + cx.tid]) : 1.0f;
-      pair64 = __syncthreads_or(!(d >= 0x1p-60f && d <= 0x1p60f)) != 0;
+      bool hard = __syncthreads_or(!(d >= 0x1p-60f && d <= 0x1p60f)) != 0;
+      if (have) {
+        for (int e = cx.tid; e < kBlk * kBlk; e += kRefThreads) {
+          const double h = __ldcg(a.inv_hi + base + e), l = __ldcg(a.inv_lo + base + e);
+          const float r = dd_to_f32(h, l);
+          const int x = kIB * kXld + e / kBlk * kXld + e % kBlk;
+          smf[x] = r;
+          smf[x + kIB * kXld] = isfinite(r) ? (float)((h - (double)r) + l) : 0.0f;
+        }
+        __syncthreads();
+      } else if (!hard) {
+        inv_triangle<ArFF>(lower, smf);
+      }
+      hard = hard || !inv_cond_below(smf, kInvCond);
+      if (cx.tid == 0) a.inv_hard[q] = hard;
+      pair64 = hard && !have;
+      __syncthreads();
     }
     if (pair64) {
       inv_load<double>(smd, cx.n, b, lower, get);
       inv_triangle<ArDD>(lower, smd);
-    } else {
-      inv_triangle<ArFF>(lower, smf);
     }
-    const size_t base = ((size_t)(lower ? 0 : 1) * cx.nblk + b) * kBlk * kBlk;
-    const int nr = min(kBlk, cx.n - b * kBlk);
     // for wide solves the blocks go on the diagonals of the superblocks
     const size_t wbase = wide ? wide_row(a, lower ? 0 : 1, b * kBlk) + (b * kBlk) % kSuper : 0;
     const bool w32 = wide && !dd;
@@ -856,10 +881,8 @@ __device__ __noinline__ bool build_inverses(Cx& cx, const RefineArgs& a, bool dd
       const bool in = i < nr && k < nr;
       if (pair64) {
         const double h = in ? smd[x] : 0.0, l = in ? smd[x + kIB * kXld] : 0.0;
-        if (dd) {
-          a.inv_hi[base + e] = h;
-          a.inv_lo[base + e] = l;
-        }
+        a.inv_hi[base + e] = h;
+        a.inv_lo[base + e] = l;
         if (want32) {
           const float r = dd_to_f32(h, l);
           o32h[(size_t)i * ld32 + k] = r;
@@ -888,7 +911,8 @@ __device__ __noinline__ bool build_inverses(Cx& cx, const RefineArgs& a, bool dd
 // take three 16-byte loads per inner step; terms outside the triangle of the
 // inverse are zero and skipped (a warp has 8 rows, warps w and w + 4 of one
 // scheduler have long and short sums).  Measured (n = 8192): 7.2 -> 1.0 ms
-// against fp64 sums.
+// against fp64 sums.  Rows of blocks marked inv_hard take those: the fp64
+// inverse, fp64 sums in the order of k, rounded once.
 template <typename F>
 __device__ __noinline__ bool build_scaled32(Cx& cx, const RefineArgs& a) {
   float* Xh = (float*)cx.ssm;  // [k][i], kBlk x kSc32Ld
@@ -904,6 +928,18 @@ __device__ __noinline__ bool build_scaled32(Cx& cx, const RefineArgs& a) {
     const size_t ib = ((size_t)(lower ? 0 : 1) * nb + b) * kBlk * kBlk;
     const int r0 = b * kBlk, q0 = j * kBlk;
     __syncthreads();  // the previous staging is no longer read
+    if (__ldcg(a.inv_hard + (lower ? 0 : nb) + b)) {
+      for (int e = cx.tid; e < kBlk * kBlk; e += kRefThreads) {
+        const int i = e / kBlk, row = r0 + i, col = q0 + e % kBlk;
+        if (row >= n || col >= n) continue;
+        double s = 0.0;
+        const int k0 = lower ? 0 : i, k1 = lower ? i + 1 : min(kBlk, n - r0);
+        for (int k = k0; k < k1; ++k)
+          s = __fma_rn(__ldcg(a.inv_hi + ib + (size_t)i * kBlk + k), factor_at<F>(a, (size_t)(r0 + k) * ld + col), s);
+        a.M32[(size_t)row * ld + col] = __double2float_rn(s);
+      }
+      continue;
+    }
     for (int e = cx.tid; e < kBlk * kBlk; e += kRefThreads) {
       const int i = e / kBlk, k = e % kBlk;
       Xh[k * kSc32Ld + i] = __ldcg(a.inv32 + ib + e);
