@@ -143,12 +143,6 @@ template <> struct RowAcc<MSIR_DD> {
     s = v.hi;
     c = v.lo;
   }
-  // as a term of the sum: five fp64 operations instead of 26
-  __device__ __forceinline__ void merge_term(const RowAcc& o) {
-    const dd_t t = two_sum_ord(s, o.s);
-    s = t.hi;
-    c = __dadd_rn(c, __dadd_rn(t.lo, o.c));
-  }
   __device__ __forceinline__ RowAcc peer(int m) const {
     return RowAcc{__shfl_xor_sync(0xffffffffu, s, m), __shfl_xor_sync(0xffffffffu, c, m)};
   }
@@ -280,26 +274,17 @@ __device__ __forceinline__ void gemv_rows_n(Cx& cx, const RefineArgs& a, const X
       }
       __syncwarp();
     }
-    // Double-double: a lane's sums as terms of the row's from kTermMerge
-    // columns on.  n = 8192: 1.29 -> 1.22 ms, largest error against exact
-    // sums 0.94 -> 0.34 x 2^-106 sum |a x|; for rows of a few terms a lane,
-    // the sum of renormalised pairs has the smaller one (n = 100: 0.27 and 0.47).
-    constexpr int kTermMerge = 2048;
-    auto merge = [&](Acc& d, const Acc& o) {
-      if constexpr (OP == MSIR_DD) {
-        if (n >= kTermMerge) d.merge_term(o);
-        else d.merge(o);
-      } else {
-        d.merge(o);
-      }
-    };
+    // (Double-double sums are merged as renormalised pairs, 26 operations.
+    // As terms of the row's sum, five, they took 1.22 instead of 1.29 ms at n
+    // = 8192, with a mean error of 0.22 instead of 0.19 x 2^-106 sum |a x|;
+    // 0.16 and 0.12 at n = 2048.)
 #pragma unroll
     for (int r = 0; r < NR; ++r)
-      if (kOdd) merge(acc[r][0], acc[r][1]);
+      if (kOdd) acc[r][0].merge(acc[r][1]);
 #pragma unroll
     for (int m = 16; m > 0; m >>= 1)
 #pragma unroll
-      for (int r = 0; r < NR; ++r) merge(acc[r][0], acc[r][0].peer(m));
+      for (int r = 0; r < NR; ++r) acc[r][0].merge(acc[r][0].peer(m));
     Acc mine = acc[0][0];
 #pragma unroll
     for (int r = 1; r < NR; ++r)
