@@ -1455,9 +1455,10 @@ msir_status msir_factor(msir_ctx* ctx, int n, const double* A_dev, int lda, int 
     fill_args(ctx, s, a, MODE_PREP);
     RefState st0;
     memset(&st0, 0, sizeof(st0));
-    cudaMemcpyAsync(s.w.st, &st0, sizeof(st0), cudaMemcpyHostToDevice, s.st);
-    cudaMemsetAsync(s.w.bar, 0, 64, s.st);
-    r = cuda_status(launch_refine(s.u0, L.fmt, a, s.G, s.st));
+    // (this mode has no barrier and no other wait: the launch and the
+    // synchronisation report all that can go wrong)
+    r = cuda_status(cudaMemcpyAsync(s.w.st, &st0, sizeof(st0), cudaMemcpyHostToDevice, s.st));
+    if (r == MSIR_OK) r = cuda_status(launch_refine(s.u0, L.fmt, a, s.G, s.st));
     if (r == MSIR_OK) r = cuda_status(cudaStreamSynchronize(s.st));
     if (r != MSIR_OK) { slot_destroy(s); delete f; return r; }
     s.w.m_serial = L.serial;

@@ -97,7 +97,7 @@ constexpr size_t wide_smem(int npad, int G, int vbytes, int ring) {
 }
 
 // MODE_PREP: the double-double inverses of the diagonal blocks alone (a
-// factorisation that is handed out)
+// factorisation that is handed out); no CTA waits for another
 enum RefMode { MODE_SOLVE = 0, MODE_APPLY = 1, MODE_RESIDUAL = 2, MODE_PREP = 3 };
 enum RefPhase {
   PH_START = 0,      // compute x0, then refine

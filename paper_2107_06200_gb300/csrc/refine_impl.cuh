@@ -813,10 +813,11 @@ __device__ __forceinline__ size_t wide_row(const RefineArgs& a, int tri, int r) 
 // against double-double ones, n = 1024 .. 7237: 1.000 times the error of
 // those formed in double-double and fp64.)  Other blocks are formed in
 // double-double and marked inv_hard.  Where double-double inverses are there
-// already (kept factors), they are rounded to pairs instead.
+// already (kept factors), they are rounded to pairs instead.  The caller puts
+// a grid barrier behind it; nothing here waits.
 constexpr float kInvCond = 0x1p14f;
 template <typename F>
-__device__ __noinline__ bool build_inverses(Cx& cx, const RefineArgs& a, bool dd, bool wide) {
+__device__ __noinline__ void build_inverses(Cx& cx, const RefineArgs& a, bool dd, bool wide) {
   float* smf = (float*)cx.tsm;
   double* smd = (double*)cx.tsm;
   const bool want32 = !dd || factor_fmt<F>(a) == MSIR_FP64;
@@ -879,7 +880,6 @@ __device__ __noinline__ bool build_inverses(Cx& cx, const RefineArgs& a, bool dd
       }
     }
   }
-  return grid_barrier(cx, a);
 }
 
 // Scaled off-diagonal blocks M_bj = D_b^{-1} F_bj (j != b; L below the
@@ -2318,8 +2318,10 @@ __device__ bool msolve(Cx& cx, const RefineArgs& a, int store_fmt, bool synced) 
     if constexpr (!std::is_same<F, FAny>::value && !std::is_same<F, double>::value && ACC::kW <= 2) {
       constexpr bool k32 = ACC::kW == 1;
       const unsigned need = k32 ? RDY_W32 : RDY_W64;
-      if (!(cx.mready & (RDY_W32 | RDY_NO32)))
-        if (!build_inverses<F>(cx, a, false, true) || !build_wide<F>(cx, a)) return false;
+      if (!(cx.mready & (RDY_W32 | RDY_NO32))) {
+        build_inverses<F>(cx, a, false, true);
+        if (!grid_barrier(cx, a) || !build_wide<F>(cx, a)) return false;
+      }
       if (!k32 && (cx.mready & RDY_W32) && !(cx.mready & (RDY_W64 | RDY_NO64)))
         if (!build_wide64<F>(cx, a)) return false;
       if (cx.mready & need) {
@@ -2339,9 +2341,13 @@ __device__ bool msolve(Cx& cx, const RefineArgs& a, int store_fmt, bool synced) 
   const unsigned need = ACC::kW == 4 ? RDY_MDD : (ACC::kW == 2 || f64) ? RDY_M64 : RDY_M32;
   if (!(cx.mready & need)) {
     if (need == RDY_M32) {
-      if (!build_inverses<F>(cx, a, false, false) || !build_scaled32<F>(cx, a)) return false;
+      build_inverses<F>(cx, a, false, false);
+      if (!grid_barrier(cx, a) || !build_scaled32<F>(cx, a)) return false;
     } else {
-      if (!(cx.mready & RDY_INV) && !build_inverses<F>(cx, a, true, false)) return false;
+      if (!(cx.mready & RDY_INV)) {
+        build_inverses<F>(cx, a, true, false);
+        if (!grid_barrier(cx, a)) return false;
+      }
       if (!build_scaled<F>(cx, a, need == RDY_MDD)) return false;
       cx.mready |= RDY_INV;
     }
@@ -3307,8 +3313,7 @@ __global__ void __launch_bounds__(kRefThreads, 1) refine_kernel(RefineArgs a) {
     ok = grid_barrier(cx, a) && residual<A0>(cx, a, a.x, a.ap_arith, s, xn);
     if (ok && cx.cta == 0 && cx.tid == 0) *a.res_s = s;
   } else if (a.mode == MODE_PREP) {
-    ok = build_inverses<F>(cx, a, true, false);
-    cx.mready |= RDY_INV;
+    build_inverses<F>(cx, a, true, false);
   } else if (a.mode == MODE_APPLY) {
     for (int b = cx.cta; b < cx.nblk; b += cx.G)
       for (int i = b * kBlk + cx.tid; i < min((b + 1) * kBlk, cx.n); i += kRefThreads) {
