@@ -269,7 +269,7 @@ __global__ void __launch_bounds__(kBatchThreads, 1) batched_solve_kernel(BatchAr
       if (fmt == MSIR_FP64 && nb > 16) nb = 16;
       if (nbo % nb) nbo = nb * ((nbo + nb - 1) / nb);
       if (nbo > 64) nbo = 64;
-      nb_used = nb;
+      nb_used = min(nb, fmt == MSIR_FP64 ? 16 : 32);  // (cta_lu splits wider panels)
       nbo_used = nbo;
       void* Fl = ws + L.F[l];
       int* ipiv = (int*)(ws + L.ipiv[l]);
