@@ -12,9 +12,10 @@
 //   lu_outer_panel      (lu_panel.cuh) one thread-block cluster factors an (n-k) x W outer
 //                       block: for each nb-column panel, the pivot search,
 //                       interchange, scaling and rank-1 updates run with the
-//                       panel in registers; pivot candidates and their rows
-//                       are pushed to every CTA of the cluster through
-//                       distributed shared memory, so each column costs one
+//                       panel in registers; each CTA sends its pivot
+//                       candidate and that row to every CTA of the cluster
+//                       by asynchronous stores that an mbarrier counts, so a
+//                       column costs one message and one wait per CTA and no
 //                       cluster barrier.  The inner interchanges,
 //                       substitution and update of the outer block follow.
 //   lu_outer_swap_trsm  applies the outer block's interchanges to the other

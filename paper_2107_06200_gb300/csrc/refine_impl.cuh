@@ -159,7 +159,9 @@ template <> struct RowAcc<MSIR_DD> {
 // fixed at compile time and rows past the matrix repeat the last one: with a
 // test per row the rows' sums ran one after another (n = 2000 fp64: 43 us
 // instead of 11).  Each row has two sums (even and odd columns), because
-// the chain of one is longer than a step's loads.  What bounds it: HBM for
+// the chain of one is longer than a step's loads, and each warp starts at
+// columns of its own; fp64 sums of fp32 rows with an fp64 vector have one,
+// from the first column on (kAscending).  What bounds it: HBM for
 // fp32 sums (n = 8192: 94 -> 60 us, 4.5 TB/s), the fp64 pipe (2 multiply-adds
 // per clock and SM) for fp64 ones on fp32 data, where values are widened by
 // integer instructions (steps with a subnormal, infinite or NaN operand on
@@ -274,10 +276,10 @@ __device__ __forceinline__ void gemv_rows_n(Cx& cx, const RefineArgs& a, const X
       }
       __syncwarp();
     }
-    // (Double-double sums are merged as renormalised pairs, 26 operations.
-    // As terms of the row's sum, five, they took 1.22 instead of 1.29 ms at n
-    // = 8192, with a mean error of 0.22 instead of 0.19 x 2^-106 sum |a x|;
-    // 0.16 and 0.12 at n = 2048.)
+    // (Double-double sums are merged as renormalised pairs, 26 operations:
+    // mean error 0.114 x 2^-106 sum |a x| at n = 2048, 0.220 at 8192.  As
+    // terms of the row's sum, five operations, 0.151 at n = 2048; they took
+    // 1.22 instead of 1.29 ms at n = 8192.)
 #pragma unroll
     for (int r = 0; r < NR; ++r)
       if (kOdd) acc[r][0].merge(acc[r][1]);
