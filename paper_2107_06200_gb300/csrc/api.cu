@@ -292,7 +292,7 @@ static size_t ws_layout(Workspace& w, int n, int kcap, int G, bool alloc_f64_lev
     w.D32h = (float*)take(nd * 4);
     w.D32l = (float*)take(nd * 4);
     w.D64 = (double*)take(nd * 8);
-    w.wrow = (float*)take(4 * round_up((size_t)n, kSuper) * 4);
+    w.wrow = (float*)take(6 * round_up((size_t)n, kSuper) * 4);
     w.wflag = (int*)take(64);
   } else {
     w.D32h = w.D32l = w.wrow = nullptr;

@@ -14,8 +14,8 @@
 // unevaluated pairs h + l:
 //   ArFF  pairs of fp32 (about 2^-46 per operation, all work on the fp32
 //         pipe): for fp32 solves, whose inverse is the pair rounded to fp32,
-//         while the block's Skeel condition number (inv_cond) leaves some
-//         2^-30 of that, as it does for LU factors; other blocks take ArDD;
+//         while the block's condition (inv_cond_below) leaves some 2^-30 of
+//         that, as it does for LU factors; other blocks take ArDD;
 //   ArDD  pairs of fp64 (about 2^-104): for fp64 solves (the high word) and
 //         double-double ones.
 #pragma once
@@ -222,11 +222,30 @@ __device__ __forceinline__ void inv_triangle(bool lower, typename AR::S* sm) {
   inv_double<AR, 32>(lower, B, Xh, Xl, Th, Tl);
 }
 
-// Whether the Skeel condition number max_i (|X||B|e)_i of the triangle and
-// its inverse in sm (inv_triangle's arrangement) is at most `limit`: the
-// relative error of the pairs is that times their 2^-46.  Unlike the norms'
-// product it does not see how the rows are scaled.  False if X is not finite.
-__device__ __forceinline__ bool inv_cond_below(float* sm, float limit) {
+// |A||B| of two 64x64 arrays of row stride kXld, four by four elements a
+// thread.
+__device__ __forceinline__ void abs_product(const float* A, const float* B, float (&c)[4][4]) {
+  const int i0 = (threadIdx.x >> 4) * 4, j0 = (threadIdx.x & 15) * 4;
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) c[i][j] = 0.0f;
+  for (int k = 0; k < kIB; ++k)
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        c[i][j] = __fmaf_rn(fabsf(A[(i0 + i) * kXld + k]), fabsf(B[k * kXld + j0 + j]), c[i][j]);
+}
+
+// Whether the pairs' inverse X of the triangle B in sm (inv_triangle's
+// arrangement, twice kInvValues values) is good to 2^-46 `limit` of itself:
+// its error is 2^-46 |X||B||X|.  First by Skeel's condition number
+// max_i (|X||B|e)_i, which bounds that and does not see how the rows are
+// scaled, but grows with the scaling of the columns; where it is above the
+// limit, by the largest element of a column of |X||B||X| relative to that of
+// X.  False if X is not finite.
+static __device__ __noinline__ bool inv_cond_below(float* sm, float limit) {
   const float* X = sm + kIB * kXld;
   float* sum = sm + kInvValues - kIB;  // (the reciprocals' low words are no longer read)
   const int row = threadIdx.x >> 2, part = threadIdx.x & 3;
@@ -240,7 +259,33 @@ __device__ __forceinline__ bool inv_cond_below(float* sm, float limit) {
   for (int k = part; k < kIB; k += 4) v += fabsf(X[row * kXld + k]) * sum[k];
   v += __shfl_xor_sync(0xffffffffu, v, 1);
   v += __shfl_xor_sync(0xffffffffu, v, 2);
-  return __syncthreads_and(v <= limit) != 0;
+  if (__syncthreads_and(v <= limit)) return true;
+  float* W = sm + kInvValues;
+  int* top = (int*)(W + kIB * kXld);  // columns' largest elements of X, then of |X||B||X| (bits order like values)
+  const int i0 = (threadIdx.x >> 4) * 4, j0 = (threadIdx.x & 15) * 4;
+  float c[4][4];
+  abs_product(sm, X, c);
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) W[(i0 + i) * kXld + j0 + j] = c[i][j];
+  if (threadIdx.x < 2 * kIB) top[threadIdx.x] = 0;
+  __syncthreads();
+  abs_product(X, W, c);
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    int x = 0, y = 0;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      x = max(x, __float_as_int(fabsf(X[(i0 + i) * kXld + j0 + j])));
+      y = max(y, __float_as_int(c[i][j]));
+    }
+    atomicMax(top + j0 + j, x);
+    atomicMax(top + kIB + j0 + j, y);
+  }
+  __syncthreads();
+  const int q = threadIdx.x & (kIB - 1);
+  return __syncthreads_and(__int_as_float(top[kIB + q]) <= limit * __int_as_float(top[q])) != 0;
 }
 
 // Diagonal block b of triangle `lower` (get(i, k): the packed factor's entry

@@ -76,13 +76,14 @@ constexpr int kWideApply64 = 3072;
 // A superblock's inverse is formed in fp32 pairs (2^-46 an operation) only if
 // its row sums and diagonal lie within 2^+-60 of 1 and of each other, so that
 // no product or error term of the doubling leaves fp32's range, and its
-// Skeel condition number max_i (|X||T|e)_i is at most kWideCond: the pair's
-// error is some 2^-46 of it.  (LU factors of randsvd matrices, kappa 1e2 ..
-// 1e8, plain and with rows graded by 10^+-4, stay below 4.7e4; random
-// triangles of 2^18 gave one solve of four 1.17 times the error of the
-// 64-row one.)
+// condition is at most kWideCond: the pair's error is some 2^-46 |X||T||X|.
+// As for the 64-row blocks that is bounded by Skeel's condition number
+// max_i (|X||T|e)_i, and where this is above the limit (columns of very
+// different scale) formed and compared with X column by column.  (LU factors
+// of randsvd, normal and other dense matrices, plain and with rows or columns
+// graded by 10^+-4: at most 4.7e4 by either.)
 // kWideResid: the largest scaled residual of a pair that one Newton step
-// takes to fp64 (build_wide64).
+// takes to fp64 (wide_products).
 constexpr float kWideRange = 0x1p60f, kWideCond = 0x1p17f, kWideResid = 0x1p-32f;
 constexpr int kRingDeep = 16, kRingFlat = 8;  // steps of the ring of factor values
 // Shared memory of a wide solve in values of `vbytes` on a grid of G CTAs:
@@ -190,9 +191,10 @@ struct RefineArgs {
   float* D32h;
   float* D32l;
   double* D64;
-  // of the triangles' rows within their superblock: sum of magnitudes, then
-  // the diagonal's magnitude, [2][npad] each; what build_wide and
-  // build_wide64 found (0: safe)
+  // of the triangles' rows within their superblock: sum of magnitudes, the
+  // diagonal's magnitude, then (wide_columns) the inverse columns' largest one,
+  // [2][npad] each; what build_wide and
+  // wide_products found (0: safe)
   float* wrow;
   int* wflag;
   unsigned* bar;           // grid barrier counter (zeroed before launch)

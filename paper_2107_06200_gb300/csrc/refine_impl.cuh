@@ -807,11 +807,11 @@ __device__ __forceinline__ size_t wide_row(const RefineArgs& a, int tri, int r) 
 // `wide`: the fp32 pairs go into the superblocks' array.
 //
 // The fp32 pairs of a block are formed in pair arithmetic if its diagonal is
-// far from fp32's range ends and its Skeel condition number is at most
-// kInvCond: their error of 2^-46 times that is then below 2^-32, so that the
-// inverse's fp32 rounding is the exact inverse's but for near ties.  (LU
-// factors of randsvd matrices, kappa 1e2 .. 1e8, plain and with rows graded
-// by 10^+-4: at most 1.3e3.  Solves with such inverses and scaled blocks
+// far from fp32's range ends and |X||B||X| is at most kInvCond times X
+// (inv_cond_below): their error of 2^-46 times that is then below 2^-32, so
+// that the inverse's fp32 rounding is the exact inverse's but for near ties.
+// (LU factors of randsvd and normal matrices, plain and with rows or columns
+// graded by 10^+-4: at most 1.4e3.  Solves with such inverses and scaled blocks
 // against double-double ones, n = 1024 .. 7237: 1.000 times the error of
 // those formed in double-double and fp64.)  Other blocks are formed in
 // double-double and marked inv_hard.  Where double-double inverses are there
@@ -1456,7 +1456,7 @@ __device__ __forceinline__ bool trsv(Cx& cx, const RefineArgs& a, int store_fmt)
 // Rounding: the inverse of a diagonal superblock and z are kept as pairs in
 // fp32 solves (sums compensated), so the only fp32-sized error of a
 // component is its final rounding.  fp64 solves use fp64 values: the inverse
-// is the exact one rounded (build_wide64), so that a solve's error stays
+// is the exact one rounded (wide_products), so that a solve's error stays
 // within |X||T||y| 2^-53 as on the 64-row route (figures: see kWideMin64).
 //
 // Measured (forward + backward, alone on the GPU): n = 2000 94 -> 42 us
@@ -1566,7 +1566,8 @@ __device__ __forceinline__ void wide_rows(Cx& cx, const RefineArgs& a) {
   }
 }
 // Whether the superblocks' inverses are safe in fp32 pairs (kWideRange,
-// kWideCond): sets *wflag if not, a warp per row.  The products of a row i
+// kWideCond), a warp per row: sets *wflag to 1 if the range is not, 2 if the
+// condition may not be.  The products of a row i
 // are X_ik T_kj with k between i and j, of the size of R_k / R_j where R are
 // the rows' scales; out of range they overflow or vanish although X itself
 // does not.
@@ -1592,8 +1593,166 @@ static __device__ __noinline__ void wide_check(Cx& cx, const RefineArgs& a) {
       mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, m));
       mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, m));
     }
-    const bool safe = v <= kWideCond && mx <= kWideRange && mn >= 1.0f / kWideRange && mx <= mn * kWideRange;
-    if (cx.lane == 0 && !safe) atomicOr(a.wflag, 1);
+    const bool range = mx <= kWideRange && mn >= 1.0f / kWideRange && mx <= mn * kWideRange;
+    if (cx.lane == 0 && !(range && v <= kWideCond)) atomicOr(a.wflag, range ? 2 : 1);
+  }
+}
+
+// Running sum of fp32 products f (h + l) in three words: the first two take
+// their terms by TwoSum, the third collects what those round off (Ogita,
+// Rump and Oishi's K-fold summation, K = 3: about 2^-70 of the magnitudes).
+struct ff3_t {
+  float s0, s1, s2;
+};
+__device__ __forceinline__ void ff3_term(ff3_t& a, float f, float h, float l) {
+  const float p = __fmul_rn(f, h), pe = __fmaf_rn(f, h, -p);
+  const float q = __fmul_rn(f, l), qe = __fmaf_rn(f, l, -q);
+  float t, u1, u2, u3;
+  two_sum_f(a.s0, p, a.s0, t);
+  two_sum_f(a.s1, t, a.s1, u1);
+  two_sum_f(a.s1, pe, a.s1, u2);
+  two_sum_f(a.s1, q, a.s1, u3);
+  a.s2 = __fadd_rn(a.s2, __fadd_rn(__fadd_rn(u1, u2), __fadd_rn(u3, qe)));
+}
+
+// fp64 inverses of the diagonal superblocks from the fp32 pairs X by one
+// Newton step, X (2 I - T X) = X + X R with the residual R = I - T X.  The
+// factor's values are exact in fp32, so T X is summed on the fp32 pipe in
+// three words; R is then known to some 2^-60 of its terms, and its own
+// rounding to fp32 and the plain fp32 product X R are a correction's.  What
+// is left is R^2 and the final rounding: the result is the inverse to about
+// one fp64 rounding.  (Doubled up in plain fp64 instead, the inverses carry
+// the superblock's Skeel condition number, some 1e4 for LU factors, times
+// 2^-53, and a solve with random right-hand sides was up to 2.6 times, with
+// graded rows 13 times, as inaccurate as the 64-row one.)
+//
+// R waits in M64, whose scaled blocks belong to the 64-row route (their bit
+// is cleared).  R scaled by the row sums s of |T|, R_ij s_j / s_i, has to
+// stay below kWideResid, so that R^2 (512 terms) is below 2^-54; otherwise
+// RDY_NO64 is set and the solves keep the 64-row route.
+//
+// The same two products of tiles, with magnitudes instead (kCond), are
+// |X|(|T||X|), whose columns' largest elements relative to those of X are to
+// be at most kWideCond (wide_columns has left the latter in wrow).
+//
+// The tiles of a superblock with the most inner tiles come first.
+template <typename F, bool kCond>
+__device__ __noinline__ bool wide_products(Cx& cx, const RefineArgs& a) {
+  constexpr int NT = kSuper / kBlk, NP = NT * (NT + 1) / 2;
+  float* R = (float*)a.M64;
+  float* As = (float*)cx.tsm;     // [k][i]
+  float* Bs = As + kBlk * kWtLd;  // [k][j]
+  float* Bl = Bs + kBlk * kWtLd;
+  const int n = cx.n, ldf = a.ldf, NS = a.npad / kSuper;
+  const int i0 = (cx.tid >> 4) * 4, j0 = (cx.tid & 15) * 4;
+  cx.mready &= ~RDY_M64;
+  for (int pass = 0; pass < 2; ++pass) {
+    bool bad = false;
+    for (int t = cx.cta; t < 2 * NS * NP; t += cx.G) {
+      const int tri = t % 2, s0 = (t / 2) % NS * kSuper;
+      // the q-th pair of tiles, distance NT - 1 first
+      int q = t / (2 * NS), d = NT - 1;
+      for (int cnt = 1; q >= cnt; ++cnt, --d) q -= cnt;
+      const bool lower = tri == 0;
+      const int ti = lower ? q + d : q, tj = lower ? q : q + d;
+      const int r0 = s0 + ti * kBlk, c0 = s0 + tj * kBlk;  // first row and column of the tile
+      if (max(r0, c0) >= n) continue;
+      ff3_t acc[4][4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = ff3_t{0.0f, 0.0f, 0.0f};
+      for (int kt = min(ti, tj); kt <= max(ti, tj); ++kt) {
+        const int k0 = s0 + kt * kBlk;
+        __syncthreads();  // the previous staging is no longer read
+        for (int e = cx.tid; e < kBlk * kBlk; e += kRefThreads) {
+          const int r = e / kBlk, c = e % kBlk;
+          const int arow = r0 + r, acol = k0 + c, brow = k0 + r;
+          float av = 0.0f, bh = 0.0f, bl = 0.0f;
+          if (pass == 0) {
+            if (arow < n && acol < n && (lower ? acol < arow : acol >= arow))
+              av = (float)factor_at<F>(a, (size_t)arow * ldf + acol);
+            else if (lower && acol == arow)
+              av = 1.0f;
+          } else if (arow < n) {
+            av = __ldcg(a.D32h + wide_row(a, tri, arow) + kt * kBlk + c);
+          }
+          if (brow < n) {
+            const size_t x = wide_row(a, tri, brow) + tj * kBlk + c;
+            bh = pass == 0 ? __ldcg(a.D32h + x) : __ldcg(R + x);
+            if (pass == 0) bl = __ldcg(a.D32l + x);
+          }
+          As[c * kWtLd + r] = kCond ? fabsf(av) : av;
+          Bs[r * kWtLd + c] = kCond ? fabsf(bh) : bh;
+          if (!kCond) Bl[r * kWtLd + c] = bl;
+        }
+        __syncthreads();
+#pragma unroll 2
+        for (int k = 0; k < kBlk; ++k) {
+          const float4 f = *(const float4*)(As + k * kWtLd + i0);
+          const float4 bh = *(const float4*)(Bs + k * kWtLd + j0);
+          const float F4[4] = {f.x, f.y, f.z, f.w}, H4[4] = {bh.x, bh.y, bh.z, bh.w};
+          if (pass == 0 && !kCond) {
+            const float4 bl = *(const float4*)(Bl + k * kWtLd + j0);
+            const float L4[4] = {bl.x, bl.y, bl.z, bl.w};
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+              for (int j = 0; j < 4; ++j) ff3_term(acc[i][j], F4[i], H4[j], L4[j]);
+          } else {
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+              for (int j = 0; j < 4; ++j) acc[i][j].s0 = __fmaf_rn(F4[i], H4[j], acc[i][j].s0);
+          }
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int row = r0 + i0 + i;
+        if (row >= n) continue;
+        const size_t x = wide_row(a, tri, row) + tj * kBlk + j0;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const int col = c0 + j0 + j;
+          const ff3_t v = acc[i][j];
+          if (kCond) {
+            if (pass == 0) R[x + j] = v.s0;
+            else if (col < n) bad |= !(v.s0 <= kWideCond * __ldcg(a.wrow + (size_t)(4 + tri) * a.npad + col));
+          } else if (pass == 0) {
+            float h, l;
+            two_sum_f(__fsub_rn(v.s0, row == col ? 1.0f : 0.0f), v.s1, h, l);
+            const float r = -__fadd_rn(h, __fadd_rn(l, v.s2));
+            R[x + j] = r;
+            if (col < n)
+              bad |= !(fabsf(r) * __ldcg(a.wrow + (size_t)tri * a.npad + col) <=
+                       kWideResid * __ldcg(a.wrow + (size_t)tri * a.npad + row));
+          } else {
+            a.D64[x + j] = __dadd_rn((double)__ldcg(a.D32h + x + j),
+                                     __dadd_rn((double)__ldcg(a.D32l + x + j), (double)v.s0));
+          }
+        }
+      }
+    }
+    if (bad) atomicOr(a.wflag + (kCond ? 0 : 1), 1);
+    if (!grid_barrier(cx, a)) return false;
+  }
+  if (kCond) cx.mready |= __ldcg(a.wflag) & 1 ? RDY_NO32 : RDY_W32;
+  else cx.mready |= __ldcg(a.wflag + 1) ? RDY_NO64 : RDY_W64;
+  return true;
+}
+
+// Largest element of each column of the superblocks' inverses into wrow, a
+// lane per column; behind a grid barrier.
+static __device__ __noinline__ void wide_columns(Cx& cx, const RefineArgs& a) {
+  const int n = cx.n, nc = (n + 31) / 32, nw = cx.G * (kRefThreads / 32);
+  for (int q = cx.cta * (kRefThreads / 32) + cx.warp; q < 2 * nc; q += nw) {
+    const int tri = q < nc ? 0 : 1, col = (q % nc) * 32 + cx.lane, s0 = col / kSuper * kSuper;
+    if (col >= n) continue;
+    const int r0 = tri == 0 ? col : s0, r1 = tri == 0 ? min(s0 + kSuper, n) : col + 1;
+    float m = 0.0f;
+    for (int r = r0; r < r1; ++r) m = fmaxf(m, fabsf(__ldcg(a.D32h + wide_row(a, tri, r) + (col - s0))));
+    a.wrow[(size_t)(4 + tri) * a.npad + col] = m;
   }
 }
 
@@ -1685,143 +1844,12 @@ __device__ __noinline__ bool build_wide(Cx& cx, const RefineArgs& a) {
   }
   wide_check(cx, a);
   if (!grid_barrier(cx, a)) return false;
-  cx.mready |= __ldcg(a.wflag) ? RDY_NO32 : RDY_W32;
-  return true;
-}
-
-// Running sum of fp32 products f (h + l) in three words: the first two take
-// their terms by TwoSum, the third collects what those round off (Ogita,
-// Rump and Oishi's K-fold summation, K = 3: about 2^-70 of the magnitudes).
-struct ff3_t {
-  float s0, s1, s2;
-};
-__device__ __forceinline__ void ff3_term(ff3_t& a, float f, float h, float l) {
-  const float p = __fmul_rn(f, h), pe = __fmaf_rn(f, h, -p);
-  const float q = __fmul_rn(f, l), qe = __fmaf_rn(f, l, -q);
-  float t, u1, u2, u3;
-  two_sum_f(a.s0, p, a.s0, t);
-  two_sum_f(a.s1, t, a.s1, u1);
-  two_sum_f(a.s1, pe, a.s1, u2);
-  two_sum_f(a.s1, q, a.s1, u3);
-  a.s2 = __fadd_rn(a.s2, __fadd_rn(__fadd_rn(u1, u2), __fadd_rn(u3, qe)));
-}
-
-// fp64 inverses of the diagonal superblocks from the fp32 pairs X by one
-// Newton step, X (2 I - T X) = X + X R with the residual R = I - T X.  The
-// factor's values are exact in fp32, so T X is summed on the fp32 pipe in
-// three words; R is then known to some 2^-60 of its terms, and its own
-// rounding to fp32 and the plain fp32 product X R are a correction's.  What
-// is left is R^2 and the final rounding: the result is the inverse to about
-// one fp64 rounding.  (Doubled up in plain fp64 instead, the inverses carry
-// the superblock's Skeel condition number, some 1e4 for LU factors, times
-// 2^-53, and a solve with random right-hand sides was up to 2.6 times, with
-// graded rows 13 times, as inaccurate as the 64-row one.)
-//
-// R waits in M64, whose scaled blocks belong to the 64-row route (their bit
-// is cleared).  R scaled by the row sums s of |T|, R_ij s_j / s_i, has to
-// stay below kWideResid, so that R^2 (512 terms) is below 2^-54; otherwise
-// RDY_NO64 is set and the solves keep the 64-row route.
-//
-// The tiles of a superblock with the most inner tiles come first.
-template <typename F>
-__device__ __noinline__ bool build_wide64(Cx& cx, const RefineArgs& a) {
-  constexpr int NT = kSuper / kBlk, NP = NT * (NT + 1) / 2;
-  float* R = (float*)a.M64;
-  float* As = (float*)cx.tsm;     // [k][i]
-  float* Bs = As + kBlk * kWtLd;  // [k][j]
-  float* Bl = Bs + kBlk * kWtLd;
-  const int n = cx.n, ldf = a.ldf, NS = a.npad / kSuper;
-  const int i0 = (cx.tid >> 4) * 4, j0 = (cx.tid & 15) * 4;
-  cx.mready &= ~RDY_M64;
-  for (int pass = 0; pass < 2; ++pass) {
-    bool bad = false;
-    for (int t = cx.cta; t < 2 * NS * NP; t += cx.G) {
-      const int tri = t % 2, s0 = (t / 2) % NS * kSuper;
-      // the q-th pair of tiles, distance NT - 1 first
-      int q = t / (2 * NS), d = NT - 1;
-      for (int cnt = 1; q >= cnt; ++cnt, --d) q -= cnt;
-      const bool lower = tri == 0;
-      const int ti = lower ? q + d : q, tj = lower ? q : q + d;
-      const int r0 = s0 + ti * kBlk, c0 = s0 + tj * kBlk;  // first row and column of the tile
-      if (max(r0, c0) >= n) continue;
-      ff3_t acc[4][4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = ff3_t{0.0f, 0.0f, 0.0f};
-      for (int kt = min(ti, tj); kt <= max(ti, tj); ++kt) {
-        const int k0 = s0 + kt * kBlk;
-        __syncthreads();  // the previous staging is no longer read
-        for (int e = cx.tid; e < kBlk * kBlk; e += kRefThreads) {
-          const int r = e / kBlk, c = e % kBlk;
-          const int arow = r0 + r, acol = k0 + c, brow = k0 + r;
-          float av = 0.0f, bh = 0.0f, bl = 0.0f;
-          if (pass == 0) {
-            if (arow < n && acol < n && (lower ? acol < arow : acol >= arow))
-              av = (float)factor_at<F>(a, (size_t)arow * ldf + acol);
-            else if (lower && acol == arow)
-              av = 1.0f;
-          } else if (arow < n) {
-            av = __ldcg(a.D32h + wide_row(a, tri, arow) + kt * kBlk + c);
-          }
-          if (brow < n) {
-            const size_t x = wide_row(a, tri, brow) + tj * kBlk + c;
-            bh = pass == 0 ? __ldcg(a.D32h + x) : __ldcg(R + x);
-            if (pass == 0) bl = __ldcg(a.D32l + x);
-          }
-          As[c * kWtLd + r] = av;
-          Bs[r * kWtLd + c] = bh;
-          Bl[r * kWtLd + c] = bl;
-        }
-        __syncthreads();
-#pragma unroll 2
-        for (int k = 0; k < kBlk; ++k) {
-          const float4 f = *(const float4*)(As + k * kWtLd + i0);
-          const float4 bh = *(const float4*)(Bs + k * kWtLd + j0);
-          const float F4[4] = {f.x, f.y, f.z, f.w}, H4[4] = {bh.x, bh.y, bh.z, bh.w};
-          if (pass == 0) {
-            const float4 bl = *(const float4*)(Bl + k * kWtLd + j0);
-            const float L4[4] = {bl.x, bl.y, bl.z, bl.w};
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-              for (int j = 0; j < 4; ++j) ff3_term(acc[i][j], F4[i], H4[j], L4[j]);
-          } else {
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-              for (int j = 0; j < 4; ++j) acc[i][j].s0 = __fmaf_rn(F4[i], H4[j], acc[i][j].s0);
-          }
-        }
-      }
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int row = r0 + i0 + i;
-        if (row >= n) continue;
-        const size_t x = wide_row(a, tri, row) + tj * kBlk + j0;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const int col = c0 + j0 + j;
-          const ff3_t v = acc[i][j];
-          if (pass == 0) {
-            float h, l;
-            two_sum_f(__fsub_rn(v.s0, row == col ? 1.0f : 0.0f), v.s1, h, l);
-            const float r = -__fadd_rn(h, __fadd_rn(l, v.s2));
-            R[x + j] = r;
-            if (col < n)
-              bad |= !(fabsf(r) * __ldcg(a.wrow + (size_t)tri * a.npad + col) <=
-                       kWideResid * __ldcg(a.wrow + (size_t)tri * a.npad + row));
-          } else {
-            a.D64[x + j] = __dadd_rn((double)__ldcg(a.D32h + x + j),
-                                     __dadd_rn((double)__ldcg(a.D32l + x + j), (double)v.s0));
-          }
-        }
-      }
-    }
-    if (bad) atomicOr(a.wflag + 1, 1);
-    if (!grid_barrier(cx, a)) return false;
+  const int flag = __ldcg(a.wflag);
+  if (flag == 2) {
+    wide_columns(cx, a);
+    return wide_products<F, true>(cx, a);
   }
-  cx.mready |= __ldcg(a.wflag + 1) ? RDY_NO64 : RDY_W64;
+  cx.mready |= flag ? RDY_NO32 : RDY_W32;
   return true;
 }
 
@@ -2325,7 +2353,7 @@ __device__ bool msolve(Cx& cx, const RefineArgs& a, int store_fmt, bool synced) 
         if (!grid_barrier(cx, a) || !build_wide<F>(cx, a)) return false;
       }
       if (!k32 && (cx.mready & RDY_W32) && !(cx.mready & (RDY_W64 | RDY_NO64)))
-        if (!build_wide64<F>(cx, a)) return false;
+        if (!wide_products<F, false>(cx, a)) return false;
       if (cx.mready & need) {
         if (!synced && !grid_barrier(cx, a)) return false;
         {

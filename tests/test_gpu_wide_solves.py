@@ -133,3 +133,25 @@ def test_routes_share_a_workspace(ctx, monkeypatch):
                 assert np.array_equal(got, x.setdefault((route, arith), got))
         f.close()
     assert not np.array_equal(x["0", OF.FP64], x["1", OF.FP64])
+
+
+@pytest.mark.parametrize("n,arith", [(1300, OF.FP32), (1900, OF.FP64)])
+@pytest.mark.parametrize("uf", [OF.BF16, OF.FP32])
+def test_graded_columns_keep_the_wide_route(ctx, monkeypatch, n, arith, uf):
+    """Columns scaled by 10^+-4 change neither the accuracy of an inverse nor
+    that of a solve (x is scaled back), though Skeel's condition number of
+    U's blocks is 2^30 and more.  The routes' results differ, and the wide
+    one's error, component by component in units of its scale, is the smaller."""
+    import paper_2107_06200_gb300 as M
+    A, _, R = system(n, 1e4, False)
+    d = 10.0 ** np.random.default_rng(n).uniform(-4, 4, n)
+    f = ctx.factor(to_dev(A * d[None, :]), OF.FP32, uf, M.params_default())
+    assert f.info == 0 and f.nonfinite == 0
+    ref = f.apply(to_dev(R), OF.DD, OF.FP64).cpu().numpy()
+    e = []
+    for route in ("1", "0"):
+        monkeypatch.setenv("MSIR_WIDE_APPLY", route)
+        e.append(np.abs(f.apply(to_dev(R), arith, arith).cpu().numpy() - ref) * d[:, None])
+    f.close()
+    assert not np.array_equal(e[0], e[1])
+    assert np.exp(np.log(e[0].mean(0) / e[1].mean(0)).mean()) <= 1
