@@ -191,10 +191,10 @@ struct RefineArgs {
   float* D32h;
   float* D32l;
   double* D64;
-  // of the triangles' rows within their superblock: sum of magnitudes, the
-  // diagonal's magnitude, then (wide_columns) the inverse columns' largest one,
-  // [2][npad] each; what build_wide and
-  // wide_products found (0: safe)
+  // of the triangles within their superblocks, [2][npad] each: the rows' sums
+  // of magnitudes, the diagonal's magnitudes, the largest one of each column
+  // of the inverse (wide_columns); what build_wide and wide_products found
+  // (0: safe)
   float* wrow;
   int* wflag;
   unsigned* bar;           // grid barrier counter (zeroed before launch)
